@@ -16,21 +16,12 @@
 // Node update: for each time level the node's EG2 operator (eq. (EG2)) is
 // evaluated on that reconstruction.  The Mach-cone base is a circle of radius
 // c' tau around P' = node - u' tau; it crosses the grid lines through the
-// node at cos(theta) = u'/c' and sin(theta) = v'/c', which splits it into at
-// most four arcs, each inside one cell.  On an arc a cell's biquadratic is a
-// polynomial in cos and sin of degree <= 2 in each (a Taylor shift of the
-// monomials), the EG2 weights raise that to degree <= 6, and every arc
-// integral is taken exactly from the arc's end points with the recurrences
-//   (m+n) J_mn = [cos^(m-1) sin^(n+1)] + (m-1) J_(m-2)n
-//   (m+n) J_mn = -[cos^(m+1) sin^(n-1)] + (n-1) J_m(n-2)
-// for J_mn = int cos^m sin^n dtheta.  The sum over the cells' arcs is taken
-// by inclusion-exclusion (one cell's coefficients over the whole circle, plus
-// differences of coefficients over the two half-circles cut off by the grid
-// lines and over their intersection; see "EG2 arc sums by inclusion-
-// exclusion" below), which needs no crossing sort and makes half of the
-// integrals vanish by symmetry.  All data are taken relative to the node's
-// own t^n value, which the operators reproduce exactly, so FP32 keeps its
-// relative accuracy in the perturbations.
+// node at cos(theta) = u'/c' and sin(theta) = v'/c'.  The reconstruction on it
+// is the reference cell's polynomial plus truncated powers of the distances
+// from the grid lines (see "EG2 arc sums in the truncated-power form" below);
+// every integral is taken exactly, without a crossing sort.  All data are
+// taken relative to the node's own t^n value, which the operators reproduce
+// exactly, so FP32 keeps its relative accuracy in the perturbations.
 #include <type_traits>
 
 #include "af_common.cuh"
@@ -39,6 +30,11 @@
 namespace af {
 
 namespace {
+
+// keeps the loads on either side in order: the compiler otherwise moves the next
+// stage's record loads up over the current one's arithmetic and holds them in
+// registers (4096^2 vortex: 2.45 ms without, 2.43 with)
+__device__ __forceinline__ void keep_order() { asm volatile("" ::: "memory"); }
 
 constexpr float PI_F = 3.14159265358979f;
 constexpr float INV_PI = 0.318309886183791f;
@@ -56,9 +52,14 @@ __device__ __forceinline__ float sqrt_nn(float t) { return t > 0.0f ? t * rsqrtf
 // of the heights in tile_heights (the batched path picks one by timing).
 constexpr int TX = 32;
 constexpr int HX = TX + 2;                   // with a one-cell halo on each side
-constexpr int CELL_F = 52;                   // floats per cell in shared memory
-// per cell: 4 variables x (9 monomial coefficients + 3 pad) = 48 floats, then Ubar (4)
-constexpr int UBAR_OFF = 48;
+// Cell records in shared memory, row by row: first the row's Ubar (HX cells, 4
+// floats each), then the records of its HX - 1 cells that node updates read:
+// per cell 4 variables x 8 monomial coefficients and the four values m00, 36
+// floats (9 float4, an odd number: consecutive cells' 128-bit accesses meet no
+// bank conflicts).  The last row and column of the halo hold Ubar only (Alg. 2
+// reads no more there).  76.5 KB for an 8-row tile and its raw data.
+constexpr int CELL_F = 36, M00_OFF = 32;
+constexpr int ROW_F = HX * 4 + (HX - 1) * CELL_F;
 // Raw t^n data of a tile, staged by TMA: for each of the node arrays (vertex,
 // x-edge, y-edge) and the cell averages a box of RAW_W x (TY + 3) points x 4
 // variables.  The box starts 4 points left of the first halo point so that
@@ -67,7 +68,7 @@ constexpr int RAW_W = TX + 8;
 template <int TY>
 struct Tile {
   static constexpr int HY = TY + 2;
-  static constexpr int REC_FLOATS = HX * HY * CELL_F;
+  static constexpr int REC_FLOATS = (HY - 1) * ROW_F + HX * 4;
   static constexpr int RAW_H = TY + 3;
   static constexpr int RAW_ARR = RAW_W * RAW_H * NV;  // floats per array
   static constexpr int RAW_FLOATS = 4 * RAW_ARR;
@@ -120,12 +121,23 @@ __device__ __forceinline__ void unpack4(float4 w, float U[4]) {
 // rows of cell records the running kernel's tile holds (checking builds)
 __shared__ int rec_rows;
 #endif
-// shared-memory cell record of tile-local cell (a, b), a in [0, HX), b in [0, HY)
+// shared-memory record of tile-local cell (a, b), a in [0, HX - 1), b in [0, HY - 1)
 __device__ __forceinline__ const float *cell_rec(const float *sm, int a, int b) {
+#ifdef AF_CHECK_BOUNDS
+  if (!bounds_ok(a >= 0 && a < HX - 1 && b >= 0 && b < rec_rows - 1, BD_RECORD)) return sm;
+#endif
+  return sm + b * ROW_F + HX * 4 + a * CELL_F;
+}
+// U_c (the monomials m00 of the four variables) of a record
+__device__ __forceinline__ float4 cell_m00(const float *rec) {
+  return reinterpret_cast<const float4 *>(rec + M00_OFF)[0];
+}
+// Ubar of tile-local cell (a, b), a in [0, HX), b in [0, HY)
+__device__ __forceinline__ const float *cell_ubar(const float *sm, int a, int b) {
 #ifdef AF_CHECK_BOUNDS
   if (!bounds_ok(a >= 0 && a < HX && b >= 0 && b < rec_rows, BD_RECORD)) return sm;
 #endif
-  return sm + (b * HX + a) * CELL_F;
+  return sm + b * ROW_F + a * 4;
 }
 
 // ----------------------------------------------------------------- prologue
@@ -147,10 +159,11 @@ __device__ __forceinline__ void to_monomial(const float f[3][3], float m[3][3]) 
   }
 }
 
-// prep of cell (ci, cj) and its record in shared memory, from the staged tile
+// prep of cell (ci, cj) from the staged tile: its Ubar, and its record unless
+// rec is null
 template <int TY>
 __device__ __forceinline__ void build_cell(const Grid &g, const float *raw, int i0, int j0, int ci, int cj,
-                                           float *rec) {
+                                           float *ub, float *rec) {
   float N[8][4];  // corners (ll, lr, ul, ur), then edges (left, right, bottom, top)
   raw4<TY>(raw, RAW_VTX, ci, cj, i0, j0, N[0]);
   raw4<TY>(raw, RAW_VTX, ci + 1, cj, i0, j0, N[1]);
@@ -164,197 +177,277 @@ __device__ __forceinline__ void build_cell(const Grid &g, const float *raw, int 
 #pragma unroll
   for (int v = 0; v < NV; v++) Qa[v] = raw_at<TY>(raw, RAW_AVG, v, ci, cj, i0, j0);
   cell_prep(N, Qa, g.gamma, g.ubar_c2p, Uc, Ub);
+  *reinterpret_cast<float4 *>(ub) = make_float4(Ub[0], Ub[1], Ub[2], Ub[3]);
+  if (!rec) return;
+  float4 *r4 = reinterpret_cast<float4 *>(rec);
 #pragma unroll
   for (int v = 0; v < NV; v++) {
     const float f[3][3] = {{N[0][v], N[4][v], N[2][v]}, {N[6][v], Uc[v], N[7][v]}, {N[1][v], N[5][v], N[3][v]}};
     float m[3][3];
     to_monomial(f, m);
-    float4 *r4 = reinterpret_cast<float4 *>(rec + 12 * v);
-    r4[0] = make_float4(m[0][0], m[0][1], m[0][2], m[1][0]);
-    r4[1] = make_float4(m[1][1], m[1][2], m[2][0], m[2][1]);
-    r4[2] = make_float4(m[2][2], 0.0f, 0.0f, 0.0f);
-    rec[UBAR_OFF + v] = Ub[v];
+    r4[2 * v] = make_float4(m[1][0], m[2][0], m[0][1], m[0][2]);
+    r4[2 * v + 1] = make_float4(m[1][1], m[1][2], m[2][1], m[2][2]);
+  }
+  r4[M00_OFF / 4] = make_float4(Uc[0], Uc[1], Uc[2], Uc[3]);
+}
+
+// ---- EG2 arc sums in the truncated-power form of the reconstruction
+// In the frame reflected so that u', v' >= 0 (cos -> fx cos, sin -> fy sin),
+// with X = rx (cos - a), Y = ry (sin - b) the coordinates relative to the node
+// on the Mach circle (a = |u'|/c', b = |v'|/c'), the reconstruction around a
+// vertex is
+//   q = q_ref + [X > 0] Dx + [Y > 0] Dy + [X > 0, Y > 0] Dxy,
+// q_ref the biquadratic of the cell on side -- (it holds P') and
+//   Dx = X d1(y) + X^2 d2(y),  Dy = Y d1(x) + Y^2 d2(x),
+//   Dxy = X Y (g11 + g21 X + g12 Y + g22 X Y):
+// q is continuous across a grid line, so the difference of the two cells
+// vanishes on it, and only the jumps of the normal derivatives (6 numbers a
+// line, 4 for the crossing) enter instead of 9 coefficients a cell.  An edge
+// midpoint has one line: q_ref + [X > 0] Dx.  The integrals of cos^m sin^n
+// times q_ref over the whole circle are constants; Dx is integrated over
+// {cos > a} = (-acos a, acos a), where with
+//   L_m = int (cos - a)^m,  N_m = int (cos - a)^m sin^2
+// the end-point terms vanish and
+//   m L_m = (m-1) (1 - a^2) L_(m-2) - (2m-1) a L_(m-1),
+//   m N_(m-1) = L_(m+1) + a L_m = int cos (cos - a)^m;
+// Dy likewise with the roles of cos and sin exchanged, and Dxy over the arc
+// (asin b, acos a) (empty unless a^2 + b^2 < 1) from two identities of the
+// same kind (quarter_moments).  All sums are taken divided by pi.
+//
+// The stages (circle, X, Y, crossing) each build their own small table and run
+// over p, u and v, reading the records again, so that one table is live at a
+// time; the terms in X and X^2 go together through the packed FP32x2
+// instructions.  Bound by issue and latency at 16 warps an SM (128
+// registers): 3735 thread instructions a cell at 66 % of the issue slots.  The
+// earlier form took differences of all 9 coefficients of each cell on the
+// circle with two half tables and an arc table live together (4990
+// instructions).  Measured, point values, 4096^2 vortex moving / at rest
+// (crossings at no / every vertex): 3.05 / 3.32 -> 2.37 / 2.53 ms; Alg. 1
+// linearisation at 2048^2 1.16 -> 0.87 ms, Riemann data with every limiter
+// 1.17 -> 0.96 ms.  80 or 96 registers (24 or 20 warps) spill to a local memory
+// that the L1 beside the shared memory cannot hold: 2.97 and 2.88 ms.
+
+__device__ __forceinline__ float2 pair(float x) { return make_float2(x, x); }
+
+// Taylor coefficients t of q(x) = a0 + a1 x + a2 x^2 at x0 (the last is a2)
+__device__ __forceinline__ void taylor(float a0, float a1, float a2, float x0, float &t0, float &t1) {
+  const float t = fmaf(a2, x0, a1);
+  t0 = fmaf(t, x0, a0);
+  t1 = fmaf(a2, x0, t);
+}
+__device__ __forceinline__ float horner(float a0, float a1, float a2, float x0) {
+  return fmaf(fmaf(a2, x0, a1), x0, a0);
+}
+
+// sums over the circle, divided by pi, with the reflected cos and sin:
+// p: int p, int p cos, int p sin; u: int u cos, int u (2 cos^2 - 1/2),
+// int u sin cos; v: int v sin, int v (2 sin^2 - 1/2), int v sin cos
+struct Sums {
+  float p[3], u[3], v[3];
+};
+__device__ __forceinline__ float total(float2 a) { return a.x + a.y; }
+__device__ __forceinline__ void taylor2(float2 a0, float2 a1, float2 a2, float x0, float2 &t0, float2 &t1) {
+  const float2 t = __ffma2_rn(a2, pair(x0), a1);
+  t0 = __ffma2_rn(t, pair(x0), a0);
+  t1 = __ffma2_rn(a2, pair(x0), t);
+}
+
+// a cell's coefficients of one variable: m[i][e] of x^i y^e (m00 apart)
+struct Coef {
+  float4 lin, mix;  // (m10, m20, m01, m02), (m11, m12, m21, m22)
+};
+__device__ __forceinline__ Coef coef(const float *rec, int v) {
+  const float4 *r = reinterpret_cast<const float4 *>(rec) + 2 * v;
+  return Coef{r[0], r[1]};
+}
+
+// the circle x = x0 + rx cos, y = y0 + ry sin in the reference cell's centred
+// units (rx, ry carry the reflection signs), and the factors of the sums
+struct Circle {
+  float x0, y0, rx, ry, rx2, ry2;
+};
+
+// whole-circle sums of q_ref (value m00 - K at the cell centre): its Taylor
+// coefficients at P' times the circle's constant integrals; only those that
+// the variable's sums use
+template <int VAR>
+__device__ __forceinline__ void circle_sums(const Coef &m, float m00, const Circle &c, float s[3], float &centre) {
+  // x first (p, u) or y first (v): r[i][e] of (first axis about P')^i
+  // (second)^e, then t[i][e] about P' in both
+  constexpr bool YF = VAR == 2;
+  const float f0 = YF ? c.y0 : c.x0, s0 = YF ? c.x0 : c.y0;
+  const float m20 = YF ? m.lin.w : m.lin.y, m21 = YF ? m.mix.y : m.mix.z;
+  float r00, r10, r01, r11, r02, r12;
+  taylor(m00, YF ? m.lin.z : m.lin.x, m20, f0, r00, r10);
+  taylor(YF ? m.lin.x : m.lin.z, m.mix.x, m21, f0, r01, r11);
+  taylor(YF ? m.lin.y : m.lin.w, YF ? m.mix.z : m.mix.y, m.mix.w, f0, r02, r12);
+  float t00, t01, t10, t11;
+  taylor(r00, r01, r02, s0, t00, t01);
+  taylor(r10, r11, r12, s0, t10, t11);
+  const float t20 = horner(m20, m21, m.mix.w, s0);
+  const float rf = YF ? c.ry : c.rx, rs = YF ? c.rx : c.ry, rf2 = YF ? c.ry2 : c.rx2, rs2 = YF ? c.rx2 : c.ry2;
+  centre = t00;
+  if (VAR == 0) {
+    const float t21 = fmaf(2.0f * s0, m.mix.w, m21);
+    s[0] = fmaf(2.0f, t00, fmaf(rf2, fmaf(0.25f * rs2, m.mix.w, t20), rs2 * r02));
+    s[1] = rf * fmaf(0.25f * rs2, r12, t10);
+    s[2] = rs * fmaf(0.25f * rf2, t21, t01);
+  } else {
+    s[0] = rf * fmaf(0.25f * rs2, r12, t10);
+    s[1] = fmaf(rf2, fmaf(0.125f * rs2, m.mix.w, t20), t00);
+    s[2] = (0.25f * rf) * (rs * t11);
   }
 }
 
-// J[m][n] = int_{t0}^{t1} cos^m sin^n for m, n <= 4, m + n <= 6
-__device__ __forceinline__ void jtable(float t0, float c0, float s0, float t1, float c1, float s1,
-                                       float J[5][5]) {
-  float c0s = c0 * c0, c1s = c1 * c1, c0c = c0s * c0, c1c = c1s * c1;
-  float s0s = s0 * s0, s1s = s1 * s1, s0c = s0s * s0, s1c = s1s * s1;
-  float s0q = s0s * s0s, s1q = s1s * s1s;
-  float Ds = s1 - s0, Dc = c1 - c0, Ds2 = s1s - s0s;
-  float Dcs = c1 * s1 - c0 * s0, Dc2s = c1s * s1 - c0s * s0, Dc3s = c1c * s1 - c0c * s0;
-  float Dcs2 = c1 * s1s - c0 * s0s, Dc2s2 = c1s * s1s - c0s * s0s, Dc3s2 = c1c * s1s - c0c * s0s;
-  float Dcs3 = c1 * s1c - c0 * s0c, Dc2s3 = c1s * s1c - c0s * s0c, Dc3s3 = c1c * s1c - c0c * s0c;
-  float Dcs4 = c1 * s1q - c0 * s0q, Dc2s4 = c1s * s1q - c0s * s0q;
-  float Dcs5 = c1 * s1q * s1 - c0 * s0q * s0;
-  J[0][0] = t1 - t0;
-  J[1][0] = Ds;
-  J[0][1] = -Dc;
-  J[1][1] = 0.5f * Ds2;
-  J[2][0] = 0.5f * (Dcs + J[0][0]);
-  J[3][0] = (Dc2s + 2.0f * J[1][0]) * (1.0f / 3.0f);
-  J[4][0] = 0.25f * (Dc3s + 3.0f * J[2][0]);
-  J[2][1] = (Dcs2 + J[0][1]) * (1.0f / 3.0f);
-  J[3][1] = 0.25f * (Dc2s2 + 2.0f * J[1][1]);
-  J[4][1] = 0.2f * (Dc3s2 + 3.0f * J[2][1]);
-  J[0][2] = 0.5f * (J[0][0] - Dcs);
-  J[1][2] = (J[1][0] - Dc2s) * (1.0f / 3.0f);
-  J[2][2] = 0.25f * (Dcs3 + J[0][2]);
-  J[3][2] = 0.2f * (Dc2s3 + 2.0f * J[1][2]);
-  J[4][2] = (Dc3s3 + 3.0f * J[2][2]) * (1.0f / 6.0f);
-  J[0][3] = (2.0f * J[0][1] - Dcs2) * (1.0f / 3.0f);
-  J[1][3] = 0.25f * (2.0f * J[1][1] - Dc2s2);
-  J[2][3] = 0.2f * (Dcs4 + J[0][3]);
-  J[3][3] = (Dc2s4 + 2.0f * J[1][3]) * (1.0f / 6.0f);
-  J[0][4] = 0.25f * (3.0f * J[0][2] - Dcs3);
-  J[1][4] = 0.2f * (3.0f * J[1][2] - Dc2s3);
-  J[2][4] = (Dcs5 + J[0][4]) * (1.0f / 6.0f);
-}
-
-// Taylor shift of q(x) = a0 + a1 x + a2 x^2 to x = x0 + r c:  q = b0 + b1 c + b2 c^2
-__device__ __forceinline__ void shift(float a0, float a1, float a2, float x0, float r, float r2,
-                                      float &b0, float &b1, float &b2) {
-  const float t = fmaf(a2, x0, a1);
-  b0 = fmaf(t, x0, a0);
-  b1 = fmaf(a2, x0, t) * r;
-  b2 = a2 * r2;
-}
-
-// coefficients b[a][e] of cos^a sin^e of (cell polynomial - K) on the circle
-// x = x0 + rx cos, y = y0 + ry sin (cell-centred units)
-__device__ __forceinline__ void circle_coef(const float *rec, float K, float x0, float y0, float rx,
-                                            float rx2, float ry, float ry2, float b[3][3]) {
-  const float4 p0 = reinterpret_cast<const float4 *>(rec)[0];
-  const float4 p1 = reinterpret_cast<const float4 *>(rec)[1];
-  const float m22 = reinterpret_cast<const float4 *>(rec)[2].x;
-  // m[a][e]: x^a y^e;  p0 = (m00, m01, m02, m10), p1 = (m11, m12, m20, m21)
-  float q[3][3];  // q[a][e]: cos^a y^e
-  shift(p0.x - K, p0.w, p1.z, x0, rx, rx2, q[0][0], q[1][0], q[2][0]);
-  shift(p0.y, p1.x, p1.w, x0, rx, rx2, q[0][1], q[1][1], q[2][1]);
-  shift(p0.z, p1.y, m22, x0, rx, rx2, q[0][2], q[1][2], q[2][2]);
-#pragma unroll
-  for (int a = 0; a < 3; a++) shift(q[a][0], q[a][1], q[a][2], y0, ry, ry2, b[a][0], b[a][1], b[a][2]);
-}
-
-// value of (cell polynomial - K) at (x0, y0)
-__device__ __forceinline__ float eval_at(const float *rec, float K, float x0, float y0) {
-  const float4 p0 = reinterpret_cast<const float4 *>(rec)[0];
-  const float4 p1 = reinterpret_cast<const float4 *>(rec)[1];
-  const float m22 = reinterpret_cast<const float4 *>(rec)[2].x;
-  const float e0 = fmaf(fmaf(p1.z, x0, p0.w), x0, p0.x - K);
-  const float e1 = fmaf(fmaf(p1.w, x0, p1.x), x0, p0.y);
-  const float e2 = fmaf(fmaf(m22, x0, p1.y), x0, p0.z);
+// value of (cell polynomial - K) at (x0, y0); m00 already relative to K
+__device__ __forceinline__ float eval_at(const Coef &m, float m00, float x0, float y0) {
+  const float e0 = fmaf(fmaf(m.lin.y, x0, m.lin.x), x0, m00);
+  const float e1 = fmaf(fmaf(m.mix.z, x0, m.mix.x), x0, m.lin.z);
+  const float e2 = fmaf(fmaf(m.mix.w, x0, m.mix.y), x0, m.lin.w);
   return fmaf(fmaf(e2, y0, e1), y0, e0);
 }
 
-// ---- EG2 arc sums by inclusion-exclusion
-// In the frame reflected so that u', v' >= 0 (cos -> fx cos, sin -> fy sin),
-// the grid lines through the node split the circle into the sides
-// X = {cos > a} (a = |u'|/c') and Y = {sin > b} (b = |v'|/c'): X is the arc
-// (-acos a, acos a), Y the arc (asin b, pi - asin b), and X and Y meet in the
-// single arc (asin b, acos a) when a^2 + b^2 < 1, else not at all.  With b_q
-// the circle coefficients of the cell on side q (++, +-, -+, --), the sum
-// over the cells' arcs of int b_q w is
-//   int_circle b_-- w + int_X (b_+- - b_--) w + int_Y (b_-+ - b_--) w
-//   + int_(X and Y) (b_++ - b_+- - b_-+ + b_--) w,
-// exactly (inclusion-exclusion of the four quadrants).  Over the whole circle
-// only even powers of both cos and sin integrate to non-zero values; over X
-// (symmetric about 0) only even powers of sin, over Y (symmetric about
-// pi/2) only even powers of cos.  An edge-midpoint node (one grid line) keeps
-// the first two terms (XE) or the first and third (YE).
-
-// H[m][n] = int_{-al}^{al} cos^m sin^n for n even (al = acos a, s = sin al):
-// twice the integrals from 0, by the recurrences of jtable with the start
-// point (1, 0); the entries m <= 4, n <= 4, m + n <= 6 the moments use
-__device__ __forceinline__ void half_table(float a, float s, float al, float H[5][5]) {
-  const float s2 = s * s, s3 = s2 * s, a2 = a * a, a3 = a2 * a;
-  const float as = a * s, as3 = a * s3;
-  const float I20 = 0.5f * (as + al), I02 = 0.5f * (al - as), I12 = s3 * (1.0f / 3.0f);
-  const float I22 = 0.25f * (as3 + I02), I04 = 0.25f * (3.0f * I02 - as3);
-  H[0][0] = 2.0f * al;
-  H[1][0] = 2.0f * s;
-  H[2][0] = 2.0f * I20;
-  H[3][0] = (2.0f / 3.0f) * (a2 * s + 2.0f * s);
-  H[4][0] = 0.5f * (a3 * s + 3.0f * I20);
-  H[0][2] = 2.0f * I02;
-  H[1][2] = 2.0f * I12;
-  H[2][2] = 2.0f * I22;
-  H[3][2] = 0.4f * (a2 * s3 + 2.0f * I12);
-  H[4][2] = (1.0f / 3.0f) * (a3 * s3 + 3.0f * I22);
-  H[0][4] = 2.0f * I04;
-  H[1][4] = 0.4f * (3.0f * I12 - a2 * s3);
-  H[2][4] = (1.0f / 3.0f) * (as3 * s2 + I04);
+// moments over {cos > a} divided by pi: [k] for X (k = 0) and X^2 (k = 1), the
+// weights 1, cos (c), 2 cos^2 - 1/2 (K), 2 sin^2 - 1/2 (V); the second row of
+// each times sin^2.  r, r2: the factors of X and X^2.
+struct HalfTable {
+  float2 one[2], c[2], K[2], V[2];  // [times sin^2], the pair (X, X^2)
+};
+// a = |normal velocity| / c' (clamped to 1), s = sin(acos a), al = acos a.
+// With W_m = int (cos - a)^m sin^4 the same integration by parts gives
+//   N_1 = (2/3) s^3 - a N_0,  (m+3) N_(m+1) = m (1 - a^2) N_(m-1) - (2m+3) a N_m,
+//   m W_(m-1) = 3 (N_(m+1) + a N_m) = 3 int cos (cos - a)^m sin^2,
+// and the weights are 2 cos^2 - 1/2 = 3/2 - 2 sin^2, 2 sin^2 - 1/2.
+__device__ __forceinline__ void half_table(float a, float s, float al, float r, float r2, HalfTable &H) {
+  const float q = s * s;
+  const float L0 = (2.0f * INV_PI) * al, L1 = (2.0f * INV_PI) * fmaf(-a, al, s);
+  const float L2 = 0.5f * fmaf(q, L0, -3.0f * (a * L1));
+  const float N0 = fmaf(a, L1, L2);
+  const float N1 = fmaf((2.0f * INV_PI / 3.0f) * q, s, -a * N0);
+  const float N2 = 0.25f * fmaf(q, N0, -5.0f * (a * N1));
+  const float N3 = fmaf(0.4f * q, N1, -1.4f * (a * N2));
+  const float N4 = fmaf(0.5f * q, N2, -1.5f * (a * N3));
+  const float CN1 = fmaf(a, N1, N2), CN2 = fmaf(a, N2, N3), CN3 = fmaf(a, N3, N4);
+  const float2 rr = make_float2(r, r2);
+  H.one[0] = __fmul2_rn(rr, make_float2(L1, L2));
+  H.one[1] = __fmul2_rn(rr, make_float2(N1, N2));
+  H.c[0] = __fmul2_rn(rr, make_float2(N0, 2.0f * N1));
+  H.c[1] = __fmul2_rn(rr, make_float2(CN1, CN2));
+  const float2 W = __fmul2_rn(rr, make_float2(3.0f * CN2, 2.0f * CN3));  // 2 int X^k sin^4
+  H.K[0] = __ffma2_rn(pair(1.5f), H.one[0], __fmul2_rn(pair(-2.0f), H.one[1]));
+  H.K[1] = __ffma2_rn(pair(-1.0f), W, __fmul2_rn(pair(1.5f), H.one[1]));
+  H.V[0] = __ffma2_rn(pair(-1.0f), H.K[0], H.one[0]);
+  H.V[1] = __ffma2_rn(pair(-0.5f), H.one[1], W);
 }
 
-// int over the whole circle of cos^m sin^n for the (m, n) the moments use
-// (zero unless m and n are even)
-__host__ __device__ constexpr float jfull(int m, int n) {
-  return ((m & 1) || (n & 1)) ? 0.0f
-         : (m == 0 && n == 0) ? 2.0f * PI_F
-         : (m + n == 2) ? PI_F
-         : (m == 2 && n == 2) ? 0.25f * PI_F
-         : (m + n == 4) ? 0.75f * PI_F
-         : (m + n == 6 && m != 0 && n != 0) ? 0.125f * PI_F
-         : 0.0f;
-}
-
-// table kinds: full arc table, X-side table H (odd n vanish), Y-side table
-// (odd m vanish; stored transposed, H[n][m]), whole circle (constants)
-enum { TB_ARC = 0, TB_X = 1, TB_Y = 2, TB_CIRCLE = 3 };
-
-// acc + sum_{i,e <= 2} b[i][e] T(i + DI, e + DE), skipping the entries the
-// table's symmetry makes zero
-template <int DI, int DE, int KIND>
-__device__ __forceinline__ float contract(const float b[3][3], const float T[5][5], float acc) {
+// jumps across a grid line: the derivatives' coefficients along the line
+// (tangential powers 0, 1, 2), cell-centred; YL: the line is horizontal
+// (x and y change roles); f the reflection sign of the normal axis
+template <bool YL>
+__device__ __forceinline__ void jumps(const Coef &R, const Coef &O, float f, float2 d[3]) {
+  const float r1[3] = {YL ? R.lin.z : R.lin.x, R.mix.x, YL ? R.mix.z : R.mix.y};
+  const float r2[3] = {YL ? R.lin.w : R.lin.y, YL ? R.mix.y : R.mix.z, R.mix.w};
+  const float o1[3] = {YL ? O.lin.z : O.lin.x, O.mix.x, YL ? O.mix.z : O.mix.y};
+  const float o2[3] = {YL ? O.lin.w : O.lin.y, YL ? O.mix.y : O.mix.z, O.mix.w};
 #pragma unroll
-  for (int i = 0; i < 3; i++)
-#pragma unroll
-    for (int e = 0; e < 3; e++) {
-      const int m = i + DI, n = e + DE;
-      if (KIND == TB_X && (n & 1)) continue;
-      if (KIND == TB_Y && (m & 1)) continue;
-      if (KIND == TB_CIRCLE && ((m | n) & 1)) continue;
-      const float t = KIND == TB_CIRCLE ? jfull(m, n) : (KIND == TB_Y ? T[n][m] : T[m][n]);
-      acc = fmaf(b[i][e], t, acc);
-    }
-  return acc;
+  for (int n = 0; n < 3; n++) d[n] = make_float2(fmaf(f, o1[n] - r1[n], -(o2[n] + r2[n])), o2[n] - r2[n]);
 }
 
-// the EG2 moments of one variable against one table: p (VAR 0): int p,
-// int p cos, int p sin; u (1): int u cos, int u cos^2, int u, int u sin cos;
-// v (2): int v sin, int v sin^2, int v, int v sin cos
-template <int VAR, int KIND>
-__device__ __forceinline__ void moments(const float b[3][3], const float T[5][5], float acc[4]) {
+// adds the half-circle sums of Dx (or Dy) of one variable: t0, rt, rt2 the
+// circle along the line (tangential coordinate t = t0 + rt sin); VAR 0: p;
+// 1: the velocity normal to the line; 2: the tangential one.  m in the frame
+// of the line: p: 1, cos, sin; normal: cos, 2 cos^2 - 1/2, sin cos;
+// tangential: sin, 2 sin^2 - 1/2, sin cos
+template <int VAR>
+__device__ __forceinline__ void half_sums(const float2 d[3], float t0, float rt, float rt2, const HalfTable &H,
+                                          float &m0, float &m1, float &m2) {
+  float2 e0, e1, a, b, c;
+  taylor2(d[0], d[1], d[2], t0, e0, e1);
+  e1 = __fmul2_rn(e1, pair(rt));
+  const float2 e2 = __fmul2_rn(d[2], pair(rt2));
   if (VAR == 0) {
-    acc[0] = contract<0, 0, KIND>(b, T, acc[0]);
-    acc[1] = contract<1, 0, KIND>(b, T, acc[1]);
-    acc[2] = contract<0, 1, KIND>(b, T, acc[2]);
+    a = __ffma2_rn(e0, H.one[0], __fmul2_rn(e2, H.one[1]));
+    b = __ffma2_rn(e0, H.c[0], __fmul2_rn(e2, H.c[1]));
+    c = __fmul2_rn(e1, H.one[1]);
   } else if (VAR == 1) {
-    acc[0] = contract<1, 0, KIND>(b, T, acc[0]);
-    acc[1] = contract<2, 0, KIND>(b, T, acc[1]);
-    acc[2] = contract<0, 0, KIND>(b, T, acc[2]);
-    acc[3] = contract<1, 1, KIND>(b, T, acc[3]);
+    a = __ffma2_rn(e0, H.c[0], __fmul2_rn(e2, H.c[1]));
+    b = __ffma2_rn(e0, H.K[0], __fmul2_rn(e2, H.K[1]));
+    c = __fmul2_rn(e1, H.c[1]);
   } else {
-    acc[0] = contract<0, 1, KIND>(b, T, acc[0]);
-    acc[1] = contract<0, 2, KIND>(b, T, acc[1]);
-    acc[2] = contract<0, 0, KIND>(b, T, acc[2]);
-    acc[3] = contract<1, 1, KIND>(b, T, acc[3]);
+    a = __fmul2_rn(e1, H.one[1]);
+    b = __ffma2_rn(e0, H.V[0], __fmul2_rn(e2, H.V[1]));
+    c = __fmul2_rn(e1, H.c[1]);
+  }
+  m0 += total(a);
+  m1 += total(b);
+  m2 += total(c);
+}
+
+// moments over the quarter (asin b, acos a), divided by pi, with c = cos,
+// s = sin: entries XY, X^2 Y, X Y^2, X^2 Y^2 without the radii.  With
+// q_mn = int (c - a)^m (s - b)^n, kap = 1 - a^2 - b^2 and both factors
+// vanishing at an end point each, d[(c-a)^m (s-b)^n] and c^2 + s^2 = 1 give
+//   m (q_(m-1,n+1) + b q_(m-1,n)) = n (q_(m+1,n-1) + a q_(m,n-1)),
+//   q_(m+2,n) + 2 a q_(m+1,n) + q_(m,n+2) + 2 b q_(m,n+1) = kap q_mn.
+struct QuarterTable {
+  float2 one[2], c[2], s[2], K[2], V[2], Z[2];  // (XY, X^2 Y), (X Y^2, X^2 Y^2)
+};
+__device__ __forceinline__ void quarter_moments(float a, float b, float sa, float sb, float phi, QuarterTable &T) {
+  const float kap = fmaf(-a, a, fmaf(-b, b, 1.0f));
+  const float q00 = INV_PI * phi, q10 = fmaf(-a, q00, INV_PI * (sa - b)), q01 = fmaf(-b, q00, INV_PI * (sb - a));
+  // q11 = int cos sin - b int cos - a int sin + a b phi
+  const float q11 = fmaf(INV_PI * 0.5f, kap, -fmaf(INV_PI * b, sa - b, fmaf(a, INV_PI * (sb - a), -a * b * q00)));
+  const float h = 0.5f * fmaf(kap, q00, -fmaf(a, q10, b * q01));
+  const float q20 = fmaf(-a, q10, h), q02 = fmaf(-b, q01, h);
+  const float q12 = (1.0f / 3.0f) * fmaf(kap, q10, -fmaf(4.0f * b, q11, a * q20));
+  const float q21 = (1.0f / 3.0f) * fmaf(kap, q01, -fmaf(4.0f * a, q11, b * q02));
+  const float t = 0.5f * fmaf(kap, q11, -fmaf(a, q21, b * q12));  // int c X^2 Y = int s X Y^2
+  const float q31 = fmaf(-a, q21, t), q13 = fmaf(-b, q12, t);
+  const float q30 = fmaf(2.0f, fmaf(b, q11, q12), -a * q20);
+  const float q22 = 0.25f * fmaf(kap, q20, -fmaf(5.0f * b, q21, a * q30));
+  const float D41 = 0.6f * fmaf(kap, q21, -fmaf(a, q31, b * q22));  // int c X^3 Y
+  const float D14 = 0.6f * fmaf(kap, q12, -fmaf(b, q13, a * q22));  // int s X Y^3
+  const float E23 = (2.0f / 3.0f) * D41, E32 = (2.0f / 3.0f) * D14;  // int s X^2 Y^2, int c X^2 Y^2
+  const float q41 = fmaf(-a, q31, D41), q23 = fmaf(-b, q22, E23), q32 = fmaf(-a, q22, E32);
+  const float F = 0.5f * fmaf(kap, q22, -fmaf(a, q32, b * q23));                // int c X^3 Y^2
+  const float Gs = (1.0f / 3.0f) * fmaf(kap, q31, -fmaf(a, q41, b * q32));      // int s X^3 Y^2
+  T.one[0] = make_float2(q11, q21);
+  T.one[1] = make_float2(q12, q22);
+  const float c11 = fmaf(a, q11, q21), c12 = fmaf(a, q12, q22), s11 = fmaf(b, q11, q12), s21 = fmaf(b, q21, q22);
+  T.c[0] = make_float2(c11, t);
+  T.c[1] = make_float2(c12, E32);
+  T.s[0] = make_float2(s11, s21);
+  T.s[1] = make_float2(t, E23);
+  const float2 cc[2] = {make_float2(fmaf(a, c11, t), fmaf(a, t, D41)), make_float2(fmaf(a, c12, E32), fmaf(a, E32, F))};
+  T.Z[0] = make_float2(fmaf(a, s11, s21), fmaf(a, s21, fmaf(b, q31, q32)));
+  T.Z[1] = make_float2(fmaf(a, t, E23), fmaf(a, E23, Gs));
+#pragma unroll
+  for (int k = 0; k < 2; k++) {
+    T.K[k] = __ffma2_rn(pair(2.0f), cc[k], __fmul2_rn(pair(-0.5f), T.one[k]));
+    T.V[k] = __ffma2_rn(pair(-1.0f), T.K[k], T.one[k]);
   }
 }
-
-// tile-local cell indices of the cells around node (K, i, j)
-template <int K>
-__device__ __forceinline__ void arc_cell(int li, int lj, int right, int top, int &a, int &b) {
-  a = (K == YE) ? li + 1 : li + right;
-  b = (K == XE) ? lj + 1 : lj + top;
+// adds the sums of Dxy with coefficients g (radii folded in)
+__device__ __forceinline__ void quarter_sums(const float2 g[2], const float2 w0[2], const float2 w1[2],
+                                             const float2 w2[2], float &m0, float &m1, float &m2) {
+  m0 += total(__ffma2_rn(g[0], w0[0], __fmul2_rn(g[1], w0[1])));
+  m1 += total(__ffma2_rn(g[0], w1[0], __fmul2_rn(g[1], w1[1])));
+  m2 += total(__ffma2_rn(g[0], w2[0], __fmul2_rn(g[1], w2[1])));
 }
-// node position in the cell-centred units of that cell, before the shift by -u' tau
+
+// the jumps across an edge midpoint's own line, between the cells below / left
+// (reference) and above / right of it: the same for both time levels.  Seen
+// from the other side (f = -1) d1 is the same and d2 changes sign.
+struct LineJumps {
+  float2 p[3], u[3], v[3];
+};
 template <int K>
-__device__ __forceinline__ void node_in_cell(int right, int top, float &xn, float &yn) {
-  xn = (K == YE) ? 0.0f : (right ? -0.5f : 0.5f);
-  yn = (K == XE) ? 0.0f : (top ? -0.5f : 0.5f);
+__device__ __forceinline__ void line_jumps(const float *sm, int li, int lj, LineJumps &J) {
+  if (K == VTX) return;
+  const float *r = cell_rec(sm, K == YE ? li + 1 : li, K == XE ? lj + 1 : lj), *o = cell_rec(sm, li + 1, lj + 1);
+  jumps<K == YE>(coef(r, 3), coef(o, 3), 1.0f, J.p);
+  jumps<K == YE>(coef(r, 1), coef(o, 1), 1.0f, J.u);
+  jumps<K == YE>(coef(r, 2), coef(o, 2), 1.0f, J.v);
 }
 
 // EG2 of the cpq reconstruction at node (K, li, lj) of the tile, linearised
@@ -363,15 +456,13 @@ __device__ __forceinline__ void node_in_cell(int right, int top, float &xn, floa
 // linearisation state fails; the value is then not an EG2 value).
 template <int K>
 __device__ __forceinline__ bool eg2(const Grid &g, const float *sm, int li, int lj, const float Kr[4],
-                                    const float ul_in[4], float tau, float out[4]) {
-  // an inadmissible linearisation state gives NaN outputs; the arithmetic
-  // runs on a harmless substitute so that no branch splits the evaluation
-  const bool good = ul_in[0] > 0.0f && ul_in[3] > 0.0f && tau > 0.0f;
-  const float ul[4] = {good ? ul_in[0] : 1.0f, good ? ul_in[1] : 0.0f, good ? ul_in[2] : 0.0f,
-                       good ? ul_in[3] : 1.0f};
-  const float cp2 = __fdividef(g.gamma * ul[3], ul[0]), icp = rsqrtf(cp2), cp = cp2 * icp;
+                                    const float ul[4], float tau, const LineJumps &J, float out[4]) {
+  // an inadmissible linearisation state gives NaN outputs: c' becomes NaN and
+  // every sum with it, so that no branch splits the evaluation
+  const bool good = ul[0] > 0.0f && ul[3] > 0.0f && tau > 0.0f;
+  const float cp2 = good ? __fdividef(g.gamma * ul[3], ul[0]) : __int_as_float(0x7fc00000);
+  const float icp = rsqrtf(cp2), cp = cp2 * icp;
   const float R = cp * tau;
-  const float am = ul[1] * icp, bm = ul[2] * icp;
   bool inside;
   {
     const float ex = fabsf(ul[1]) * tau + R, ey = fabsf(ul[2]) * tau + R;
@@ -379,141 +470,138 @@ __device__ __forceinline__ bool eg2(const Grid &g, const float *sm, int li, int 
     inside = !(ex > lx || ey > ly);
   }
   const float rx = R * g.idx, ry = R * g.idy, rx2 = rx * rx, ry2 = ry * ry;
-  const float sx = ul[1] * tau * g.idx, sy = ul[2] * tau * g.idy;
+  // reflection signs (u', v' >= 0 in the reflected frame)
+  const bool nx_ = K != YE && ul[1] < 0.0f, ny_ = K != XE && ul[2] < 0.0f;
+  const float fx = nx_ ? -1.0f : 1.0f, fy = ny_ ? -1.0f : 1.0f;
+  const float ax = fabsf(ul[1] * icp), by = fabsf(ul[2] * icp);
+  const float frx = fx * rx, fry = fy * ry;
+  // cells by side of the reflected frame: reference --, across the vertical
+  // line (X side), across the horizontal line (Y side); P' in the
+  // reference cell's centred units
+  const int ar = (K == YE) ? li + 1 : li + (nx_ ? 1 : 0), br = (K == XE) ? lj + 1 : lj + (ny_ ? 1 : 0);
+  const int ao = (K == YE) ? ar : li + (nx_ ? 0 : 1), bo = (K == XE) ? br : lj + (ny_ ? 0 : 1);
+  const float *rr = cell_rec(sm, ar, br);
+  const float x0 = fmaf(-ul[1] * tau, g.idx, (K == YE) ? 0.0f : 0.5f * fx);
+  const float y0 = fmaf(-ul[2] * tau, g.idy, (K == XE) ? 0.0f : 0.5f * fy);
 
-  // reflection signs (u', v' >= 0 in the reflected frame) and the sides met
-  const float fx = (K != YE && ul[1] < 0.0f) ? -1.0f : 1.0f, fy = (K != XE && ul[2] < 0.0f) ? -1.0f : 1.0f;
-  const float ax = fabsf(am), by = fabsf(bm);
-  // a line the circle does not cross gives a half table of zeros (al = 0,
-  // sin al = 0), so the X and Y stages run without branches
-  constexpr bool hx = K != YE, hy = K != XE;
-  const bool hq = K == VTX && ax < 1.0f && by < 1.0f && fmaf(ax, ax, by * by) < 1.0f;
-  float Tx[5][5], Ty[5][5], Jq[5][5];
+  Sums S;
+  float drP, dpP, unused;
+  const float4 m00 = cell_m00(rr);
+  // the signed radii carry the reflection: the sums are those of the
+  // reflected cos and sin
+  const Circle C{x0, y0, frx, fry, rx2, ry2};
+  drP = eval_at(coef(rr, 0), m00.x - Kr[0], x0, y0);
+  circle_sums<0>(coef(rr, 3), m00.w - Kr[3], C, S.p, dpP);
+  keep_order();
+  circle_sums<1>(coef(rr, 1), m00.y - Kr[1], C, S.u, unused);
+  keep_order();
+  circle_sums<2>(coef(rr, 2), m00.z - Kr[2], C, S.v, unused);
+  keep_order();
+
   float alx = 0.0f, snx = 0.0f, aly = 0.0f, sny = 0.0f;
-  if (hx) {
+  float2 d[3];
+  if (K != YE) {
     const float a = fminf(ax, 1.0f);
     alx = acosf(a);
     snx = sqrt_nn(fmaf(-a, a, 1.0f));
-    half_table(a, snx, alx, Tx);
+    HalfTable H;
+    if (K == XE) {
+      half_table(a, snx, alx, rx, fx * rx2, H);
+      half_sums<0>(J.p, y0, fry, ry2, H, S.p[0], S.p[1], S.p[2]);
+      half_sums<1>(J.u, y0, fry, ry2, H, S.u[0], S.u[1], S.u[2]);
+      half_sums<2>(J.v, y0, fry, ry2, H, S.v[0], S.v[1], S.v[2]);
+    } else {
+      half_table(a, snx, alx, rx, rx2, H);
+      const float *ro = cell_rec(sm, ao, br);
+      jumps<false>(coef(rr, 3), coef(ro, 3), fx, d);
+      half_sums<0>(d, y0, fry, ry2, H, S.p[0], S.p[1], S.p[2]);
+      keep_order();
+      jumps<false>(coef(rr, 1), coef(ro, 1), fx, d);
+      half_sums<1>(d, y0, fry, ry2, H, S.u[0], S.u[1], S.u[2]);
+      keep_order();
+      jumps<false>(coef(rr, 2), coef(ro, 2), fx, d);
+      half_sums<2>(d, y0, fry, ry2, H, S.v[0], S.v[1], S.v[2]);
+      keep_order();
+    }
   }
-  if (hy) {
+  if (K != XE) {
     const float b = fminf(by, 1.0f);
     aly = acosf(b);
     sny = sqrt_nn(fmaf(-b, b, 1.0f));
-    half_table(b, sny, aly, Ty);
-  }
-  // X and Y meet in (asin b, acos a): (cos, sin) = (sin aly, b) to (a, sin alx)
-  if (hq) jtable(0.5f * PI_F - aly, sny, by, alx, ax, snx, Jq);
-  const float frx = fx * rx, fry = fy * ry;
-
-  // circle coefficients of variable (record offset off, reference Kv) of
-  // the cell on side (px, py) (1: the + side) of the reflected frame
-  auto side = [&](int px, int py, int off, float Kv, float q[3][3]) {
-    const int right = px ? (fx > 0.0f) : (fx < 0.0f), top = py ? (fy > 0.0f) : (fy < 0.0f);
-    int a, b;
-    arc_cell<K>(li, lj, right, top, a, b);
-    float xn, yn;
-    node_in_cell<K>(right, top, xn, yn);
-    circle_coef(cell_rec(sm, a, b) + off, Kv, xn - sx, yn - sy, frx, rx2, fry, ry2, q);
-  };
-  // all moments of one variable: b_-- over the circle, then the differences
-  // over X, Y and their intersection
-  auto var_moments = [&](auto var_tag, int off, float Kv, float acc[4]) {
-    constexpr int VAR = decltype(var_tag)::value;
-    float b0[3][3], S[3][3], d[3][3];
-    side(0, 0, off, Kv, b0);
-    moments<VAR, TB_CIRCLE>(b0, Tx, acc);
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-      for (int e = 0; e < 3; e++) S[i][e] = b0[i][e];
-    if (hx) {
-      side(1, 0, off, Kv, d);
-#pragma unroll
-      for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int e = 0; e < 3; e++) {
-          S[i][e] -= d[i][e];
-          d[i][e] -= b0[i][e];
-        }
-      moments<VAR, TB_X>(d, Tx, acc);
+    HalfTable H;
+    if (K == YE) {
+      half_table(b, sny, aly, ry, fy * ry2, H);
+      half_sums<0>(J.p, x0, frx, rx2, H, S.p[0], S.p[2], S.p[1]);
+      half_sums<1>(J.v, x0, frx, rx2, H, S.v[0], S.v[1], S.v[2]);
+      half_sums<2>(J.u, x0, frx, rx2, H, S.u[0], S.u[1], S.u[2]);
+    } else {
+      half_table(b, sny, aly, ry, ry2, H);
+      const float *ro = cell_rec(sm, ar, bo);
+      jumps<true>(coef(rr, 3), coef(ro, 3), fy, d);
+      half_sums<0>(d, x0, frx, rx2, H, S.p[0], S.p[2], S.p[1]);
+      keep_order();
+      jumps<true>(coef(rr, 2), coef(ro, 2), fy, d);
+      half_sums<1>(d, x0, frx, rx2, H, S.v[0], S.v[1], S.v[2]);
+      keep_order();
+      jumps<true>(coef(rr, 1), coef(ro, 1), fy, d);
+      half_sums<2>(d, x0, frx, rx2, H, S.u[0], S.u[1], S.u[2]);
+      keep_order();
     }
-    if (hy) {
-      side(0, 1, off, Kv, d);
-#pragma unroll
-      for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int e = 0; e < 3; e++) {
-          S[i][e] -= d[i][e];
-          d[i][e] -= b0[i][e];
-        }
-      moments<VAR, TB_Y>(d, Ty, acc);
-    }
-    if (hq) {
-      side(1, 1, off, Kv, d);
-#pragma unroll
-      for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int e = 0; e < 3; e++) d[i][e] += S[i][e];
-      moments<VAR, TB_ARC>(d, Jq, acc);
-    }
-  };
-  // the moments enter the result as soon as each variable is done (moments
-  // odd in cos change sign with fx, odd in sin with fy, back in the grid frame)
-  const float rp = ul[0], rc = rp * cp, irc = __fdividef(icp, rp), icp2 = icp * icp, rpi = rp * icp;
-  float o[4], M[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  var_moments(std::integral_constant<int, 0>(), 36, Kr[3], M);  // p0, pc, ps
-  o[0] = M[0] * icp2;
-  o[1] = -fx * M[1] * irc;
-  o[2] = -fy * M[2] * irc;
-  o[3] = M[0];
-  M[0] = M[1] = M[2] = M[3] = 0.0f;
-  var_moments(std::integral_constant<int, 1>(), 12, Kr[1], M);  // uc, u2, u0, usc
-  const float uc = fx * M[0];
-  o[0] = fmaf(-rpi, uc, o[0]);
-  o[3] = fmaf(-rc, uc, o[3]);
-  o[1] += 2.0f * M[1] - 0.5f * M[2];
-  o[2] += 2.0f * fx * fy * M[3];
-  M[0] = M[1] = M[2] = M[3] = 0.0f;
-  var_moments(std::integral_constant<int, 2>(), 24, Kr[2], M);  // vs, v2, v0, vsc
-  const float vs = fy * M[0];
-  o[0] = fmaf(-rpi, vs, o[0]);
-  o[3] = fmaf(-rc, vs, o[3]);
-  o[2] += 2.0f * M[1] - 0.5f * M[2];
-  o[1] += 2.0f * fx * fy * M[3];
-  // rho and p at P' (the cell on side --: its closure holds P')
-  float drP, dpP;
-  {
-    const int right = fx < 0.0f, top = fy < 0.0f;
-    int a, b;
-    arc_cell<K>(li, lj, right, top, a, b);
-    const float *rec = cell_rec(sm, a, b);
-    float xn, yn;
-    node_in_cell<K>(right, top, xn, yn);
-    drP = eval_at(rec, Kr[0], xn - sx, yn - sy);
-    dpP = eval_at(rec + 36, Kr[3], xn - sx, yn - sy);
   }
-  out[0] = Kr[0] + drP - 2.0f * dpP * icp2 + INV_PI * o[0];
-  out[1] = Kr[1] + INV_PI * o[1];
-  out[2] = Kr[2] + INV_PI * o[2];
-  out[3] = Kr[3] - dpP + INV_PI * o[3];
-  if (!good) {
-#pragma unroll
-    for (int v = 0; v < NV; v++) out[v] = __int_as_float(0x7fc00000);
-    return true;
+  if (K == VTX && ax < 1.0f && by < 1.0f && fmaf(ax, ax, by * by) < 1.0f) {
+    QuarterTable T;
+    quarter_moments(ax, by, snx, sny, alx + aly - 0.5f * PI_F, T);
+    const float *rX = cell_rec(sm, ao, br), *rY = cell_rec(sm, ar, bo), *rQ = cell_rec(sm, ao, bo);
+    const float rxy = rx * ry;
+    auto crossing = [&](int v, float2 gq[2]) {
+      // mixed coefficients (m11, m12, m21, m22) of the four cells: jumps
+      // across the vertical line below and above, then of those across the
+      // horizontal one
+      const float4 m = reinterpret_cast<const float4 *>(rr)[2 * v + 1], mx = reinterpret_cast<const float4 *>(rX)[2 * v + 1];
+      const float4 my = reinterpret_cast<const float4 *>(rY)[2 * v + 1], mq = reinterpret_cast<const float4 *>(rQ)[2 * v + 1];
+      const float l1 = fmaf(fx, mx.x - m.x, -(mx.z + m.z)), l2 = fmaf(fx, mx.y - m.y, -(mx.w + m.w));
+      const float u1 = fmaf(fx, mq.x - my.x, -(mq.z + my.z)), u2 = fmaf(fx, mq.y - my.y, -(mq.w + my.w));
+      const float k1 = mx.z - m.z, k2 = mx.w - m.w, w1 = mq.z - my.z, w2 = mq.w - my.w;
+      gq[0] = make_float2(rxy * fmaf(fy, u1 - l1, -(u2 + l2)), rxy * rx * fmaf(fy, w1 - k1, -(w2 + k2)));
+      gq[1] = make_float2(rxy * ry * (u2 - l2), rxy * rxy * (w2 - k2));
+    };
+    float2 gq[2];
+    crossing(3, gq);
+    quarter_sums(gq, T.one, T.c, T.s, S.p[0], S.p[1], S.p[2]);
+    keep_order();
+    crossing(1, gq);
+    quarter_sums(gq, T.c, T.K, T.Z, S.u[0], S.u[1], S.u[2]);
+    keep_order();
+    crossing(2, gq);
+    quarter_sums(gq, T.s, T.V, T.Z, S.v[0], S.v[1], S.v[2]);
+    keep_order();
   }
+  // sums odd in cos change sign with fx, odd in sin with fy, back in the grid
+  // frame; div = int (u cos + v sin)
+  const float irc = __fdividef(icp, ul[0]), icp2 = icp * icp;
+  const float z = fmaf(-ul[0] * cp, fmaf(fx, S.u[0], fy * S.v[0]), S.p[0]);
+  const float fxy = 2.0f * fx * fy;
+  out[0] = fmaf(icp2, fmaf(-2.0f, dpP, z), Kr[0] + drP);
+  out[1] = Kr[1] + fmaf(-fx * irc, S.p[1], fmaf(fxy, S.v[2], S.u[1]));
+  out[2] = Kr[2] + fmaf(-fy * irc, S.p[2], fmaf(fxy, S.u[2], S.v[1]));
+  out[3] = Kr[3] + (z - dpP);
   return inside;
 }
 
 // ---------------------------------------------------------------- Alg. 3 parts
-// Records are read as float4 only: the record stride (52 words, 13 float4) is
-// free of bank conflicts for 128-bit accesses of consecutive cells.
 __device__ __forceinline__ float4 ubar4(const float *sm, int a, int b) {
-  return reinterpret_cast<const float4 *>(cell_rec(sm, a, b) + UBAR_OFF)[0];
+  return reinterpret_cast<const float4 *>(cell_ubar(sm, a, b))[0];
 }
-// U_c (the monomial m00) of variable v of tile-local cell (a, b)
-__device__ __forceinline__ float centre(const float *sm, int a, int b, int v) {
-  return reinterpret_cast<const float4 *>(cell_rec(sm, a, b) + 12 * v)[0].x;
+// U_c of tile-local cell (a, b)
+__device__ __forceinline__ void centre(const float *sm, int a, int b, float U[4]) {
+  unpack4(cell_m00(cell_rec(sm, a, b)), U);
+}
+
+// tile-local cell indices of the cells around node (K, i, j)
+template <int K>
+__device__ __forceinline__ void arc_cell(int li, int lj, int right, int top, int &a, int &b) {
+  a = (K == YE) ? li + 1 : li + right;
+  b = (K == XE) ? lj + 1 : lj + top;
 }
 
 // EG1 (Sec. 3.3) on piecewise-constant primitive averages, relative to Kr
@@ -781,17 +869,22 @@ __device__ __forceinline__ void correction(const Grid &g, const float *sm, const
                                            int i0, int j0, const float U[4], float T[4]) {
   float Ux[4], Uy[4];
   const int a = i - i0 + 1, b = j - j0 + 1;
+  float Cp[4], Cm[4];  // U_c on either side of the edge
+  if (K != VTX) {
+    centre(sm, a, b, Cp);
+    centre(sm, K == XE ? a - 1 : a, K == XE ? b : b - 1, Cm);
+  }
 #pragma unroll
   for (int v = 0; v < NV; v++) {
     if (K == VTX) {
       Ux[v] = (raw_at<TY>(raw, RAW_YE, v, i, j, i0, j0) - raw_at<TY>(raw, RAW_YE, v, i - 1, j, i0, j0)) * g.idx;
       Uy[v] = (raw_at<TY>(raw, RAW_XE, v, i, j, i0, j0) - raw_at<TY>(raw, RAW_XE, v, i, j - 1, i0, j0)) * g.idy;
     } else if (K == XE) {
-      Ux[v] = (centre(sm, a, b, v) - centre(sm, a - 1, b, v)) * g.idx;
+      Ux[v] = (Cp[v] - Cm[v]) * g.idx;
       Uy[v] = (raw_at<TY>(raw, RAW_VTX, v, i, j + 1, i0, j0) - raw_at<TY>(raw, RAW_VTX, v, i, j, i0, j0)) * g.idy;
     } else {
       Ux[v] = (raw_at<TY>(raw, RAW_VTX, v, i + 1, j, i0, j0) - raw_at<TY>(raw, RAW_VTX, v, i, j, i0, j0)) * g.idx;
-      Uy[v] = (centre(sm, a, b, v) - centre(sm, a, b - 1, v)) * g.idy;
+      Uy[v] = (Cp[v] - Cm[v]) * g.idy;
     }
   }
   const float r = U[0], u = U[1], v = U[2], p = U[3], gm = g.gamma, ir = __fdividef(1.0f, r);
@@ -879,7 +972,9 @@ __device__ __forceinline__ void node_update(const Args &A, const float *sm, cons
 #pragma unroll
     for (int v = 0; v < NV; v++) ul[v] = U0[v];
   } else if (FULL && A.lin_mode == 2) {
-    cfl_bad |= !eg2<K>(g, sm, li, lj, U0, U0, 0.25f * A.dt, ul);
+    // Alg. 1: level 0 of the loop below turns this into EG2's value over dt/4
+#pragma unroll
+    for (int v = 0; v < NV; v++) ul[v] = U0[v];
   } else {
     const bool wx = (K != YE) && ((i == 0 && g.bc[0] == BC_REFLECTING) || (i == g.nx && g.bc[1] == BC_REFLECTING));
     const bool wy = (K != XE) && ((j == 0 && g.bc[2] == BC_REFLECTING) || (j == g.ny && g.bc[3] == BC_REFLECTING));
@@ -910,9 +1005,11 @@ __device__ __forceinline__ void node_update(const Args &A, const float *sm, cons
     if (K == VTX && sw) cnt[CNT_TSW]++;
   }
 
+  LineJumps J;
+  line_jumps<K>(sm, li, lj, J);
 #pragma unroll 1
-  for (int lev = 1; lev <= 2; lev++) {
-    const float tau = lev == 1 ? 0.5f * A.dt : A.dt;
+  for (int lev = FULL && A.lin_mode == 2 ? 0 : 1; lev <= 2; lev++) {
+    const float tau = lev == 1 ? 0.5f * A.dt : (FULL && lev == 0 ? 0.25f * A.dt : A.dt);
     if (lev == 2) {
       if (FULL && sw) {
         lin_avg<K>(sm, li, lj, ul);
@@ -922,8 +1019,13 @@ __device__ __forceinline__ void node_update(const Args &A, const float *sm, cons
       }
     }
     float ho[4];
-    const bool inb = eg2<K>(g, sm, li, lj, U0, ul, tau, ho);
+    const bool inb = eg2<K>(g, sm, li, lj, U0, ul, tau, J, ho);
     cfl_bad |= !inb;
+    if (FULL && lev == 0) {
+#pragma unroll
+      for (int v = 0; v < NV; v++) ul[v] = ho[v];
+      continue;
+    }
     const float ht = 0.5f * tau * tau;
 #pragma unroll
     for (int v = 0; v < NV; v++) ho[v] = fmaf(ht, T[v], ho[v]);
@@ -946,7 +1048,7 @@ __device__ __forceinline__ void node_update(const Args &A, const float *sm, cons
       for (int v = 0; v < NV; v++) res[v] = th * res[v] + (1.0f - th) * lo[v];
     }
 #pragma unroll
-    for (int v = 0; v < NV; v++) nonfinite |= !isfinite(res[v]);
+    for (int v = 0; v < NV; v++) nonfinite |= (FULL || !ok) && !isfinite(res[v]);  // (lean: an ok value is finite)
     if (NF && lev == 1) {
 #pragma unroll
       for (int v = 0; v < NV; v++) scr[v * (TX * TY)] = res[v];
@@ -956,23 +1058,30 @@ __device__ __forceinline__ void node_update(const Args &A, const float *sm, cons
   if (NF) node_flux<K, TY>(A, i, j, U0, res, scr);
 }
 
-// prologue: the block builds the records of its (TX+2) x (TY+2) cells; only
-// cells -1..nx, -1..ny can be referenced by owned nodes, the others are
-// skipped.  The last column and row of the halo (cells i0 + TX, j0 + TY) are
-// read only by Alg. 2's indicator at the tile's last edge nodes: without
-// Alg. 2 they are not built (297 instead of 340 records at TY = 8).
-template <int TY, int W, int H>
-__device__ __forceinline__ void build_records(const Args &A, const float *raw, float *sm, int i0, int j0, int tid) {
-  for (int k = tid; k < W * H; k += TX * TY) {
-    const int a = k % W, b = k / W, ci = i0 - 1 + a, cj = j0 - 1 + b;
-    if (ci <= A.g.nx && cj <= A.g.ny) build_cell<TY>(A.g, raw, i0, j0, ci, cj, const_cast<float *>(cell_rec(sm, a, b)));
-  }
-}
+// prologue: the block builds the records of the tile's cells and its halo on
+// the low sides, (TX+1) x (TY+1); only cells -1..nx, -1..ny can be referenced
+// by owned nodes, the others are skipped.  The last column and row of the halo
+// (cells i0 + TX, j0 + TY) are read only by Alg. 2's indicator at the tile's
+// last edge nodes, and only their Ubar.
 template <int TY>
 __device__ __forceinline__ void tile_prologue(const Args &A, const float *raw, float *sm, int i0, int j0,
                                               int tid) {
-  if (A.tsw) build_records<TY, HX, Tile<TY>::HY>(A, raw, sm, i0, j0, tid);
-  else build_records<TY, HX - 1, Tile<TY>::HY - 1>(A, raw, sm, i0, j0, tid);
+  constexpr int W = HX - 1, H = Tile<TY>::HY - 1;
+  for (int k = tid; k < W * H; k += TX * TY) {
+    const int a = k % W, b = k / W, ci = i0 - 1 + a, cj = j0 - 1 + b;
+    if (ci <= A.g.nx && cj <= A.g.ny)
+      build_cell<TY>(A.g, raw, i0, j0, ci, cj, const_cast<float *>(cell_ubar(sm, a, b)),
+                     const_cast<float *>(cell_rec(sm, a, b)));
+  }
+}
+template <int TY>
+__device__ __noinline__ void tile_prologue_tsw(const Args &A, const float *raw, float *sm, int i0, int j0, int tid) {
+  constexpr int W = HX - 1, H = Tile<TY>::HY - 1;
+  for (int k = tid; k < W + H + 1; k += TX * TY) {
+    const int a = k < W ? k : W, b = k < W ? H : k - W, ci = i0 - 1 + a, cj = j0 - 1 + b;
+    if (ci <= A.g.nx && cj <= A.g.ny)
+      build_cell<TY>(A.g, raw, i0, j0, ci, cj, const_cast<float *>(cell_ubar(sm, a, b)), nullptr);
+  }
 }
 
 // the block's maximum wave speed of the new point values (node-flux
@@ -1098,6 +1207,7 @@ __device__ __forceinline__ void tile_body(const Args &A, const TileMaps &T, floa
     return;
   }
   tile_prologue<TY>(A, raw, sm, i0, j0, tid);
+  if (FT != PV_LEAN && A.tsw) tile_prologue_tsw<TY>(A, raw, sm, i0, j0, tid);
   __syncthreads();
   tile_nodes<TY, FT>(A, sm, raw, i0, j0, threadIdx.x, threadIdx.y, sm + Tile<TY>::REC_FLOATS + tid);
 }
@@ -1107,14 +1217,13 @@ __device__ __forceinline__ float *tile_smem(float4 *smem4) {
   return reinterpret_cast<float *>((reinterpret_cast<size_t>(smem4) + 127) & ~size_t(127));
 }
 
-// Blocks per SM that the register budget is sized for, the most that the
-// tile's shared memory allows: two for 8 rows (128 registers a thread, 16
-// warps), one for 16 rows (the 512 threads cap it at 128 anyway), three for
-// 4 rows (170 registers, 12 warps).  Without the bound the compiler may take
-// more registers than two 8-row blocks can share.
+// Blocks per SM that the register budget is sized for: two for 8 rows (128
+// registers a thread, 16 warps), one for 16 rows, four for 4 rows (the same 16
+// warps; with five blocks the 96 registers spill: 2.88 against 2.39 ms at
+// 4096^2).
 template <int TY>
 constexpr int min_blocks() {
-  return TY == 4 ? 3 : (TY == 8 ? 2 : 1);
+  return TY == 4 ? 4 : (TY == 8 ? 2 : 1);
 }
 
 // L2 prefetch of the tile that the block PREFETCH_AHEAD places later in
