@@ -923,6 +923,8 @@ static int step64(af_ctx *h, double dt) {
   S.ph.gam = h->gamma;
   S.ph.dx = h->dx;
   S.ph.dy = h->dy;
+  S.ph.idx = 1.0 / h->dx;
+  S.ph.idy = 1.0 / h->dy;
   S.avg = h->f64_avg;
   for (int k = 0; k < 3; k++) {
     S.n0[k] = h->f64_lev[0][k];

@@ -269,7 +269,7 @@ int *gemm_default_err();
 // Sec. 3 limiters (accuracy studies below the FP32 floor)
 // gamma and the cell sizes in double (the grid description holds FP32 copies)
 struct Phys64 {
-  double gam, dx, dy;
+  double gam, dx, dy, idx, idy;
 };
 struct Step64 {
   Grid g;
