@@ -396,7 +396,7 @@ long long af_batch_active_cells(af_batch *b);
 int af_batch_set_stream(af_batch *b, void *stream);
 
 /* ------------------------------------------------------------------------
- * Tensor-core GEMM used by the surrogate's training: D (+)= A B^T (+ bias)
+ * Tensor-core GEMM: D (+)= A B^T (+ bias)
  * with A (M x K) and B (N x K) row-major BF16 device arrays (leading
  * dimensions lda, ldb in elements) and D (M x N, leading dimension ldd) FP32,
  * accumulated in FP32 on the tcgen05 tensor cores.  0 < N <= 128; K, lda and
@@ -434,7 +434,7 @@ int af_mlp_get_params(af_mlp *m, float *host_out);
  * scales rms(T[:, k]) from device arrays X (n x 64) and T (n x 8). */
 int af_mlp_fit_scales(af_mlp *m, const float *X, const float *T, long long n);
 /* Y (n x 8, device) = the network at the rows of X (n x 64, device),
- * including both scales.  Through the training path's GEMM kernels. */
+ * including both scales.  Through the training path's forward kernel. */
 int af_mlp_forward(af_mlp *m, const float *X, float *Y, int n, void *stream);
 /* Mean squared error over the 8 outputs of the n rows (targets divided by
  * the output scales) and its gradient with respect to the trained

@@ -1,6 +1,7 @@
 // af_gemm.cu -- BF16 x BF16 -> FP32 matrix product on the tcgen05 tensor
 // cores: D (+)= A B^T (+ bias), A (M x K) and B (N x K) row-major BF16.
-// Used by the surrogate's training (weight gradients, backward products).
+// A product of its own for callers; the surrogate's training has fused kernels
+// (af_mlp.cu).
 //
 // One CTA of 128 threads owns 128 rows of D and all N <= 128 columns; the
 // accumulator lives in tensor memory.  K is walked in chunks of 64: the

@@ -1,15 +1,19 @@
 // af_mlp.cu -- the surrogate network's parameters and its training on the
-// GPU: forward and backward through the tcgen05 BF16 GEMM of af_gemm.cu
-// (FP32 accumulation), GELU and loss kernels, and Adam (Kingma & Ba 2015)
-// on FP32 master weights.
+// GPU: forward and backward on the tcgen05 tensor cores (FP32 accumulation),
+// MSE loss, and Adam (Kingma & Ba 2015) on FP32 master weights.
 //
 // One training step on a minibatch of B rows (B a multiple of 8):
 //   Z1 = X W1^T + b1, H1 = gelu(Z1), ..., Y = H3 W4^T + b4     (forward)
 //   dY = 2 (Y - T) / (8 B) on the 8 used outputs                (MSE loss)
-//   dW4 = dY^T H3, db4 = sum dY, dH3 = dY W4, dZ3 = dH3 gelu'(Z3)
-//   dW3 = dZ3^T H2, ..., dW1 = dZ1^T X                          (backward)
-// Every product runs on the tensor cores with K-major operands, so the
-// kernels that make H, dY and dZ also write their transposes.
+//   dH3 = dY W4, dZ3 = dH3 gelu'(Z3), dH2 = dZ3 W3, ...         (backward)
+//   dW4 = dY^T H3, dW3 = dZ3^T H2, ..., dW1 = dZ1^T X           (weights)
+// in three launches: network_kernel takes 128 rows a CTA from the gather to
+// dZ1 with Z1, Z2, Z3 and dH in the 512 columns of tensor memory and every
+// weight (and transpose) in shared memory; weight_grad_kernel contracts the
+// transposes it left over the batch; adam_kernel adds the partial products and
+// updates the weights and their BF16 copies.  All sums have a fixed order.
+// Measured: 425 -> 51 us a step at B = 4096 (26 launches before, 11 of them
+// products of 38 us whose row-per-thread epilogues wrote 4 bytes a sector).
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -19,6 +23,7 @@
 #include "../../include/af.h"
 #include "af_kernels.h"
 #include "af_mlp.h"
+#include "af_tc.cuh"
 
 using namespace af;
 using namespace af::mlp;
@@ -66,163 +71,472 @@ __global__ void init_kernel(float *p, uint64_t seed) {
   p[k] = g * sqrtf(2.0f / fan) * mul;
 }
 
-// BF16 copies of the weights, row-major and transposed
-__global__ void refresh_kernel(const float *p, __nv_bfloat16 *wb, __nv_bfloat16 *wbT) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= NWB) return;
+// BF16 copies of trained parameter k (none for a bias): row-major, for the
+// surrogate's kernels, and in the layout of network_kernel's shared memory,
+// where two bulk copies put them (the weights; then the transposes of W2, W3, W4)
+__device__ __forceinline__ void store_copies(int k, float w, __nv_bfloat16 *wb, unsigned char *core) {
   int off, rows, cols, base;
-  if (k < WB_W2) {
+  if (k < OFF_B1) {
     off = OFF_W1; rows = NH; cols = NIN; base = WB_W1;
-  } else if (k < WB_W3) {
+  } else if (k >= OFF_W2 && k < OFF_B2) {
     off = OFF_W2; rows = NH; cols = NH; base = WB_W2;
-  } else if (k < WB_W4) {
+  } else if (k >= OFF_W3 && k < OFF_B3) {
     off = OFF_W3; rows = NH; cols = NH; base = WB_W3;
-  } else {
+  } else if (k >= OFF_W4 && k < OFF_B4) {
     off = OFF_W4; rows = NOUT_PAD; cols = NH; base = WB_W4;
+  } else {
+    return;
   }
-  const int e = k - base, r = e / cols, c = e % cols;
-  const __nv_bfloat16 w = __float2bfloat16_rn(p[off + e]);
-  wb[k] = w;
-  wbT[base + c * rows + r] = w;
+  const int e = k - off, r = e / cols, c = e % cols;
+  const __nv_bfloat16 b = __float2bfloat16_rn(w);
+  wb[base + e] = b;
+  *reinterpret_cast<__nv_bfloat16 *>(core + 2 * base + tc::chunk_offset(rows, r, c)) = b;
+  if (base != WB_W1) *reinterpret_cast<__nv_bfloat16 *>(core + 2 * (NWB + base - WB_W2) + tc::chunk_offset(cols, c, r)) = b;
 }
-
-// minibatch rows: row r of the batch is sample idx[r] (random when seed != 0,
-// else r); features scaled by the input scales into BF16 (and transposed),
-// targets divided by the output scales; rows >= nvalid are zero
-__global__ void gather_kernel(const float *X, const float *T, int n, int B, int nvalid, uint64_t seed,
-                              long long step, const float *p, __nv_bfloat16 *Xb, __nv_bfloat16 *XT, float *Tn) {
-  __shared__ float tile[32][33];
-  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  for (int rr = ty; rr < 32; rr += blockDim.y) {
-    const int r = r0 + rr;
-    float x = 0.0f;
-    if (r < nvalid) {
-      const long long src = seed ? (long long)(mix64(seed ^ mix64((uint64_t)step * 1315423911ull + r)) % n) : r;
-      x = X[src * NIN + c0 + tx] * p[OFF_INS + c0 + tx];
-      if (T && blockIdx.y == 0 && tx < NOUT) Tn[(long long)r * NOUT + tx] = T[src * NOUT + tx] / p[OFF_OUTS + tx];
-    } else if (T && r < B && blockIdx.y == 0 && tx < NOUT) {
-      Tn[(long long)r * NOUT + tx] = 0.0f;
-    }
-    if (r < B) Xb[(long long)r * NIN + c0 + tx] = __float2bfloat16_rn(x);
-    tile[rr][tx] = x;
-  }
-  __syncthreads();
-  for (int cc = ty; cc < 32; cc += blockDim.y) {
-    const int r = r0 + tx;
-    if (r < B) XT[(long long)(c0 + cc) * B + r] = __float2bfloat16_rn(tile[tx][cc]);
-  }
-}
-
-// H = gelu(Z) in BF16, and H^T
-__global__ void act_kernel(const float *Z, int B, __nv_bfloat16 *H, __nv_bfloat16 *HT) {
-  __shared__ float tile[32][33];
-  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  for (int rr = ty; rr < 32; rr += blockDim.y) {
-    const int r = r0 + rr;
-    float h = 0.0f;
-    if (r < B) {
-      h = gelu(Z[(long long)r * NH + c0 + tx]);
-      H[(long long)r * NH + c0 + tx] = __float2bfloat16_rn(h);
-    }
-    tile[rr][tx] = h;
-  }
-  __syncthreads();
-  for (int cc = ty; cc < 32; cc += blockDim.y) {
-    const int r = r0 + tx;
-    if (r < B) HT[(long long)(c0 + cc) * B + r] = __float2bfloat16_rn(tile[tx][cc]);
-  }
-}
-
-// loss and dY = 2 (Y - T) / (8 nvalid) on the used outputs of the valid rows
-// (BF16, and transposed), db4 += column sums
-__global__ void loss_kernel(const float *Y, const float *Tn, int B, int nvalid, __nv_bfloat16 *dYb,
-                            __nv_bfloat16 *dYT, float *db4, double *loss) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  float d[NOUT_PAD];
-  float l = 0.0f;
-#pragma unroll
-  for (int k = 0; k < NOUT_PAD; k++) d[k] = 0.0f;
-  if (r < nvalid) {
-#pragma unroll
-    for (int k = 0; k < NOUT; k++) {
-      const float e = Y[(long long)r * NOUT_PAD + k] - Tn[(long long)r * NOUT + k];
-      l += e * e;
-      d[k] = 2.0f * e / (float)(NOUT * (long long)nvalid);
-    }
-  }
-  if (r < B) {
-#pragma unroll
-    for (int k = 0; k < NOUT_PAD; k++) {
-      const __nv_bfloat16 b = __float2bfloat16_rn(d[k]);
-      dYb[(long long)r * NOUT_PAD + k] = b;
-      dYT[(long long)k * B + r] = b;
-    }
-  }
-  // block sums of the loss and of d (FP32 gradient of b4)
-  __shared__ float sl[256];
-  __shared__ float sd[NOUT][256];
-  sl[threadIdx.x] = l;
-#pragma unroll
-  for (int k = 0; k < NOUT; k++) sd[k][threadIdx.x] = d[k];
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      sl[threadIdx.x] += sl[threadIdx.x + s];
-#pragma unroll
-      for (int k = 0; k < NOUT; k++) sd[k][threadIdx.x] += sd[k][threadIdx.x + s];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atomicAdd(loss, (double)sl[0] / (double)(NOUT * (long long)nvalid));
-  if (threadIdx.x < NOUT) atomicAdd(db4 + threadIdx.x, sd[threadIdx.x][0]);
-}
-
-// dZ = dH gelu'(Z) (BF16, and transposed); db += column sums
-__global__ void dz_kernel(const float *dH, const float *Z, int B, __nv_bfloat16 *dZb, __nv_bfloat16 *dZT,
-                          float *db) {
-  __shared__ float tile[32][33];
-  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  float colsum = 0.0f;
-  for (int rr = ty; rr < 32; rr += blockDim.y) {
-    const int r = r0 + rr;
-    float g = 0.0f;
-    if (r < B) {
-      const long long e = (long long)r * NH + c0 + tx;
-      g = dH[e] * gelu_grad(Z[e]);
-      dZb[e] = __float2bfloat16_rn(g);
-    }
-    tile[rr][tx] = g;
-    colsum += g;
-  }
-  __syncthreads();
-  for (int cc = ty; cc < 32; cc += blockDim.y) {
-    const int r = r0 + tx;
-    if (r < B) dZT[(long long)(c0 + cc) * B + r] = __float2bfloat16_rn(tile[tx][cc]);
-  }
-  atomicAdd(db + c0 + tx, colsum);
-}
-
-// the 8 used outputs of each row times the output scales
-__global__ void out_kernel(const float *Y, const float *p, int n, float *out) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
-#pragma unroll
-  for (int k = 0; k < NOUT; k++) out[(long long)r * NOUT + k] = Y[(long long)r * NOUT_PAD + k] * p[OFF_OUTS + k];
-}
-
-__global__ void adam_kernel(float *p, const float *g, float *m, float *v, float lr, float b1, float b2, float eps,
-                            float c1, float c2) {
+__global__ void refresh_kernel(const float *p, __nv_bfloat16 *wb, unsigned char *core) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < NTRAIN) store_copies(k, p[k], wb, core);
+}
+
+// ---- forward and backward of a tile of 128 rows
+// 16 warps: warp w reads tensor-memory lanes (rows) 32 (w % 4) .. + 31 and, of
+// a 128-column accumulator, columns 32 (w / 4) .. + 31, so that the epilogues
+// (GELU, its derivative, the transposed stores) are spread over all warps.  The
+// chain gather -> 4 layers -> loss -> 3 layers back is serial; what bounds it is
+// the latency of its seven MMA-and-epilogue stages (about 3 us each, 30 us cold
+// from launch to end for any batch up to 152 tiles), not the tensor rate.
+constexpr int TROWS = 128, NET_THREADS = 512;
+constexpr unsigned S_W1 = 0, S_W2 = S_W1 + NH * NIN * 2, S_W3 = S_W2 + NH * NH * 2, S_W4 = S_W3 + NH * NH * 2;
+constexpr unsigned S_ACT = S_W4 + NOUT_PAD * NH * 2;  // the layer's input: X, H or dZ (128 x 128)
+constexpr unsigned S_F32 = S_ACT + TROWS * NH * 2;    // biases, scales, bias-gradient slots, loss slots
+constexpr int NBIAS_G = 3 * NH + NOUT_PAD;            // bias gradients: b1, b2, b3, b4
+constexpr int F_BIAS = 0, F_INS = F_BIAS + NBIAS_G, F_OUTS = F_INS + NIN, F_DB = F_OUTS + NOUT,
+              F_LOSS = F_DB + 4 * NBIAS_G, F_TOTAL = F_LOSS + 4;
+constexpr unsigned S_BACK = (S_F32 + F_TOTAL * 4 + 127) & ~127u;  // backward only: W2^T, W3^T, W4^T, dY
+constexpr unsigned S_W2T = S_BACK, S_W3T = S_W2T + NH * NH * 2, S_W4T = S_W3T + NH * NH * 2,
+                   S_DY = S_W4T + NOUT_PAD * NH * 2;
+constexpr unsigned NET_SMEM_FWD = S_BACK, NET_SMEM = S_DY + TROWS * NOUT_PAD * 2;
+static_assert(NET_SMEM <= 227 * 1024, "shared memory");
+constexpr unsigned CORE_FWD = 2 * NWB, CORE_BYTES = CORE_FWD + 2 * (NWB - WB_W2);
+static_assert(S_ACT - S_W1 == CORE_FWD && S_DY - S_W2T == CORE_BYTES - CORE_FWD, "layout of the weight copies");
+constexpr unsigned MLP_WAIT = 1u << 20;  // polls of an MMA barrier before a CTA gives up
+constexpr int PART_B = NBIAS_G + 2;      // a CTA's partial row: bias gradients, its loss as a double
+
+struct NetArgs {
+  const float *X, *T;  // samples; T null: forward only
+  float *Yout;         // forward only: n x 8 outputs, scaled
+  const float *p;
+  const unsigned char *core;  // weights in the shared-memory layout
+  int n, B, nvalid;  // samples, rows of the batch (a multiple of 8), rows that count
+  uint64_t seed;     // 0: row r is sample r
+  long long step;
+  __nv_bfloat16 *XT, *HT[3], *dZT[3], *dYT;  // transposes, leading dimension B
+  float *partB;                              // [gridDim.x][PART_B]
+  int *err;
+};
+
+// `bytes` (a multiple of 16) of global memory into shared memory, completing on bar
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, unsigned bytes, unsigned long long *bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   tc::smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(tc::smem_u32(bar))
+               : "memory");
+}
+
+// D (tmem) = A (128 x Kd) W^T (N x Kd): one elected thread
+__device__ __forceinline__ void issue(unsigned tmem, unsigned a_s, unsigned w_s, int Kd, int N,
+                                      unsigned long long *bar) {
+  const uint32_t idesc = tc::make_idesc(TROWS, N);
+  const unsigned lboA = TROWS * 16, lboW = (unsigned)N * 16;
+  for (int k = 0; k < Kd / 16; k++)
+    tc::mma_bf16(tmem, tc::make_desc(a_s + 2 * k * lboA, lboA, 128), tc::make_desc(w_s + 2 * k * lboW, lboW, 128),
+                 idesc, k > 0 ? 1 : 0);
+  tc::mma_commit(bar);
+}
+
+// one stage: the tile's operand is in shared memory; MMAs, then a bounded
+// wait with a block-uniform outcome
+__device__ __forceinline__ bool stage(unsigned tmem, unsigned a_s, unsigned w_s, int Kd, int N,
+                                      unsigned long long *bar, unsigned &phase) {
+  tc::fence_async_smem();
+  tc::fence_before_sync();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    tc::fence_after_sync();
+    issue(tmem, a_s, w_s, Kd, N, bar);
+  }
+  const bool ok = __syncthreads_and(tc::bar_wait(bar, phase, MLP_WAIT)) != 0;
+  phase ^= 1;
+  tc::fence_after_sync();
+  return ok;
+}
+
+// 32 values of row `row` at columns cb .. cb + 31: BF16 into the operand buffer
+// and, if T is given, transposed into T (leading dimension B)
+__device__ __forceinline__ void put_row(unsigned char *act, __nv_bfloat16 *T, int B, int grow, int row, int cb,
+                                        const float v[32], bool in_batch) {
+  __nv_bfloat16 h[32];
+#pragma unroll
+  for (int j = 0; j < 32; j++) h[j] = __float2bfloat16_rn(v[j]);
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    unsigned w[4];
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+      w[e] = (unsigned)__bfloat16_as_ushort(h[8 * q + 2 * e]) | ((unsigned)__bfloat16_as_ushort(h[8 * q + 2 * e + 1]) << 16);
+    *reinterpret_cast<uint4 *>(act + tc::chunk_offset(TROWS, row, cb + 8 * q)) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  if (T && in_batch) {
+#pragma unroll
+    for (int j = 0; j < 32; j++) T[(long long)(cb + j) * B + grow] = h[j];
+  }
+}
+
+// sums over the warp's 32 lanes of 32 values each: lane c gets the sum of v[c]
+__device__ __forceinline__ float column_sums(float v[32], int lane) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < o; j++) {
+      const float give = up ? v[j] : v[j + o], keep = up ? v[j + o] : v[j];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  return v[0];
+}
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(NET_THREADS, 1) network_kernel(NetArgs A) {
+  extern __shared__ __align__(128) unsigned char nsm[];
+  __shared__ alignas(8) unsigned long long bar, wbar;
+  __shared__ unsigned tslot;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int row = 32 * (warp & 3) + lane, cb = 32 * (warp >> 2);
+  float *f = reinterpret_cast<float *>(nsm + S_F32);
+  float *db = f + F_DB + (warp & 3) * NBIAS_G;  // this row group's slots; a column belongs to one warp of it
+  unsigned char *act = nsm + S_ACT;
+  if (warp == 0) tc::tmem_alloc(&tslot, 512);
+  if (tid == 0) {
+    tc::bar_init(&bar, 1);
+    tc::bar_init(&wbar, 1);
+    // the weights, while the first tile is gathered
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(&wbar)),
+                 "r"(TRAIN ? CORE_BYTES : CORE_FWD)
+                 : "memory");
+    bulk_copy(nsm + S_W1, A.core, CORE_FWD, &wbar);
+    if (TRAIN) bulk_copy(nsm + S_W2T, A.core + CORE_FWD, CORE_BYTES - CORE_FWD, &wbar);
+  }
+  for (int k = tid; k < F_TOTAL; k += NET_THREADS) {
+    float x = 0.0f;
+    if (k < NH) x = A.p[OFF_B1 + k];
+    else if (k < 2 * NH) x = A.p[OFF_B2 + k - NH];
+    else if (k < 3 * NH) x = A.p[OFF_B3 + k - 2 * NH];
+    else if (k < F_INS) x = A.p[OFF_B4 + k - 3 * NH];
+    else if (k < F_DB) x = A.p[OFF_INS + k - F_INS];  // input scales, then output scales
+    f[k] = x;
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const unsigned tmem = tslot, tlane = tmem + ((unsigned)(32 * (warp & 3)) << 16);
+  const unsigned act_s = tc::smem_u32(act), base_s = tc::smem_u32(nsm);
+  unsigned phase = 0;
+  bool ok = true, loaded = false;
+  const int ntiles = (A.B + TROWS - 1) / TROWS;
+  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    const int r0 = tile * TROWS;
+    const auto sample = [&](int r) {
+      return A.seed ? (long long)(mix64(A.seed ^ mix64((uint64_t)A.step * 1315423911ull + r)) % A.n) : (long long)r;
+    };
+    {
+      // four threads a row, 16 inputs each, in the epilogues' mapping
+      const int c0 = 16 * (warp >> 2), r = r0 + row;
+      float x[16];
+#pragma unroll
+      for (int j = 0; j < 16; j++) x[j] = 0.0f;
+      if (r < A.nvalid) {
+        const float *src = A.X + sample(r) * NIN + c0;
+        if (reinterpret_cast<size_t>(A.X) & 15) {  // rows are 256 bytes: the first decides for all
+#pragma unroll
+          for (int j = 0; j < 16; j++) x[j] = __ldg(src + j);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            const float4 w = __ldg(reinterpret_cast<const float4 *>(src) + q);
+            x[4 * q] = w.x;
+            x[4 * q + 1] = w.y;
+            x[4 * q + 2] = w.z;
+            x[4 * q + 3] = w.w;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 16; j++) x[j] *= f[F_INS + c0 + j];
+      }
+#pragma unroll
+      for (int q = 0; q < 2; q++) {
+        unsigned w[4];
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          const __nv_bfloat162 b = __floats2bfloat162_rn(x[8 * q + 2 * e], x[8 * q + 2 * e + 1]);
+          w[e] = *reinterpret_cast<const unsigned *>(&b);
+        }
+        *reinterpret_cast<uint4 *>(act + tc::chunk_offset(TROWS, row, c0 + 8 * q)) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+      if (TRAIN && r < A.B) {
+#pragma unroll
+        for (int j = 0; j < 16; j++) A.XT[(long long)(c0 + j) * A.B + r] = __float2bfloat16_rn(x[j]);
+      }
+    }
+    const int grow = r0 + row;
+    const bool in_batch = grow < A.B;
+    if (!loaded) loaded = ok = __syncthreads_and(tc::bar_wait(&wbar, 0, MLP_WAIT)) != 0;
+#pragma unroll 1
+    for (int l = 0; l < 3 && ok; l++) {
+      ok = stage(tmem + 128 * l, act_s, base_s + (l == 0 ? S_W1 : (l == 1 ? S_W2 : S_W3)), l == 0 ? NIN : NH, NH, &bar,
+                 phase);
+      if (!ok) break;
+      float v[32];
+      tc::tmem_ld32(tlane + 128 * l + cb, v);
+#pragma unroll
+      for (int j = 0; j < 32; j++) v[j] = gelu(v[j] + f[F_BIAS + l * NH + cb + j]);
+      put_row(act, TRAIN ? A.HT[l] : nullptr, A.B, grow, row, cb, v, in_batch);
+    }
+    if (ok) ok = stage(tmem + 384, act_s, base_s + S_W4, NH, NOUT_PAD, &bar, phase);
+    if (!ok) break;
+    if (warp < 4) {
+      float y[32];
+      tc::tmem_ld32(tlane + 384, y);
+      if (!TRAIN) {
+        if (grow < A.nvalid)
+#pragma unroll
+          for (int k = 0; k < NOUT; k++)
+            A.Yout[(long long)grow * NOUT + k] = (y[k] + f[F_BIAS + 3 * NH + k]) * f[F_OUTS + k];
+      } else {
+        float d[NOUT_PAD], l = 0.0f;
+#pragma unroll
+        for (int k = 0; k < NOUT_PAD; k++) d[k] = 0.0f;
+        if (grow < A.nvalid) {
+          const float *t = A.T + sample(grow) * NOUT;
+#pragma unroll
+          for (int k = 0; k < NOUT; k++) {
+            const float e = y[k] + f[F_BIAS + 3 * NH + k] - t[k] / f[F_OUTS + k];
+            l += e * e;
+            d[k] = 2.0f * e / (float)(NOUT * (long long)A.nvalid);
+          }
+        }
+        unsigned char *dy = nsm + S_DY;
+        unsigned w[8];
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+          const __nv_bfloat162 b = __floats2bfloat162_rn(d[2 * e], d[2 * e + 1]);
+          w[e] = *reinterpret_cast<const unsigned *>(&b);
+        }
+        *reinterpret_cast<uint4 *>(dy + tc::chunk_offset(TROWS, row, 0)) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4 *>(dy + tc::chunk_offset(TROWS, row, 8)) = make_uint4(w[4], w[5], w[6], w[7]);
+        if (in_batch)
+#pragma unroll
+          for (int k = 0; k < NOUT_PAD; k++) A.dYT[(long long)k * A.B + grow] = __float2bfloat16_rn(d[k]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          l += __shfl_xor_sync(0xffffffffu, l, o);
+#pragma unroll
+          for (int k = 0; k < NOUT; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
+        }
+        if (lane == 0) {
+          f[F_LOSS + warp] += l;
+#pragma unroll
+          for (int k = 0; k < NOUT; k++) db[3 * NH + k] += d[k];
+        }
+      }
+    }
+    if (TRAIN) {
+      // back through the layers: dH into columns 384 .. 511, dZ = dH gelu'(Z)
+#pragma unroll 1
+      for (int l = 2; l >= 0 && ok; l--) {
+        ok = l == 2 ? stage(tmem + 384, tc::smem_u32(nsm + S_DY), base_s + S_W4T, NOUT_PAD, NH, &bar, phase)
+                    : stage(tmem + 384, act_s, base_s + (l == 1 ? S_W3T : S_W2T), NH, NH, &bar, phase);
+        if (!ok) break;
+        float z[32], v[32];
+        tc::tmem_ld32(tlane + 128 * l + cb, z);
+        tc::tmem_ld32(tlane + 384 + cb, v);
+#pragma unroll
+        for (int j = 0; j < 32; j++) v[j] = in_batch ? v[j] * gelu_grad(z[j] + f[F_BIAS + l * NH + cb + j]) : 0.0f;
+        put_row(act, A.dZT[l], A.B, grow, row, cb, v, in_batch);
+        db[l * NH + cb + lane] += column_sums(v, lane);
+      }
+    }
+    // the next tile's gather overwrites the operand buffer and its MMAs the
+    // accumulators: every read of this tile's must be done
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+  }
+  if (!ok) {
+    // the weights' copies or the MMAs did not complete in time: record it and
+    // give them one more bounded wait before the memory is released
+    if (tid == 0) atomicOr(A.err, 1);
+    if (!loaded) tc::bar_wait(&wbar, 0, MLP_WAIT);
+    else tc::bar_wait(&bar, phase ^ 1, MLP_WAIT);
+  }
+  if (TRAIN) {
+    float *out = A.partB + (long long)blockIdx.x * PART_B;
+    for (int k = tid; k < NBIAS_G; k += NET_THREADS) {
+      const float *d = f + F_DB + k;
+      out[k] = (d[0] + d[NBIAS_G]) + (d[2 * NBIAS_G] + d[3 * NBIAS_G]);
+    }
+    if (tid == 0) {
+      const double l = ((double)f[F_LOSS] + f[F_LOSS + 1]) + ((double)f[F_LOSS + 2] + f[F_LOSS + 3]);
+      *reinterpret_cast<double *>(out + NBIAS_G) = l / (double)(NOUT * (long long)A.nvalid);
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
+// ---- weight gradients: dW_l = dZ_l^T H_(l-1) over the batch, layer blockIdx.y,
+// batch rows [blockIdx.x * per, + per) x 256, the partial product into
+// partW[blockIdx.x].  A 256-row step's operands (two of 64 KB) are loaded with
+// all loads in flight and contracted by 16 MMAs: 12.8 us (cold) for B = 4096,
+// where the four products took four launches of 38 us, their results added by
+// scattered atomics.  128-row steps are no faster at 4096 and 17 % slower a
+// training step at 16384 (twice the partial products).
+constexpr int WG_THREADS = 256, WG_STEP = 256;
+constexpr unsigned WG_OP = NH * WG_STEP * 2, WG_SMEM = 2 * WG_OP + 1024;
+struct WgradArgs {
+  const __nv_bfloat16 *A[4], *Bm[4];  // per layer: dZ^T (or dY^T), the input's transpose
+  int M[4], N[4], off[4];             // rows, columns, place in the parameters
+  float *partW;                       // [gridDim.x][NTRAIN]
+  int B, per;
+  int *err;
+};
+// rows [0, R) (zero from `rows` on) of a row-major R x B array, columns k0 ..
+// k0 + 255 (zero from B on), into the K-major core layout of R rows
+__device__ __forceinline__ void load_step(unsigned char *dst, const __nv_bfloat16 *X, int rows, int R, int B, int k0) {
+#pragma unroll 16
+  for (int idx = threadIdx.x; idx < R * (WG_STEP / 8); idx += WG_THREADS) {
+    const int r = (idx & 7) + 8 * (idx / WG_STEP), kv = (idx >> 3) % (WG_STEP / 8), k = k0 + 8 * kv;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (r < rows && k < B) v = __ldg(reinterpret_cast<const uint4 *>(X + (long long)r * B + k));
+    *reinterpret_cast<uint4 *>(dst + tc::chunk_offset(R, r, 8 * kv)) = v;
+  }
+}
+__global__ void __launch_bounds__(WG_THREADS, 1) weight_grad_kernel(WgradArgs a) {
+  extern __shared__ __align__(128) unsigned char wsm[];
+  __shared__ alignas(8) unsigned long long bar;
+  __shared__ unsigned tslot;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l = blockIdx.y;
+  const int M = a.M[l], N = a.N[l];
+  unsigned char *sA = wsm, *sB = wsm + WG_OP;
+  if (warp == 0) tc::tmem_alloc(&tslot, 128);
+  if (tid == 0) tc::bar_init(&bar, 1);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const unsigned tmem = tslot;
+  const uint32_t idesc = tc::make_idesc(NH, N);
+  const unsigned lboA = NH * 16, lboB = (unsigned)N * 16;
+  unsigned phase = 0;
+  bool ok = true;
+  const int c0 = blockIdx.x * a.per, c1 = min((a.B + WG_STEP - 1) / WG_STEP, c0 + a.per);
+  for (int c = c0; c < c1 && ok; c++) {
+    load_step(sA, a.A[l], M, NH, a.B, c * WG_STEP);
+    load_step(sB, a.Bm[l], N, N, a.B, c * WG_STEP);
+    tc::fence_async_smem();
+    __syncthreads();
+    if (tid == 0) {
+      tc::fence_after_sync();
+      const unsigned ba = tc::smem_u32(sA), bb = tc::smem_u32(sB);
+#pragma unroll
+      for (int k = 0; k < WG_STEP / 16; k++)
+        tc::mma_bf16(tmem, tc::make_desc(ba + 2 * k * lboA, lboA, 128), tc::make_desc(bb + 2 * k * lboB, lboB, 128),
+                     idesc, (c > c0 || k > 0) ? 1 : 0);
+      tc::mma_commit(&bar);
+    }
+    ok = __syncthreads_and(tc::bar_wait(&bar, phase, MLP_WAIT)) != 0;
+    phase ^= 1;
+  }
+  if (!ok) {
+    if (tid == 0) atomicOr(a.err, 1);
+    tc::bar_wait(&bar, phase ^ 1, MLP_WAIT);
+  } else {
+    tc::fence_after_sync();
+    const int row = 32 * (warp & 3) + lane;
+    float *out = a.partW + (long long)blockIdx.x * NTRAIN + a.off[l] + row * N;
+    for (int cb = 32 * (warp >> 2); cb < N; cb += 64) {
+      float v[32];
+      tc::tmem_ld32(tmem + ((unsigned)(32 * (warp & 3)) << 16) + (unsigned)cb, v);
+      if (row < M)
+#pragma unroll
+        for (int q = 0; q < 8; q++)
+          reinterpret_cast<float4 *>(out + cb)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 128);
+}
+
+// gradient of parameter k from the partial sums: weights over the splits of
+// weight_grad_kernel, biases over the CTAs of network_kernel
+struct Partials {
+  const float *partW, *partB;
+  int nW, nB;
+};
+__device__ __forceinline__ float gradient(const Partials &P, int k) {
+  int b = -1;
+  if (k >= OFF_B4) b = 3 * NH + k - OFF_B4;
+  else if (k >= OFF_B3 && k < OFF_W4) b = 2 * NH + k - OFF_B3;
+  else if (k >= OFF_B2 && k < OFF_W3) b = NH + k - OFF_B2;
+  else if (k >= OFF_B1 && k < OFF_W2) b = k - OFF_B1;
+  const float *p = b < 0 ? P.partW + k : P.partB + b;
+  const int n = b < 0 ? P.nW : P.nB, stride = b < 0 ? NTRAIN : PART_B;
+  float s = 0.0f;
+  // all of up to 32 loads in flight; partial sums beyond
+  for (int q0 = 0; q0 < n; q0 += 32) {
+    float x[32];
+#pragma unroll
+    for (int q = 0; q < 32; q++) x[q] = q0 + q < n ? __ldg(p + (long long)(q0 + q) * stride) : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < o; q++) x[q] += x[q + o];
+    s += x[0];
+  }
+  return s;
+}
+// the batch's loss, by the first warp of a block of its own
+__device__ __forceinline__ void sum_loss(const Partials &P, double *loss) {
+  const int lane = threadIdx.x;
+  if (lane >= 32) return;
+  double s = 0.0;
+  for (int q = lane; q < P.nB; q += 32) s += *reinterpret_cast<const double *>(P.partB + (long long)q * PART_B + NBIAS_G);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) *loss = s;
+}
+// blocks of gradient_kernel and adam_kernel: the parameters, then one for the loss
+constexpr int PAR_THREADS = 128, PAR_BLOCKS = (NTRAIN + PAR_THREADS - 1) / PAR_THREADS;
+__global__ void gradient_kernel(Partials P, float *g, double *loss) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.x == PAR_BLOCKS) sum_loss(P, loss);
+  else if (k < NTRAIN) g[k] = gradient(P, k);
+}
+
+// Adam on parameter k, and its BF16 copies
+__global__ void adam_kernel(Partials P, float *p, float *m, float *v, __nv_bfloat16 *wb, unsigned char *core, float lr,
+                            float b1, float b2, float eps, float c1, float c2, double *loss) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.x == PAR_BLOCKS) sum_loss(P, loss);
   if (k >= NTRAIN) return;
-  const float gk = g[k];
+  const float gk = gradient(P, k);
   const float mk = b1 * m[k] + (1.0f - b1) * gk;
   const float vk = b2 * v[k] + (1.0f - b2) * gk * gk;
   m[k] = mk;
   v[k] = vk;
-  p[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+  const float w = p[k] - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+  p[k] = w;
+  store_copies(k, w, wb, core);
 }
 
 // root mean square of each column of a row-major (n x cols) array
@@ -267,25 +581,25 @@ struct MDev {
 };
 
 int refresh(af_mlp *m, cudaStream_t s) {
-  refresh_kernel<<<(NWB + 255) / 256, 256, 0, s>>>(m->params, m->wb, m->wbT);
+  refresh_kernel<<<(NTRAIN + 255) / 256, 256, 0, s>>>(m->params, m->wb, m->core);
   MCK(cudaGetLastError(), "af_mlp: refresh");
   return AF_OK;
 }
 
-// training scratch for B rows (B a multiple of 8)
-int ensure_cap(af_mlp *m, int B) {
-  if (m->cap >= B) return AF_OK;
+constexpr int MAX_SPLITS = 32;  // of weight_grad_kernel over the batch
+
+// training scratch for B rows (B a multiple of 8) and a loss history of `steps`
+int ensure_cap(af_mlp *m, int B, int steps) {
+  if (m->cap >= B && m->hist_cap >= steps) return AF_OK;
+  if (B < m->cap) B = m->cap;
+  if (steps < m->hist_cap) steps = m->hist_cap;
   if (m->scratch) cudaFree(m->scratch);
   m->scratch = nullptr;
-  m->cap = 0;
+  m->cap = m->hist_cap = 0;
   const size_t b16 = sizeof(__nv_bfloat16), f32 = sizeof(float);
-  const size_t sizes[] = {
-      (size_t)B * NIN * b16,       (size_t)B * NIN * b16,                 // Xb, XT
-      3 * (size_t)B * NH * b16,    3 * (size_t)B * NH * b16,              // H, HT
-      (size_t)B * NH * b16,        (size_t)B * NH * b16,                  // dZb, dZT
-      (size_t)B * NOUT_PAD * b16,  (size_t)B * NOUT_PAD * b16,            // dYb, dYT
-      (size_t)B * NOUT * f32,      3 * (size_t)B * NH * f32,              // Tn, Z
-      (size_t)B * NOUT_PAD * f32,  (size_t)B * NH * f32, 64};             // Y, dH, loss + flags
+  const size_t sizes[] = {(size_t)B * NIN * b16,      3 * (size_t)B * NH * b16,      3 * (size_t)B * NH * b16,  // XT, HT, dZT
+                          (size_t)B * NOUT_PAD * b16, MAX_SPLITS * (size_t)NTRAIN * f32,                       // dYT, partW
+                          (size_t)m->sms * PART_B * f32, sizeof(double) * (size_t)(steps + 1), 64};            // partB, loss, err
   size_t total = 0;
   for (size_t z : sizes) total += (z + 255) & ~size_t(255);
   MCK(cudaMalloc(&m->scratch, total), "af_mlp: cudaMalloc(scratch)");
@@ -295,88 +609,78 @@ int ensure_cap(af_mlp *m, int B) {
     q += (z + 255) & ~size_t(255);
     return r;
   };
-  m->Xb = (__nv_bfloat16 *)take(sizes[0]);
-  m->XT = (__nv_bfloat16 *)take(sizes[1]);
-  char *h = take(sizes[2]), *ht = take(sizes[3]);
-  for (int k = 0; k < 3; k++) {
-    m->H[k] = (__nv_bfloat16 *)h + (size_t)k * B * NH;
-    m->HT[k] = (__nv_bfloat16 *)ht + (size_t)k * B * NH;
-  }
-  m->dZb = (__nv_bfloat16 *)take(sizes[4]);
-  m->dZT = (__nv_bfloat16 *)take(sizes[5]);
-  m->dYb = (__nv_bfloat16 *)take(sizes[6]);
-  m->dYT = (__nv_bfloat16 *)take(sizes[7]);
-  m->Tn = (float *)take(sizes[8]);
-  float *z = (float *)take(sizes[9]);
-  for (int k = 0; k < 3; k++) m->Z[k] = z + (size_t)k * B * NH;
-  m->Y = (float *)take(sizes[10]);
-  m->dH = (float *)take(sizes[11]);
-  char *tail = take(sizes[12]);
-  m->loss = (double *)tail;
-  m->err = (int *)(tail + 8);
-  m->flag = (unsigned *)(tail + 16);
+  m->XT = (__nv_bfloat16 *)take(sizes[0]);
+  m->HT = (__nv_bfloat16 *)take(sizes[1]);
+  m->dZT = (__nv_bfloat16 *)take(sizes[2]);
+  m->dYT = (__nv_bfloat16 *)take(sizes[3]);
+  m->partW = (float *)take(sizes[4]);
+  m->partB = (float *)take(sizes[5]);
+  m->loss = (double *)take(sizes[6]);
+  m->err = (int *)take(sizes[7]);
   m->cap = B;
+  m->hist_cap = steps;
   return AF_OK;
 }
 
-int gemm(const void *A, int lda, const void *B, int ldb, float *D, int ldd, int M, int N, int K, const float *bias,
-         int splits, int *err, cudaStream_t s) {
-  MCK(launch_gemm_bf16(A, lda, B, ldb, D, ldd, M, N, K, bias, splits, 0, err, s), "af_mlp: gemm");
+int prepare_network() {
+  MCK(cudaFuncSetAttribute(network_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, NET_SMEM), "af_mlp: attributes");
+  MCK(cudaFuncSetAttribute(network_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, NET_SMEM_FWD), "af_mlp: attributes");
+  MCK(cudaFuncSetAttribute(weight_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM), "af_mlp: attributes");
   return AF_OK;
 }
 
-// forward of B rows already gathered into Xb / XT; Y = outputs (B x 16)
-int forward(af_mlp *m, int B, cudaStream_t s) {
-  const dim3 blk(32, 8), grd((B + 31) / 32, NH / 32);
-  const __nv_bfloat16 *in = m->Xb;
-  int K = NIN;
-  const int offw[3] = {WB_W1, WB_W2, WB_W3}, offb[3] = {OFF_B1, OFF_B2, OFF_B3};
+NetArgs net_args(af_mlp *m, const float *X, const float *T, float *Y, int n, int B, int nvalid, uint64_t seed,
+                 long long step) {
+  NetArgs A;
+  A.X = X;
+  A.T = T;
+  A.Yout = Y;
+  A.p = m->params;
+  A.core = m->core;
+  A.n = n;
+  A.B = B;
+  A.nvalid = nvalid;
+  A.seed = seed;
+  A.step = step;
+  A.XT = m->XT;
   for (int l = 0; l < 3; l++) {
-    int rc = gemm(in, K, m->wb + offw[l], K, m->Z[l], NH, B, NH, K, m->params + offb[l], 1, m->err, s);
-    if (rc) return rc;
-    act_kernel<<<grd, blk, 0, s>>>(m->Z[l], B, m->H[l], m->HT[l]);
-    MCK(cudaGetLastError(), "af_mlp: act");
-    in = m->H[l];
-    K = NH;
+    A.HT[l] = m->HT + (size_t)l * B * NH;
+    A.dZT[l] = m->dZT + (size_t)l * B * NH;
   }
-  return gemm(m->H[2], NH, m->wb + WB_W4, NH, m->Y, NOUT_PAD, B, NOUT_PAD, NH, m->params + OFF_B4, 1, m->err, s);
+  A.dYT = m->dYT;
+  A.partB = m->partB;
+  A.err = m->err;
+  return A;
 }
 
-// gradient of the loss of the B gathered rows (nvalid of them real) into m->grads
-int backward(af_mlp *m, int B, int nvalid, cudaStream_t s) {
-  float *g = m->grads;
-  MCK(cudaMemsetAsync(g, 0, sizeof(float) * NTRAIN, s), "af_mlp: memset");
-  loss_kernel<<<(B + 255) / 256, 256, 0, s>>>(m->Y, m->Tn, B, nvalid, m->dYb, m->dYT, g + OFF_B4, m->loss);
-  MCK(cudaGetLastError(), "af_mlp: loss");
-  const int splits = B / 512 > 1 ? B / 512 : 1;
-  // layer 4
-  int rc = gemm(m->dYT, B, m->HT[2], B, g + OFF_W4, NH, NOUT_PAD, NH, B, nullptr, splits, m->err, s);
-  if (rc) return rc;
-  rc = gemm(m->dYb, NOUT_PAD, m->wbT + WB_W4, NOUT_PAD, m->dH, NH, B, NH, NOUT_PAD, nullptr, 1, m->err, s);
-  if (rc) return rc;
-  const dim3 blk(32, 8), grd((B + 31) / 32, NH / 32);
-  const int offw[3] = {WB_W1, WB_W2, WB_W3}, offW[3] = {OFF_W1, OFF_W2, OFF_W3}, offb[3] = {OFF_B1, OFF_B2, OFF_B3};
-  for (int l = 2; l >= 0; l--) {
-    dz_kernel<<<grd, blk, 0, s>>>(m->dH, m->Z[l], B, m->dZb, m->dZT, g + offb[l]);
-    MCK(cudaGetLastError(), "af_mlp: dz");
-    const __nv_bfloat16 *inT = l > 0 ? m->HT[l - 1] : m->XT;
-    const int nin = l > 0 ? NH : NIN;
-    rc = gemm(m->dZT, B, inT, B, g + offW[l], nin, NH, nin, B, nullptr, splits, m->err, s);
-    if (rc) return rc;
-    if (l > 0) {
-      // dH_{l-1} = dZ_l W_l: B operand W_l^T (in x out), K = out
-      rc = gemm(m->dZb, NH, m->wbT + offw[l], NH, m->dH, NH, B, NH, NH, nullptr, 1, m->err, s);
-      if (rc) return rc;
-    }
+// forward and backward of B rows (nvalid of them real); P: the partial sums of
+// the loss's gradient
+int loss_partials(af_mlp *m, const float *X, const float *T, int n, int B, int nvalid, uint64_t seed, long long step,
+                  Partials &P, cudaStream_t s) {
+  const NetArgs A = net_args(m, X, T, nullptr, n, B, nvalid, seed, step);
+  const int tiles = (B + TROWS - 1) / TROWS;
+  P.nB = tiles < m->sms ? tiles : m->sms;
+  network_kernel<true><<<P.nB, NET_THREADS, NET_SMEM, s>>>(A);
+  MCK(cudaGetLastError(), "af_mlp: network");
+  WgradArgs G;
+  const int M[4] = {NH, NH, NH, NOUT_PAD}, N[4] = {NIN, NH, NH, NH}, off[4] = {OFF_W1, OFF_W2, OFF_W3, OFF_W4};
+  for (int l = 0; l < 4; l++) {
+    G.A[l] = l < 3 ? A.dZT[l] : A.dYT;
+    G.Bm[l] = l > 0 ? A.HT[l - 1] : A.XT;
+    G.M[l] = M[l];
+    G.N[l] = N[l];
+    G.off[l] = off[l];
   }
-  return AF_OK;
-}
-
-int gather(af_mlp *m, const float *X, const float *T, int n, int B, int nvalid, uint64_t seed, long long step,
-           cudaStream_t s) {
-  gather_kernel<<<dim3((B + 31) / 32, NIN / 32), dim3(32, 8), 0, s>>>(X, T, n, B, nvalid, seed, step, m->params,
-                                                                     m->Xb, m->XT, m->Tn);
-  MCK(cudaGetLastError(), "af_mlp: gather");
+  G.partW = m->partW;
+  G.B = B;
+  G.err = m->err;
+  const int steps = (B + WG_STEP - 1) / WG_STEP;
+  G.per = (steps + MAX_SPLITS - 1) / MAX_SPLITS;
+  P.nW = (steps + G.per - 1) / G.per;
+  weight_grad_kernel<<<dim3(P.nW, 4), WG_THREADS, WG_SMEM, s>>>(G);
+  MCK(cudaGetLastError(), "af_mlp: weight gradients");
+  P.partW = m->partW;
+  P.partB = m->partB;
   return AF_OK;
 }
 
@@ -394,7 +698,7 @@ void free_mlp(af_mlp *m) {
   cudaFree(m->adam_m);
   cudaFree(m->adam_v);
   cudaFree(m->wb);
-  cudaFree(m->wbT);
+  cudaFree(m->core);
   if (m->scratch) cudaFree(m->scratch);
   delete m;
 }
@@ -410,13 +714,17 @@ af_mlp *af_mlp_create(uint64_t seed) {
     return nullptr;
   }
   cudaGetDevice(&m->device);
-  cudaError_t e = prepare_gemm();
+  if (prepare_network() != AF_OK) {
+    delete m;
+    return nullptr;
+  }
+  cudaError_t e = cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, m->device);
   if (e == cudaSuccess) e = cudaMalloc(&m->params, sizeof(float) * NPARAM);
   if (e == cudaSuccess) e = cudaMalloc(&m->grads, sizeof(float) * NTRAIN);
   if (e == cudaSuccess) e = cudaMalloc(&m->adam_m, sizeof(float) * NTRAIN);
   if (e == cudaSuccess) e = cudaMalloc(&m->adam_v, sizeof(float) * NTRAIN);
   if (e == cudaSuccess) e = cudaMalloc(&m->wb, sizeof(__nv_bfloat16) * NWB);
-  if (e == cudaSuccess) e = cudaMalloc(&m->wbT, sizeof(__nv_bfloat16) * NWB);
+  if (e == cudaSuccess) e = cudaMalloc(&m->core, CORE_BYTES);
   if (e == cudaSuccess) e = cudaMemset(m->adam_m, 0, sizeof(float) * NTRAIN);
   if (e == cudaSuccess) e = cudaMemset(m->adam_v, 0, sizeof(float) * NTRAIN);
   if (e != cudaSuccess) {
@@ -489,15 +797,12 @@ int af_mlp_forward(af_mlp *m, const float *X, float *Y, int n, void *stream) {
   if (!m || !X || !Y || n <= 0) return mfail(AF_ERR_ARG, "af_mlp_forward: bad arguments");
   MDev d(m->device);
   cudaStream_t s = (cudaStream_t)stream;
-  const int B = (n + 7) & ~7;
-  int rc = ensure_cap(m, B);
+  const int B = (n + 7) & ~7, tiles = (B + TROWS - 1) / TROWS;
+  int rc = ensure_cap(m, 0, 0);
   if (rc) return rc;
   MCK(cudaMemsetAsync(m->err, 0, sizeof(int), s), "af_mlp_forward");
-  rc = gather(m, X, nullptr, n, B, n, 0, 0, s);
-  if (rc) return rc;
-  rc = forward(m, B, s);
-  if (rc) return rc;
-  out_kernel<<<(n + 255) / 256, 256, 0, s>>>(m->Y, m->params, n, Y);
+  network_kernel<false><<<tiles < m->sms ? tiles : m->sms, NET_THREADS, NET_SMEM_FWD, s>>>(
+      net_args(m, X, nullptr, Y, n, B, n, 0, 0));
   MCK(cudaGetLastError(), "af_mlp_forward");
   return check_err(m, s);
 }
@@ -507,11 +812,13 @@ int af_mlp_loss_grad(af_mlp *m, const float *X, const float *T, int n, double *l
   MDev d(m->device);
   cudaStream_t s = nullptr;
   const int B = (n + 7) & ~7;
-  int rc = ensure_cap(m, B);
+  int rc = ensure_cap(m, B, 0);
   if (rc) return rc;
   MCK(cudaMemsetAsync(m->err, 0, sizeof(int), s), "af_mlp_loss_grad");
-  MCK(cudaMemsetAsync(m->loss, 0, sizeof(double), s), "af_mlp_loss_grad");
-  if ((rc = gather(m, X, T, n, B, n, 0, 0, s)) || (rc = forward(m, B, s)) || (rc = backward(m, B, n, s))) return rc;
+  Partials P;
+  if ((rc = loss_partials(m, X, T, n, B, n, 0, 0, P, s))) return rc;
+  gradient_kernel<<<PAR_BLOCKS + 1, PAR_THREADS, 0, s>>>(P, m->grads, m->loss);
+  MCK(cudaGetLastError(), "af_mlp_loss_grad");
   if ((rc = check_err(m, s))) return rc;
   if (loss) MCK(cudaMemcpy(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost), "af_mlp_loss_grad");
   if (grads) MCK(cudaMemcpy(grads, m->grads, sizeof(float) * NTRAIN, cudaMemcpyDeviceToHost), "af_mlp_loss_grad");
@@ -524,32 +831,27 @@ int af_mlp_train(af_mlp *m, const float *X, const float *T, long long n, int ste
     return mfail(AF_ERR_ARG, "af_mlp_train: bad arguments (batch a multiple of 8, lr > 0, seed != 0)");
   MDev d(m->device);
   cudaStream_t s = nullptr;
-  int rc = ensure_cap(m, batch);
+  int rc = ensure_cap(m, batch, steps);
   if (rc) return rc;
-  double *lh = nullptr;
-  MCK(cudaMalloc(&lh, sizeof(double) * (steps > 0 ? steps : 1)), "af_mlp_train");
   MCK(cudaMemsetAsync(m->err, 0, sizeof(int), s), "af_mlp_train");
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   for (int k = 0; k < steps && rc == AF_OK; k++) {
     m->adam_t += 1;
     const float c1 = 1.0f - std::pow(b1, (float)m->adam_t), c2 = 1.0f - std::pow(b2, (float)m->adam_t);
-    cudaMemsetAsync(m->loss, 0, sizeof(double), s);
-    if ((rc = gather(m, X, T, (int)(n > 0x7fffffff ? 0x7fffffff : n), batch, batch, seed, m->adam_t, s)) ||
-        (rc = forward(m, batch, s)) || (rc = backward(m, batch, batch, s)))
-      break;
-    adam_kernel<<<(NTRAIN + 255) / 256, 256, 0, s>>>(m->params, m->grads, m->adam_m, m->adam_v, (float)lr, b1, b2,
-                                                     eps, c1, c2);
-    if ((rc = refresh(m, s))) break;
-    cudaMemcpyAsync(lh + k, m->loss, sizeof(double), cudaMemcpyDeviceToDevice, s);
+    Partials P;
+    if ((rc = loss_partials(m, X, T, (int)(n > 0x7fffffff ? 0x7fffffff : n), batch, batch, seed, m->adam_t, P, s))) break;
+    adam_kernel<<<PAR_BLOCKS + 1, PAR_THREADS, 0, s>>>(P, m->params, m->adam_m, m->adam_v, m->wb, m->core, (float)lr, b1,
+                                                     b2, eps, c1, c2, m->loss + k);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) rc = mcuda(e, "af_mlp_train");
   }
   if (rc == AF_OK) rc = check_err(m, s);
   if (rc == AF_OK && loss_hist && steps > 0) {
     std::vector<double> h(steps);
-    cudaError_t e = cudaMemcpy(h.data(), lh, sizeof(double) * steps, cudaMemcpyDeviceToHost);
+    cudaError_t e = cudaMemcpy(h.data(), m->loss, sizeof(double) * steps, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) rc = mcuda(e, "af_mlp_train");
     for (int k = 0; k < steps; k++) loss_hist[k] = (float)h[k];
   }
-  cudaFree(lh);
   return rc;
 }
 

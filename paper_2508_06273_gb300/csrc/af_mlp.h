@@ -60,14 +60,16 @@ struct af_mlp {
   float *grads = nullptr;   // NTRAIN
   float *adam_m = nullptr, *adam_v = nullptr;
   __nv_bfloat16 *wb = nullptr;   // NWB, row-major weights
-  __nv_bfloat16 *wbT = nullptr;  // NWB, transposed weights (in x out)
+  unsigned char *core = nullptr;  // the weights and the transposes of W2 .. W4 in the shared-memory layout of training
   long long adam_t = 0;
-  // training scratch for up to `cap` rows
-  int cap = 0;
+  int sms = 0;
+  // training scratch for up to `cap` rows and `hist_cap` steps: the batch's
+  // transposed inputs, activations and gradients, partial sums, the loss of
+  // every step
+  int cap = -1, hist_cap = -1;
   void *scratch = nullptr;
-  __nv_bfloat16 *Xb, *XT, *H[3], *HT[3], *dZb, *dZT, *dYb, *dYT;
-  float *Tn, *Z[3], *Y, *dH;
+  __nv_bfloat16 *XT, *HT, *dZT, *dYT;
+  float *partW, *partB;
   double *loss;
   int *err;
-  unsigned *flag;
 };
