@@ -19,7 +19,7 @@ LIB = os.path.join(OUT_DIR, "libaf.so")
 # af_debug_bounds in include/af.h): its own directory, never the default library
 CHECK_DIR = os.path.join(HERE, "_build_check")
 CHECK_LIB = os.path.join(CHECK_DIR, "libaf.so")
-SOURCES = ["af_api.cu", "af_misc.cu", "af_pointvalue.cu", "af_flux.cu", "af_noalloc.cu", "af_batch.cu", "af_gemm.cu", "af_mlp.cu", "af_surrogate.cu", "af_fp64.cu"]
+SOURCES = ["af_api.cu", "af_misc.cu", "af_pointvalue.cu", "af_pointvalue_shock.cu", "af_flux.cu", "af_noalloc.cu", "af_batch.cu", "af_gemm.cu", "af_mlp.cu", "af_surrogate.cu", "af_fp64.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

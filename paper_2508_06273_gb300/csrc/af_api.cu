@@ -1,6 +1,6 @@
 // af_api.cu -- the C ABI of include/af.h: handle, device state, transfers,
 // step sequencing and reductions.  All numerical work is in the kernels of
-// af_misc.cu, af_pointvalue.cu and af_flux.cu.
+// af_misc.cu, af_pointvalue.cuh and af_flux.cu.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -98,31 +98,38 @@ int ensure_staging(af_ctx *h) {
   return AF_OK;
 }
 
-// device external arrays -> padded planes (after the periodic-duplicate check)
+// the words of host_words that kernels write: [0], [1] export_words_kernel;
+// [4], [5] the wave speed's bits and bad flag; [6] a differing periodic duplicate
+enum { HW_SPEED = 4, HW_BAD = 6 };
+
+void drop_runs(af_ctx *h) {
+  for (int p = 0; p < 2; p++)
+    if (h->run_exec[p]) {
+      cudaGraphExecDestroy(h->run_exec[p]);
+      h->run_exec[p] = nullptr;
+    }
+}
+
+// device external arrays -> padded planes with their ghosts, low words, status
+// and wave speed (after the periodic-duplicate check)
 int load_state(af_ctx *h, const float *const src[4]) {
   h->speed_valid = false;
   cudaStream_t s = h->stream;
-  CK(cudaMemsetAsync(h->d_bad, 0, sizeof(int), s), "memset");
-  for (int w = 1; w < 4; w++) {
-    int ni, nj;
-    extents(h, w, ni, nj);
-    const int dup_x = h->g.per_x && (w == 1 || w == 2), dup_y = h->g.per_y && (w == 1 || w == 3);
-    if (dup_x || dup_y) CK(launch_check_dup(src[w], ni, nj, dup_x, dup_y, h->d_bad, s), "check_dup");
+  h->host_words[HW_BAD] = 0;
+  CK(launch_check_state(h->g, src, h->host_words_dev + HW_BAD, h->d_speed, h->d_speed_bad, s), "check_dup");
+  if (h->g.per_x || h->g.per_y) {
+    CK(cudaStreamSynchronize(s), "sync");
+    if (reinterpret_cast<volatile unsigned *>(h->host_words)[HW_BAD])
+      return fail(AF_ERR_ARG, "periodic state: the duplicated last node line differs from the first%s");
   }
-  int bad = 0;
-  CK(cudaMemcpyAsync(&bad, h->d_bad, sizeof(int), cudaMemcpyDeviceToHost, s), "memcpy");
-  CK(cudaStreamSynchronize(s), "sync");
-  if (bad) return fail(AF_ERR_ARG, "periodic state: the duplicated last node line differs from the first%s");
-  float *dst[4] = {h->hi, h->lev[0].k[VTX], h->lev[0].k[XE], h->lev[0].k[YE]};
-  for (int w = 0; w < 4; w++) {
-    int ni, nj;
-    extents(h, w, ni, nj);
-    CK(launch_pack(h->g, src[w], dst[w], ni, nj, true, s), "pack");
-  }
-  CK(cudaMemsetAsync(h->lo, 0, sizeof(float) * NV * h->g.plane, s), "memset lo");
-  CK(cudaMemsetAsync(h->d_status, 0, sizeof(int), s), "memset status");
+  const StateArrays a = {{src[0], src[1], src[2], src[3]}, {h->hi, h->lev[0].k[VTX], h->lev[0].k[XE], h->lev[0].k[YE]}};
+  CK(launch_load_state(h->g, a, h->lo, h->d_status, h->d_speed, h->d_speed_bad, h->host_words_dev + HW_SPEED, h->d_ticket,
+                       s),
+     "load");
   h->has_state = true;
   h->half_valid = false;
+  h->speed_valid = h->speed_on_host = true;
+  h->ghost_valid = true;
   return AF_OK;
 }
 
@@ -215,10 +222,18 @@ af_ctx *af_create(int nx, int ny, double dx, double dy, double gamma, uint32_t b
       return nullptr;
     }
   }
+  h->tile_h = 8;
+  // A small grid leaves SMs idle: its tiles are 4 rows high with one block a
+  // node kind, so that a step's critical path is the vertex's update instead of
+  // three nodes'.  Up to two blocks an SM (8 rows, split, us a step: 32^2
+  // 18.9, 14.4; 96^2 18.9, 15.4; 256^2, beyond the line, 25.9, 27.8).
+  const long long tiles4 = (long long)((g.nxv + 31) / 32) * ((g.nyv + 3) / 4);
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+  h->tile_pv = tiles4 * 3 <= 2LL * sms ? TILE_SPLIT : 8;
   for (int b = 0; b < 2; b++) {
-    cudaError_t te = make_tile_maps(g, h->tbuf[b].k[VTX], h->tbuf[b].k[XE], h->tbuf[b].k[YE], h->hi, 8,
+    cudaError_t te = make_tile_maps(g, h->tbuf[b].k[VTX], h->tbuf[b].k[XE], h->tbuf[b].k[YE], h->hi, h->tile_pv,
                                    &h->tmaps[b]);
-    h->tile_h = 8;
     if (te != cudaSuccess) {
       cuda_fail(te, "af_create: TMA descriptors");
       cudaFree(h->base);
@@ -247,9 +262,10 @@ af_ctx *af_create(int nx, int ny, double dx, double dy, double gamma, uint32_t b
   h->d_bad = (int *)(sp + 64);
   h->d_bad_async = (int *)(sp + 96);
   h->d_speed = (unsigned *)(sp + 128);
+  h->d_ticket = (unsigned *)(sp + 136);
   h->d_speed_bad = (int *)(sp + 160);
-  h->d_counters = (unsigned long long *)(sp + 192);
-  h->d_min_keys = (unsigned *)(sp + 224);
+  h->d_min_keys = (unsigned *)(sp + 164);
+  h->d_counters = (unsigned long long *)(sp + 192);  // two slots of four
   h->d_totals = (double *)(sp + 256);
   h->d_partials = h->d_totals + NV;
   h->stream = h->own_stream;
@@ -390,12 +406,8 @@ int af_set_option(af_ctx *h, int key, double value) {
     }
     case AF_OPT_KEEP_HALF:
       if ((iv != 0) != (h->keep_half != 0)) {
-        for (int p = 0; p < 2; p++)  // captured steps hold the old launch arguments
-          if (h->run_exec[p]) {
-            DeviceGuard dg(h->device);
-            cudaGraphExecDestroy(h->run_exec[p]);
-            h->run_exec[p] = nullptr;
-          }
+        DeviceGuard dg(h->device);
+        drop_runs(h);  // captured steps hold the old launch arguments
       }
       h->keep_half = iv != 0;
       return AF_OK;
@@ -413,13 +425,13 @@ int af_set_option(af_ctx *h, int key, double value) {
       return AF_OK;
     case AF_OPT_TILE_H: {
       if (iv != 4 && iv != 8 && iv != 16) return fail(AF_ERR_ARG, "tile height must be 4, 8 or 16%s");
-      if (iv == h->tile_h) return AF_OK;
+      if (iv == h->tile_pv) return AF_OK;
       DeviceGuard dg(h->device);
       CK(cudaStreamSynchronize(h->stream), "sync");
       for (int b = 0; b < 2; b++)
         CK(make_tile_maps(h->g, h->tbuf[b].k[VTX], h->tbuf[b].k[XE], h->tbuf[b].k[YE], h->hi, iv, &h->tmaps[b]),
            "TMA descriptors");
-      h->tile_h = iv;
+      h->tile_h = h->tile_pv = iv;
       for (int p = 0; p < 2; p++)  // captured steps hold the old launch shape
         if (h->run_exec[p]) {
           cudaGraphExecDestroy(h->run_exec[p]);
@@ -487,6 +499,7 @@ int af_set_state_host(af_ctx *h, const float *avg, const float *vtx, const float
     if (rc) return rc;
   }
   h->speed_valid = false;
+  h->ghost_valid = false;
   if (!avg || !vtx || !xe || !ye) return fail(AF_ERR_ARG, "af_set_state_host: null array%s");
   DeviceGuard dg(h->device);
   int rc = ensure_staging(h);
@@ -538,28 +551,24 @@ static int get_arrays(af_ctx *h, NodeSet &ns, const float *avgsrc, float *dst[4]
     for (int w = 0; w < 4; w++)
       if (dst[w] && !is_device_ptr(dst[w])) return fail(AF_ERR_ARG, "arrays must be device memory%s");
     order_after(h, user);
-  } else {
-    int rc = ensure_staging(h);
-    if (rc) return rc;
+    CK(launch_store_state(h->g, src, dst, s), "pack");
+    order_before(h, user);
+    return AF_OK;
   }
+  int rc = ensure_staging(h);
+  if (rc) return rc;
   for (int w = 0; w < 4; w++) {
     if (!dst[w] || !src[w]) continue;
     int ni, nj;
     extents(h, w, ni, nj);
-    if (!host) {
-      CK(launch_pack(h->g, src[w], dst[w], ni, nj, false, s), "pack");
-    } else {
-      // pack on the handle's stream, copy out on the array's own stream
-      float *stg = h->staging + h->staging_off[w];
-      CK(launch_pack(h->g, src[w], stg, ni, nj, false, s), "pack");
-      CK(cudaEventRecord(h->xev[w], s), "event");
-      CK(cudaStreamWaitEvent(h->xs[w], h->xev[w], 0), "event");
-      CK(cudaMemcpyAsync(dst[w], stg, sizeof(float) * NV * ni * nj, cudaMemcpyDeviceToHost, h->xs[w]), "D2H");
-    }
+    // pack on the handle's stream, copy out on the array's own stream
+    float *stg = h->staging + h->staging_off[w];
+    CK(launch_pack(h->g, src[w], stg, ni, nj, false, s), "pack");
+    CK(cudaEventRecord(h->xev[w], s), "event");
+    CK(cudaStreamWaitEvent(h->xs[w], h->xev[w], 0), "event");
+    CK(cudaMemcpyAsync(dst[w], stg, sizeof(float) * NV * ni * nj, cudaMemcpyDeviceToHost, h->xs[w]), "D2H");
   }
-  if (host)
-    for (int w = 0; w < 4; w++) CK(cudaStreamSynchronize(h->xs[w]), "sync");
-  if (!host) order_before(h, user);
+  for (int w = 0; w < 4; w++) CK(cudaStreamSynchronize(h->xs[w]), "sync");
   return AF_OK;
 }
 
@@ -681,6 +690,7 @@ int af_set_state_host_async(af_ctx *h, const float *avg, const float *vtx, const
   CK(cudaMemsetAsync(h->lo, 0, sizeof(float) * NV * h->g.plane, s), "memset lo");
   CK(cudaMemsetAsync(h->d_status, 0, sizeof(int), s), "memset status");
   h->speed_valid = false;
+  h->ghost_valid = false;
   h->has_state = true;
   h->half_valid = false;
   h->async_pending = true;
@@ -760,7 +770,7 @@ int af_get_avg_lo(af_ctx *h, float *avg_lo, void *stream) {
 }
 
 int af_set_avg_lo(af_ctx *h, const float *avg_lo, void *stream) {
-  h->speed_valid = false;
+  if (h) h->speed_valid = h->ghost_valid = false;
   if (!h || !is_device_ptr(avg_lo)) return fail(AF_ERR_ARG, "af_set_avg_lo: need a device array%s");
   if (!h->has_state) return fail(AF_ERR_STATE, "no state set%s");
   DeviceGuard dg(h->device);
@@ -783,6 +793,15 @@ static void collect_stages(af_ctx *h) {
   h->stage_pending = false;
 }
 
+// ghost entries of the current state, if the kernel that wrote it did not fill them
+static int fill_ghosts(af_ctx *h) {
+  if (h->ghost_valid) return AF_OK;
+  CK(launch_ghost_fill(h->g, h->hi, h->lo, h->lev[0], h->stream), "ghost fill");
+  h->launches[AF_STAGE_PREP] += 1;
+  h->ghost_valid = true;
+  return AF_OK;
+}
+
 static int enqueue_step(af_ctx *h, double dt) {
   cudaStream_t s = h->stream;
   const bool prof = h->profile != 0;
@@ -792,10 +811,10 @@ static int enqueue_step(af_ctx *h, double dt) {
   }
   {
     NvtxScope st("ghost fill");
-    CK(launch_ghost_fill(h->g, h->hi, h->lo, h->lev[0], s), "ghost fill");
+    int rc = fill_ghosts(h);  // (a step leaves its new state's ghosts filled)
+    if (rc) return rc;
   }
-  h->launches[AF_STAGE_PREP] += 1;
-  CK(cudaMemsetAsync(h->d_counters, 0, 4 * sizeof(unsigned long long), s), "memset counters");
+  unsigned long long *counters = h->d_counters + 4 * h->tmap_cur;
   const float *theta[2] = {nullptr, nullptr};
   if (h->opt.shock_blend) {
     theta[0] = h->shock_theta;
@@ -808,7 +827,9 @@ static int enqueue_step(af_ctx *h, double dt) {
     NvtxScope pvr("point values");
     if (h->opt.surrogate) {
       // network at every node, then the exact operator at the nodes it rejected
-      CK(cudaMemsetAsync(h->surr_tiles, 0, sizeof(int) * h->surr_tiles_x * ((h->g.nyv + h->tile_h - 1) / h->tile_h), s),
+      // (all three kinds of a flagged tile in one block)
+      const int tile = h->tile_pv == TILE_SPLIT ? 4 : h->tile_pv, tile_rows = tile;
+      CK(cudaMemsetAsync(h->surr_tiles, 0, sizeof(int) * h->surr_tiles_x * ((h->g.nyv + tile_rows - 1) / tile_rows), s),
          "memset tiles");
       CK(launch_ubar(h->g, h->hi, h->lev[0], h->surr_ubar, s), "surrogate cell prep");
       const unsigned char *mask[3];
@@ -833,7 +854,7 @@ static int enqueue_step(af_ctx *h, double dt) {
         mask[k] = A.mask;
         A.tile_flag = h->surr_tiles;
         A.tiles_x = h->surr_tiles_x;
-        A.tile_rows = h->tile_h;
+        A.tile_rows = tile_rows;
         A.stats = h->surr_stats;
         A.status = h->d_status;
         A.test_no_issue = h->opt.test_timeout != 0;
@@ -841,7 +862,8 @@ static int enqueue_step(af_ctx *h, double dt) {
         CK(launch_surrogate(k, A, h->sms, s), "surrogate");
       }
       CK(launch_pointvalue_masked(h->g, h->lev[0], h->hi, h->tmaps[h->tmap_cur], h->lev[1], h->lev[2], (float)dt,
-                                  h->opt, h->d_status, h->d_counters, mask, h->surr_tiles, theta, h->tile_h, s),
+                                  h->opt, h->d_status, counters, mask, h->surr_tiles, theta, tile, h->d_speed,
+                                  h->d_speed_bad, s),
          "point values (fallback)");
       h->launches[AF_STAGE_POINTVALUE] += 5;
       h->half_valid = true;
@@ -849,7 +871,7 @@ static int enqueue_step(af_ctx *h, double dt) {
       // plain path: t^{n+1/2} and t^{n+1} written, the flux kernel forms the
       // node fluxes from three levels
       CK(launch_pointvalue(h->g, h->lev[0], h->hi, h->tmaps[h->tmap_cur], h->lev[1], h->lev[2], (float)dt,
-                           h->opt, h->d_status, h->d_counters, theta, h->tile_h, nullptr, s),
+                           h->opt, h->d_status, counters, theta, h->tile_pv, nullptr, h->d_speed, h->d_speed_bad, s),
          "point values");
       h->launches[AF_STAGE_POINTVALUE] += 1;
       h->half_valid = true;
@@ -864,7 +886,7 @@ static int enqueue_step(af_ctx *h, double dt) {
       CK(cudaMemsetAsync(h->d_speed, 0, sizeof(unsigned), s), "memset speed");
       CK(cudaMemsetAsync(h->d_speed_bad, 0, sizeof(int), s), "memset speed");
       CK(launch_pointvalue(h->g, h->lev[0], h->hi, h->tmaps[h->tmap_cur], h->lev[1], h->lev[2], (float)dt,
-                           h->opt, h->d_status, h->d_counters, theta, h->tile_h, &nf, s),
+                           h->opt, h->d_status, counters, theta, h->tile_pv, &nf, nullptr, nullptr, s),
          "point values");
       h->launches[AF_STAGE_POINTVALUE] += 1;
       h->half_valid = h->keep_half != 0;
@@ -879,17 +901,23 @@ static int enqueue_step(af_ctx *h, double dt) {
   if (h->opt.flux_limiter)
     CK(cudaMemcpyAsync(h->q0, h->hi, sizeof(float) * NV * (size_t)h->g.plane, cudaMemcpyDeviceToDevice, s),
        "flux limiter snapshot");
+  // the flux kernel also clears the next step's counters and, on a small grid,
+  // fills the new state's ghosts and hands the wave speed to the host
+  const bool small = flux_fills_ghosts(h->g);
+  const StepTail tail = {h->lev[2], h->d_counters + 4 * (h->tmap_cur ^ 1), small ? h->host_words_dev + HW_SPEED : nullptr,
+                         small ? h->d_ticket : nullptr};
   if (h->opt.surrogate || !h->opt.node_flux) {
     CK(launch_flux_update(h->g, h->lev[0], h->lev[1], h->lev[2], h->hi, h->lo, dt / h->dx, dt / h->dy,
-                          h->d_status, h->d_speed, h->d_speed_bad, h->opt.flux_limiter, h->q0, s),
+                          h->d_status, h->d_speed, h->d_speed_bad, h->opt.flux_limiter, h->q0, tail, s),
        "flux update");
   } else {
     const float *nf[4] = {h->nflux[0], h->nflux[1], h->nflux[2], h->nflux[3]};
     CK(launch_flux_nf(h->g, nf, h->hi, h->lo, dt / h->dx, dt / h->dy, h->d_status, h->d_speed, h->d_speed_bad,
-                      h->opt.flux_limiter, h->q0, s),
+                      h->opt.flux_limiter, h->q0, tail, s),
        "flux update");
   }
   h->speed_valid = true;
+  h->speed_on_host = h->ghost_valid = small;
   h->launches[AF_STAGE_FLUX] += 1;
   if (prof) {
     cudaEventRecord(h->ev_stage[4], s);
@@ -1018,6 +1046,14 @@ int af_run(af_ctx *h, int nsteps, double dt) {
     return AF_OK;
   }
   const int p = h->tmap_cur;
+  {
+    // (a small grid's captured steps start from filled ghosts and fill them;
+    // a large grid's begin with the fill)
+    int rc = AF_OK;
+    if (flux_fills_ghosts(h->g)) rc = fill_ghosts(h);
+    else h->ghost_valid = false;
+    if (rc) return rc;
+  }
   if (!h->run_exec[p] || h->run_dt[p] != dt || !same_options(h->run_opt[p], h->opt)) {
     NvtxScope cap("af_run/capture");
     int rc = capture_pair(h, dt);
@@ -1025,11 +1061,12 @@ int af_run(af_ctx *h, int nsteps, double dt) {
   }
   for (int k = 0; k + 1 < nsteps; k += 2) {
     CK(cudaGraphLaunch(h->run_exec[p], h->stream), "af_run: graph launch");
-    h->launches[AF_STAGE_PREP] += 2;
+    if (!flux_fills_ghosts(h->g)) h->launches[AF_STAGE_PREP] += 2;
     h->launches[AF_STAGE_POINTVALUE] += h->opt.surrogate ? 10 : 2;
     h->launches[AF_STAGE_FLUX] += 2;
   }
   h->speed_valid = true;
+  h->speed_on_host = h->ghost_valid = flux_fills_ghosts(h->g);
   if (nsteps & 1) return enqueue_step(h, dt);
   return AF_OK;
 }
@@ -1037,7 +1074,8 @@ int af_run(af_ctx *h, int nsteps, double dt) {
 int af_debug_bounds(unsigned *out) {
   if (!out) return fail(AF_ERR_ARG, "null argument%s");
   CK(cudaDeviceSynchronize(), "af_debug_bounds: sync");
-  *out = af::bounds_flux() | af::bounds_fp64() | af::bounds_misc() | af::bounds_pointvalue() | af::bounds_surrogate();
+  *out = af::bounds_flux() | af::bounds_fp64() | af::bounds_misc() | af::bounds_pointvalue() | af::bounds_pointvalue_shock() |
+         af::bounds_surrogate();
 #ifdef AF_CHECK_BOUNDS
   return 1;
 #else
@@ -1060,7 +1098,7 @@ int af_counters(af_ctx *h, int64_t out[4]) {
   if (!h || !out) return fail(AF_ERR_ARG, "null argument%s");
   DeviceGuard dg(h->device);
   unsigned long long c[4];
-  CK(cudaMemcpyAsync(c, h->d_counters, sizeof(c), cudaMemcpyDeviceToHost, h->stream), "counters");
+  CK(cudaMemcpyAsync(c, h->d_counters + 4 * (h->tmap_cur ^ 1), sizeof(c), cudaMemcpyDeviceToHost, h->stream), "counters");
   CK(cudaStreamSynchronize(h->stream), "sync");
   for (int k = 0; k < 4; k++) out[k] = (int64_t)c[k];
   return AF_OK;
@@ -1132,10 +1170,17 @@ int af_max_speed(af_ctx *h, float *out) {
     *out = bad ? NAN : (float)m;
     return AF_OK;
   }
-  if (h->speed_valid) {  // computed by the last step's flux kernel
+  volatile unsigned *w = h->host_words;
+  if (h->speed_valid) {  // computed by the last step's flux kernel or with the state's load
     unsigned bits = 0;
     int bad = 0;
-    CK(read_speed(h, bits, bad), "speed");
+    if (h->speed_on_host) {
+      CK(cudaStreamSynchronize(h->stream), "sync");
+      bits = w[HW_SPEED];
+      bad = (int)w[HW_SPEED + 1];
+    } else {
+      CK(read_speed(h, bits, bad), "speed");
+    }
     float m;
     std::memcpy(&m, &bits, sizeof(m));
     *out = bad ? NAN : m;
@@ -1164,6 +1209,7 @@ int af_max_speed(af_ctx *h, float *out) {
   std::memcpy(&m, &bits, sizeof(m));
   *out = bad ? NAN : m;
   h->speed_valid = true;
+  h->speed_on_host = false;
   return AF_OK;
 }
 
@@ -1190,6 +1236,7 @@ int af_set_inflow(af_ctx *h, int side, const double U[4]) {
   DeviceGuard dg(h->device);
   CK(cudaStreamSynchronize(h->stream), "sync");
   for (int v = 0; v < NV; v++) h->g.inflow[side][v] = (float)U[v];
+  h->ghost_valid = false;
   for (int p = 0; p < 2; p++)  // captured steps hold the old grid description
     if (h->run_exec[p]) {
       cudaGraphExecDestroy(h->run_exec[p]);

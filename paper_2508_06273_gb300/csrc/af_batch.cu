@@ -51,7 +51,11 @@ struct af_batch {
   Grid *d_grids = nullptr;
   float **d_arrays = nullptr;      // [n][2][5]
   int4 *d_pv_tiles = nullptr, *d_fx_tiles = nullptr;
-  int n_pv_tiles = 0, n_fx_tiles = 0, pv_tiles_h = 0;
+  // point-value tiles by class of their instance (the kernel instantiation its
+  // options need; class of instance k in cls[k])
+  std::vector<int> cls;
+  int n_pv_tiles[PV_CLASSES] = {};
+  int n_fx_tiles = 0, pv_tiles_h = 0;
   int n_fx_plain = -1;  // flux tiles of instances without the flux limiter (listed first)
   int4 *d_ghost_chunks = nullptr;  // (instance, array, first entry) per ghost-fill block
   int n_ghost_chunks = 0;
@@ -156,6 +160,13 @@ int upload_args(af_batch *b) {
     theta[2 * k + 1] = h->opt.shock_blend ? h->shock_theta + h->g.plane : nullptr;
     if (h->opt.shock_blend) any_blend = true;
   }
+  std::vector<int> cls(b->n);
+  for (int k = 0; k < b->n; k++) cls[k] = batch_class(pv[2 * k]);
+  if (cls != b->cls) {  // the tile list is ordered by class
+    b->cls = cls;
+    b->maps_ok = false;
+    drop_graphs(b);
+  }
   BCK(cudaMemcpy(b->d_pv, pv.data(), sizeof(PointValueArgs) * pv.size(), cudaMemcpyHostToDevice), "batch: args");
   BCK(cudaMemcpy(b->d_fx, fx.data(), sizeof(FluxArgs) * fx.size(), cudaMemcpyHostToDevice), "batch: args");
   BCK(cudaMemcpy(b->d_arrays, arrays.data(), sizeof(float *) * arrays.size(), cudaMemcpyHostToDevice),
@@ -219,15 +230,22 @@ int build_tiles(af_batch *b) {
                                      &maps[2 * k + q]);
       if (e != cudaSuccess) return bcuda(e, "batch: TMA descriptors");
     }
-    for (int j0 = 0; j0 < g.nyv; j0 += b->tile_h)
-      for (int i0 = 0; i0 < g.nxv; i0 += 32) pv.push_back(make_int4(k, i0, j0, 0));
+  }
+  for (int c = 0; c < PV_CLASSES; c++) {
+    const size_t before = pv.size();
+    for (int k = 0; k < b->n; k++) {
+      const Grid &g = b->inst[k]->g;
+      if (b->cls[k] != c) continue;
+      for (int j0 = 0; j0 < g.nyv; j0 += b->tile_h)
+        for (int i0 = 0; i0 < g.nxv; i0 += 32) pv.push_back(make_int4(k, i0, j0, 0));
+    }
+    b->n_pv_tiles[c] = (int)(pv.size() - before);
   }
   if (b->d_pv_tiles) cudaFree(b->d_pv_tiles);
   b->d_pv_tiles = nullptr;
   BCK(cudaMalloc(&b->d_pv_tiles, sizeof(int4) * pv.size()), "batch: cudaMalloc(tiles)");
   BCK(cudaMemcpy(b->d_pv_tiles, pv.data(), sizeof(int4) * pv.size(), cudaMemcpyHostToDevice), "batch: tiles");
   BCK(cudaMemcpy(b->d_maps, maps.data(), sizeof(TileMaps) * maps.size(), cudaMemcpyHostToDevice), "batch: maps");
-  b->n_pv_tiles = (int)pv.size();
   b->pv_tiles_h = b->tile_h;
   b->maps_ok = true;
   return AF_OK;
@@ -265,7 +283,7 @@ int enqueue_batch_step(af_batch *b, double *hist, int hist_steps, cudaStream_t s
   if (pre) return pre;
   BCK(launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->tile_h, s), "batch: point values");
   if (b->sampling)
-    BCK(launch_sample_batch(b->sampler, b->d_pv_tiles, b->n_pv_tiles, b->tile_h, b->d_ctl, b->d_pv, s),
+    BCK(launch_sample_batch(b->sampler, b->d_pv_tiles, b->n_pv_tiles[0] + b->n_pv_tiles[1] + b->n_pv_tiles[2], b->tile_h, b->d_ctl, b->d_pv, s),
         "batch: sampler");
   FluxBatch F;
   F.tiles = b->d_fx_tiles;

@@ -76,6 +76,28 @@ __host__ __device__ __forceinline__ long long at(const Grid &g, int v, int i, in
   return (long long)v * g.plane + (long long)(j + OY) * g.P + (i + OX);
 }
 
+// Programmatic dependent launch: a kernel launched with launch_pdl may begin
+// while the one before it in the stream is still finishing.  pdl_start lets the
+// next kernel begin (its blocks take slots that the last ones of this kernel
+// leave free); pdl_wait holds a kernel until the one before it has ended and its
+// writes are visible, and stands before every access to global memory.
+__device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grd, dim3 blk, size_t smem, cudaStream_t s, const A &...args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grd;
+  c.blockDim = blk;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 // primitive -> conservative (Sec. 2: q = (rho, rho u, rho v, E))
 __device__ __forceinline__ void p2c(const float U[4], float gm1i, float Q[4]) {
   Q[0] = U[0];

@@ -49,12 +49,17 @@ struct af_ctx {
   TileMaps tmaps[2];
   NodeSet tbuf[2];
   int tmap_cur;
-  int tile_h;  // point-value tile height (4, 8, 16): rows of 32 cells
+  int tile_h;   // AF_OPT_TILE_H: point-value tile height (4, 8, 16) in rows of 32 cells
+  int tile_pv;  // the tile the kernel takes: tile_h, or TILE_SPLIT on a small grid while the option is not set
   // small device buffers
   void *small;
   int *d_status, *d_bad, *d_speed_bad;
   unsigned *d_speed;
+  // event counters of the last two steps: a step counts into slot tmap_cur and
+  // its flux kernel clears the other one for the next
   unsigned long long *d_counters;
+  unsigned *d_ticket;  // blocks done, of the kernels whose last block writes host words
+  bool ghost_valid;    // the ghost entries of the averages and of lev[0] belong to the current state
   double *d_partials, *d_totals;
   // host transfers: one staging area and one copy stream per external array
   // (lazily created), so that the four copies of a transfer run concurrently
@@ -83,7 +88,8 @@ struct af_ctx {
   cudaGraphExec_t run_exec[2];
   double run_dt[2];
   Options run_opt[2];
-  bool speed_valid;  // d_speed holds the max wave speed of the current state
+  bool speed_valid;    // d_speed holds the max wave speed of the current state
+  bool speed_on_host;  // and so do host_words[4], [5] once the stream is done
   cudaEvent_t ev_in, ev_out;
   // profiling: events around each stage of the last step, accumulated times
   int profile;

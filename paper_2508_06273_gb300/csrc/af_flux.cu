@@ -17,6 +17,7 @@
 // without the FP64 pipe, whose throughput on this GPU is a small fraction of
 // FP32.
 #include "af_common.cuh"
+#include "af_ghost.cuh"
 #include "af_kernels.h"
 
 namespace af {
@@ -258,11 +259,53 @@ __device__ __forceinline__ void ld_nf(const Args &A, int q, int i, int j, float 
   for (int v = 0; v < NV; v++) F[v] = __ldg(A.nf[q] + at(A.g, v, i, j));
 }
 
-// the tile of cells with origin (i0, j0); NF: the node fluxes come from the
-// point-value kernel (which also folded the new point values into the wave
-// speed), else they are formed here from the three time levels
-template <bool LIM, bool NF>
-__device__ __forceinline__ void flux_tile(const Args &A, FluxSmem &S, LimSmem *L, int i0, int j0) {
+// the new (hi, lo) averages of a cell next to a side into its ghost images, by
+// the thread that stored them (read back: keeping them for a rare path costs the
+// kernel the registers of a resident block)
+__device__ __noinline__ void store_images(const Args &A, int i, int j) {
+  const Grid &g = A.g;
+  float hi[4], lo[4];
+#pragma unroll
+  for (int v = 0; v < NV; v++) {
+    hi[v] = A.hi[at(g, v, i, j)];
+    lo[v] = A.lo[at(g, v, i, j)];
+  }
+  cell_images(g, i, j, [&](int a, int b, bool fx, bool fy) {
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      const bool neg = (v == 1 && fx) || (v == 2 && fy);
+      A.hi[at(g, v, a, b)] = neg ? -hi[v] : hi[v];
+      A.lo[at(g, v, a, b)] = neg ? -lo[v] : lo[v];
+    }
+  });
+}
+
+// the last tile's block to come here hands the finished wave-speed words to the host
+__device__ __noinline__ void finish_speed(const Args &A, unsigned ntiles) {
+  __threadfence();
+  if (atomicAdd(A.ticket, 1u) != ntiles - 1) return;
+  __threadfence();
+  volatile unsigned *h = A.host_speed;
+  h[0] = atomicMax(A.speed, 0u);
+  h[1] = (unsigned)atomicOr(A.speed_bad, 0);
+  *A.ticket = 0;
+  __threadfence_system();
+}
+
+// the tile of cells with origin (i0, j0), ntiles tiles in the launch; NF: the
+// node fluxes come from the point-value kernel (which also folded the new point
+// values into the wave speed), else they are formed here from the three time
+// levels.  (A warp a row, lane by lane, with the column right of the tile on a warp
+// of its own, so that every load is one aligned line, is slower than nodes dealt out
+// in order: 0.83 against 0.71 ms at 4096^2.)
+// TAIL: the small-grid form that also stores the averages' ghost images and hands
+// the wave speed to the host.  EARLY: the averages are loaded first, beside the
+// nodes, where registers allow it (with the limiter's 48 or a small grid's: 0.403
+// -> 0.385 ms at 2048^2 with the limiter; the plain kernel's 32 registers and six
+// blocks an SM do better without: 0.71 against 0.74 ms at 4096^2).
+template <bool LIM, bool NF, bool TAIL>
+__device__ __forceinline__ void flux_tile(const Args &A, FluxSmem &S, LimSmem *L, int i0, int j0, unsigned ntiles) {
+  constexpr bool EARLY = LIM || TAIL;
   const Grid &g = A.g;
   auto &vf = S.vf;
   auto &vg = S.vg;
@@ -274,6 +317,16 @@ __device__ __forceinline__ void flux_tile(const Args &A, FluxSmem &S, LimSmem *L
   const float gm1i = 1.0f / (g.gamma - 1.0f);
   float smax = 0.0f;
   bool sbad = false;
+  float h0[4], l0[4];
+  if (EARLY) {
+    const int i = i0 + threadIdx.x, j = j0 + threadIdx.y;
+    if (threadIdx.y < TY && i < g.nx && j < g.ny)
+#pragma unroll
+      for (int v = 0; v < NV; v++) {
+        h0[v] = A.hi[at(g, v, i, j)];
+        l0[v] = A.lo[at(g, v, i, j)];
+      }
+  }
 
   // time-integrated node fluxes; nodes up to index nx / ny (periodic
   // duplicates included)
@@ -339,18 +392,18 @@ __device__ __forceinline__ void flux_tile(const Args &A, FluxSmem &S, LimSmem *L
   bool bad = false;
   if (inside) {
 #pragma unroll
-  for (int v = 0; v < NV; v++) {
-    const long long e = at(g, v, i, j);
-    float xh, xl, yh, yl, dh, dl, nh, nl;
-    scaled_diff(Fx[v][b][a + 1], Fx[v][b][a], A.lxh, A.lxl, xh, xl);
-    scaled_diff(Gy[v][b + 1][a], Gy[v][b][a], A.lyh, A.lyl, yh, yl);
-    dw_add(xh, xl, yh, yl, dh, dl);
-    dw_add(A.hi[e], A.lo[e], -dh, -dl, nh, nl);
-    A.hi[e] = nh;
-    A.lo[e] = nl;
-    qh[v] = nh + nl;
-    bad |= !isfinite(nh);
-  }
+    for (int v = 0; v < NV; v++) {
+      const long long e = at(g, v, i, j);
+      float xh, xl, yh, yl, dh, dl, nh, nl;
+      scaled_diff(Fx[v][b][a + 1], Fx[v][b][a], A.lxh, A.lxl, xh, xl);
+      scaled_diff(Gy[v][b + 1][a], Gy[v][b][a], A.lyh, A.lyl, yh, yl);
+      dw_add(xh, xl, yh, yl, dh, dl);
+      dw_add(EARLY ? h0[v] : A.hi[e], EARLY ? l0[v] : A.lo[e], -dh, -dl, nh, nl);
+      A.hi[e] = nh;
+      A.lo[e] = nl;
+      qh[v] = nh + nl;
+      bad |= !isfinite(nh);
+    }
   }
   float U[4];
   c2p(qh, g.gamma - 1.0f, U);
@@ -378,35 +431,80 @@ __device__ __forceinline__ void flux_tile(const Args &A, FluxSmem &S, LimSmem *L
     }
     atomicMax(A.speed, __float_as_uint(m));
     if (b) atomicOr(A.speed_bad, 1);
+    if (TAIL) finish_speed(A, ntiles);
+  }
+  if (TAIL && inside && (i < G || j < G || i >= g.nx - G || j >= g.ny - G)) store_images(A, i, j);
+}
+
+// a block of a single grid's launch.  TAIL: a one-dimensional grid of tiles, then
+// blocks of 320 ghost entries of the new node arrays each (the point values are
+// final: they depend on nothing this kernel computes), so that no launch of its
+// own fills them before the next step.
+template <bool LIM, bool NF, bool TAIL>
+__device__ __forceinline__ void flux_block(const Args &A, FluxSmem &S, LimSmem *L) {
+  const Grid &g = A.g;
+  pdl_start();
+  pdl_wait();
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 4 && threadIdx.y == 0) A.clear_counters[threadIdx.x] = 0;
+  if (!TAIL) {
+    flux_tile<LIM, NF, false>(A, S, L, blockIdx.x * TX, blockIdx.y * TY, 0);
+    return;
+  }
+  const unsigned tx = (g.nx + TX - 1) / TX, ntiles = tx * ((g.ny + TY - 1) / TY), block = blockIdx.x;
+  if (block < ntiles) {
+    flux_tile<LIM, NF, true>(A, S, L, (int)(block % tx) * TX, (int)(block / tx) * TY, ntiles);
+    return;
+  }
+  int c = (int)(block - ntiles);
+#pragma unroll 1
+  for (int arr = 2; arr < 5; arr++) {
+    const GhostRange R(g, arr);
+    const int n = (R.total + NTHR - 1) / NTHR;
+    if (c < n) {
+      const int k = c * NTHR + threadIdx.y * TX + threadIdx.x;
+      if (k < R.total) ghost_entry<float, true>(g, R, A.ghost[arr - 2], arr, k);
+      return;
+    }
+    c -= n;
   }
 }
 
 // 320 threads for a 32 x 8-cell tile: each of the three node loops (297,
 // 264 and 288 nodes) takes one round of loads, where 256 threads needed a
 // second, serial round for some; the two extra warps skip the cell update.
-// 32 registers a thread: six resident blocks per SM keep the loads in flight.
-__global__ void __launch_bounds__(NTHR, 4) flux_update_kernel(Args A) {
+// NF: from the point-value kernel's node fluxes, 64 B of node data a cell read
+// instead of 144 B of point values at three time levels.  The plain kernel is
+// bound by HBM (208 B a cell, 73 % of the copy rate): 32 registers a thread, six
+// resident blocks an SM keep the loads in flight (asked for as launch bounds, the
+// six give another schedule: 0.754 against 0.709 ms at 4096^2).
+// (The arguments are grid constants so that calls can take their address
+// without a local copy.)
+template <bool LIM, bool NF, bool TAIL>
+__global__ void __launch_bounds__(NTHR, 4) flux_kernel(const __grid_constant__ Args A) {
   __shared__ FluxSmem S;
-  flux_tile<false, false>(A, S, nullptr, blockIdx.x * TX, blockIdx.y * TY);
-}
-// the same from the point-value kernel's node fluxes: 64 B of node data a cell
-// read instead of 144 B of point values at three time levels
-__global__ void __launch_bounds__(NTHR, 4) flux_nf_kernel(Args A) {
-  __shared__ FluxSmem S;
-  flux_tile<false, true>(A, S, nullptr, blockIdx.x * TX, blockIdx.y * TY);
+  if constexpr (LIM) {
+    __shared__ LimSmem L;
+    flux_block<LIM, NF, TAIL>(A, S, &L);
+  } else {
+    flux_block<LIM, NF, TAIL>(A, S, nullptr);
+  }
 }
 
-// (the arguments are grid constants so that the limiter's call can take
-// their address without a local copy)
-__global__ void __launch_bounds__(NTHR, 4) flux_limited_kernel(const __grid_constant__ Args A) {
-  __shared__ FluxSmem S;
-  __shared__ LimSmem L;
-  flux_tile<true, false>(A, S, &L, blockIdx.x * TX, blockIdx.y * TY);
-}
-__global__ void __launch_bounds__(NTHR, 4) flux_nf_limited_kernel(const __grid_constant__ Args A) {
-  __shared__ FluxSmem S;
-  __shared__ LimSmem L;
-  flux_tile<true, true>(A, S, &L, blockIdx.x * TX, blockIdx.y * TY);
+// Small grids take the TAIL form: it saves the ghost fill's launch and the
+// export of the wave speed (about 3 us each on an idle GPU) and costs its tiles
+// 14 % (a fence and an atomic a block, the registers of the rare image store:
+// 0.71 -> 0.83 ms at 4096^2), which meet near 3000 tiles.
+constexpr unsigned TAIL_TILES = 2432;
+template <bool NF>
+cudaError_t launch_flux(const Args &A, const StepTail &t, cudaStream_t s) {
+  const Grid &g = A.g;
+  const dim3 tiles((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY), blk(TX, TY + 2);
+  if (t.host_speed) {
+    unsigned n = tiles.x * tiles.y;
+    for (int arr = 2; arr < 5; arr++) n += (unsigned)((GhostRange(g, arr).total + NTHR - 1) / NTHR);
+    return launch_pdl(A.flux_limiter ? flux_kernel<true, NF, true> : flux_kernel<false, NF, true>, dim3(n), blk, 0, s, A);
+  }
+  return launch_pdl(A.flux_limiter ? flux_kernel<true, NF, false> : flux_kernel<false, NF, false>, tiles, blk, 0, s, A);
 }
 
 // batched form: tile B.tiles[b] = (instance, i0, j0); the instance's dt
@@ -425,7 +523,7 @@ __global__ void __launch_bounds__(NTHR, 6) flux_batch_kernel(FluxBatch B) {
     A.lyl = c.lyl;
   }
   __syncthreads();
-  flux_tile<false, false>(A, S, nullptr, t.y, t.z);
+  flux_tile<false, false, false>(A, S, nullptr, t.y, t.z, 0);
 }
 
 // instance blockIdx.y: its t^n averages (hi, all planes) into its snapshot
@@ -460,8 +558,8 @@ __global__ void __launch_bounds__(NTHR, 4) flux_batch_limited_kernel(FluxBatch B
     A.ly = c.lyh;
   }
   __syncthreads();
-  if (A.flux_limiter) flux_tile<true, false>(A, S, &L, t.y, t.z);
-  else flux_tile<false, false>(A, S, nullptr, t.y, t.z);
+  if (A.flux_limiter) flux_tile<true, false, false>(A, S, &L, t.y, t.z, 0);
+  else flux_tile<false, false, false>(A, S, nullptr, t.y, t.z, 0);
 }
 
 }  // namespace
@@ -484,13 +582,26 @@ FluxArgs flux_args(const Grid &g, const NodeSet &n0, const NodeSet &n1, const No
   A.status = status;
   A.speed = speed;
   A.speed_bad = speed_bad;
+  A.ghost[0] = A.ghost[1] = A.ghost[2] = nullptr;
+  A.clear_counters = nullptr;
+  A.host_speed = A.ticket = nullptr;
   return A;
+}
+
+static void set_tail(Args &A, const StepTail &t) {
+  for (int k = 0; k < 3; k++) A.ghost[k] = t.ghost.k[k];
+  A.clear_counters = t.clear_counters;
+  A.host_speed = t.host_speed;
+  A.ticket = t.ticket;
+}
+bool flux_fills_ghosts(const Grid &g) {
+  return (long long)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY) <= TAIL_TILES;
 }
 
 cudaError_t launch_flux_update(const Grid &g, const NodeSet &n0, const NodeSet &n1,
                                const NodeSet &n2, float *avg_hi, float *avg_lo, double lamx,
                                double lamy, int *status, unsigned *speed, int *speed_bad, int flux_limiter,
-                               const float *q0, cudaStream_t s) {
+                               const float *q0, const StepTail &tail, cudaStream_t s) {
   Args A = flux_args(g, n0, n1, n2, avg_hi, avg_lo, status, speed, speed_bad);
   split_double(lamx, A.lxh, A.lxl);
   split_double(lamy, A.lyh, A.lyl);
@@ -501,17 +612,13 @@ cudaError_t launch_flux_update(const Grid &g, const NodeSet &n0, const NodeSet &
     if (!q0 || q0 == avg_hi) return cudaErrorInvalidValue;
     A.q0 = q0;
   }
-  cudaMemsetAsync(speed, 0, sizeof(unsigned), s);
-  cudaMemsetAsync(speed_bad, 0, sizeof(int), s);
-  dim3 grd((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY), blk(TX, TY + 2);
-  if (flux_limiter) flux_limited_kernel<<<grd, blk, 0, s>>>(A);
-  else flux_update_kernel<<<grd, blk, 0, s>>>(A);
-  return cudaGetLastError();
+  set_tail(A, tail);
+  return launch_flux<false>(A, tail, s);
 }
 
 cudaError_t launch_flux_nf(const Grid &g, const float *const nf[4], float *avg_hi, float *avg_lo, double lamx,
                            double lamy, int *status, unsigned *speed, int *speed_bad, int flux_limiter,
-                           const float *q0, cudaStream_t s) {
+                           const float *q0, const StepTail &tail, cudaStream_t s) {
   NodeSet none = {{nullptr, nullptr, nullptr}};
   Args A = flux_args(g, none, none, none, avg_hi, avg_lo, status, speed, speed_bad);
   for (int q = 0; q < 4; q++) A.nf[q] = nf[q];
@@ -524,10 +631,8 @@ cudaError_t launch_flux_nf(const Grid &g, const float *const nf[4], float *avg_h
     if (!q0 || q0 == avg_hi) return cudaErrorInvalidValue;
     A.q0 = q0;
   }
-  dim3 grd((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY), blk(TX, TY + 2);
-  if (flux_limiter) flux_nf_limited_kernel<<<grd, blk, 0, s>>>(A);
-  else flux_nf_kernel<<<grd, blk, 0, s>>>(A);
-  return cudaGetLastError();
+  set_tail(A, tail);
+  return launch_flux<true>(A, tail, s);
 }
 
 cudaError_t launch_snapshot_batch(const FluxBatch &B, int n, cudaStream_t s) {

@@ -124,7 +124,7 @@ __device__ void build_record(const Grid &g, double gam, const double *avg, const
 }
 
 // ---- EG2 (eq. (EG2)) in FP64: the FP32 kernel's sums in truncated-power form
-// (af_pointvalue.cu, "EG2 arc sums in the truncated-power form"; the same
+// (af_pointvalue.cuh, "EG2 arc sums in the truncated-power form"; the same
 // symbols and recurrences), in double and reading the records through L1.
 // The kernel is bound by the FP64 pipe (2 multiply-adds a clock and SM), so what
 // counts is the number of FP64 operations: the tables come from recurrences on

@@ -76,6 +76,10 @@ struct PointValueArgs {
   unsigned *speed;
   int *speed_bad;
   int write_half;  // with nflux: also write the t^{n+1/2} level into n1
+  // without nflux: the first block clears these for the flux kernel that
+  // follows (NULL: not here)
+  unsigned *clear_speed;
+  int *clear_bad;
 };
 inline PointValueArgs pointvalue_args(const Grid &g, const NodeSet &n0, const float *avg_hi, const NodeSet &n1,
                                       const NodeSet &n2, const Options &o, int *status,
@@ -106,6 +110,8 @@ inline PointValueArgs pointvalue_args(const Grid &g, const NodeSet &n0, const fl
   A.speed = nullptr;
   A.speed_bad = nullptr;
   A.write_half = 1;
+  A.clear_speed = nullptr;
+  A.clear_bad = nullptr;
   return A;
 }
 
@@ -127,6 +133,23 @@ struct FluxArgs {
   int *status;
   unsigned *speed;  // max of max(|u|,|v|) + c over the new state, as float bits
   int *speed_bad;   // set if a new value is not admissible
+  // single grid only (NULL in a batch): what the next step and the host need,
+  // done here so that a small grid's step is two launches
+  float *ghost[3];                     // node arrays of the new state, whose ghost entries the blocks
+                                       // beyond the tiles fill; the averages' images are stored with them
+  unsigned long long *clear_counters;  // the next step's event counters
+  unsigned *host_speed;                // mapped host words: speed bits and the bad flag, by the last block
+  unsigned *ticket;                    // blocks done so far (returns to 0)
+};
+// whether the flux kernel of this grid takes the form that fills the new state's
+// ghosts and hands the wave speed to the host (host_speed and ticket are then
+// given, else NULL; clear_counters always)
+bool flux_fills_ghosts(const Grid &g);
+// what FluxArgs::ghost .. ticket are set to for a single grid
+struct StepTail {
+  NodeSet ghost;
+  unsigned long long *clear_counters;
+  unsigned *host_speed, *ticket;
 };
 FluxArgs flux_args(const Grid &g, const NodeSet &n0, const NodeSet &n1, const NodeSet &n2, float *avg_hi,
                    float *avg_lo, int *status, unsigned *speed, int *speed_bad);
@@ -176,13 +199,25 @@ struct GhostBatch {
 // ghost layers of the t^n state (cell averages hi/lo and the three node arrays)
 cudaError_t launch_ghost_fill(const Grid &g, float *avg_hi, float *avg_lo, const NodeSet &n,
                               cudaStream_t s);
-// tile_h: the point-value tile height the maps are for (4, 8 or 16)
+// Point-value tile of the single-grid kernel: 4, 8 or 16 rows of 32 cells, or
+// TILE_SPLIT: 4 rows with one block for each node kind
+constexpr int TILE_SPLIT = -4;
+// tile_h: the point-value tile the maps are for (4, 8, 16 or TILE_SPLIT)
 cudaError_t make_tile_maps(const Grid &g, float *vtx, float *xe, float *ye, float *avg, int tile_h,
                            TileMaps *out);
 // one-time kernel attributes (shared-memory size) on the current device
 cudaError_t prepare_pointvalue();
-// batched point values over a tile list of tile height tile_h (4, 8 or 16)
-cudaError_t launch_pointvalue_batch(const PointValueBatch &B, int ntiles, int tile_h, cudaStream_t s);
+// batched point values over a tile list of tile height tile_h (4, 8 or 16): the
+// tiles of the instances of class 0 first, ntiles[0] of them, then those of class 1
+// and 2 (batch_class of an instance's arguments: which instantiation of the
+// kernel its options need; a launch a class)
+constexpr int PV_CLASSES = 3;
+int batch_class(const PointValueArgs &A);
+// of the unit with the switches for discontinuous data (af_pointvalue_shock.cu)
+cudaError_t prepare_pointvalue_shock();
+cudaError_t launch_pointvalue_shock(const PointValueArgs &A, const TileMaps &maps, int tile_h, cudaStream_t s);
+void launch_pointvalue_shock_batch(const PointValueBatch &B, int ntiles, int tile_h, cudaStream_t s);
+cudaError_t launch_pointvalue_batch(const PointValueBatch &B, const int ntiles[PV_CLASSES], int tile_h, cudaStream_t s);
 // t^n snapshot (hi -> q0) of every active instance with the flux limiter on
 cudaError_t launch_snapshot_batch(const FluxBatch &B, int n, cudaStream_t s);
 // batched flux / update over a tile list of 32 x 8 cells: the first nplain
@@ -221,19 +256,21 @@ struct NodeFluxOut {
 cudaError_t launch_pointvalue(const Grid &g, const NodeSet &n0, const float *avg_hi, const TileMaps &maps,
                               const NodeSet &n1, const NodeSet &n2, float dt, const Options &o,
                               int *status, unsigned long long *counters, const float *const theta[2],
-                              int tile_h, const NodeFluxOut *nf, cudaStream_t s);
+                              int tile_h, const NodeFluxOut *nf, unsigned *clear_speed, int *clear_bad,
+                              cudaStream_t s);
 // Simpson fluxes and the finite-volume update of the averages (compensated
-// hi/lo); also the max wave speed of the new state into *speed (float bits)
+// hi/lo), the ghost entries of the new state; also the max wave speed of the new
+// state into *speed (float bits), which the point-value kernel cleared
 cudaError_t launch_flux_update(const Grid &g, const NodeSet &n0, const NodeSet &n1,
                                const NodeSet &n2, float *avg_hi, float *avg_lo, double lamx,
                                double lamy, int *status, unsigned *speed, int *speed_bad, int flux_limiter,
-                               const float *q0, cudaStream_t s);
+                               const float *q0, const StepTail &tail, cudaStream_t s);
 // the same from the node fluxes nf[4] that the point-value kernel wrote (see
 // PointValueArgs::nflux); folds only the new averages into *speed, which the
 // caller cleared before the point-value kernel
 cudaError_t launch_flux_nf(const Grid &g, const float *const nf[4], float *avg_hi, float *avg_lo, double lamx,
                            double lamy, int *status, unsigned *speed, int *speed_bad, int flux_limiter,
-                           const float *q0, cudaStream_t s);
+                           const float *q0, const StepTail &tail, cudaStream_t s);
 // max over averages and owned point values of max(|u|,|v|) + c (as float bits)
 // words a and b (b may be null) into mapped host memory dst, clearing a if
 // clear_a: small results reach the host without a copy engine, so that they
@@ -249,6 +286,22 @@ cudaError_t launch_max_speed(const Grid &g, const float *avg_hi, const NodeSet &
 constexpr int TOTALS_BLOCKS = 256;
 cudaError_t launch_totals(const Grid &g, const float *avg_hi, const float *avg_lo, double *partials,
                           double *out, cudaStream_t s);
+// a state's four external arrays (averages, vertices, x-edges, y-edges; device
+// memory) into the padded planes in one launch: ghost entries included, low
+// words and *status cleared, and the state's max wave speed into *speed /
+// *speed_bad (cleared by the caller) and, by the last block, host_speed[0..1]
+struct StateArrays {
+  const float *ext[4];  // external (NULL: skipped by store_state)
+  float *pad[4];        // averages hi, vertices, x-edges, y-edges
+};
+cudaError_t launch_load_state(const Grid &g, const StateArrays &a, float *avg_lo, int *status, unsigned *speed,
+                              int *speed_bad, unsigned *host_speed, unsigned *ticket, cudaStream_t s);
+// padded planes into the external arrays that are given, in one launch
+cudaError_t launch_store_state(const Grid &g, const float *const pad[4], float *const ext[4], cudaStream_t s);
+// whether the periodic duplicate lines of the external arrays differ: *bad set
+// (mapped host memory); also clears *speed and *speed_bad for launch_load_state
+cudaError_t launch_check_state(const Grid &g, const float *const ext[4], unsigned *bad, unsigned *speed,
+                               int *speed_bad, cudaStream_t s);
 // external compact arrays <-> padded planes
 cudaError_t launch_pack(const Grid &g, const float *src, float *dst, int ni, int nj, bool to_padded,
                         cudaStream_t s);
@@ -338,7 +391,7 @@ cudaError_t launch_pointvalue_masked(const Grid &g, const NodeSet &n0, const flo
                                      const NodeSet &n1, const NodeSet &n2, float dt, const Options &o, int *status,
                                      unsigned long long *counters, const unsigned char *const mask[3],
                                      const int *tile_flag, const float *const theta[2], int tile_h,
-                                     cudaStream_t s);
+                                     unsigned *clear_speed, int *clear_bad, cudaStream_t s);
 
 // record a message for af_last_error on this host thread; returns code
 int set_error(int code, const char *msg);
@@ -349,6 +402,7 @@ unsigned bounds_flux();
 unsigned bounds_fp64();
 unsigned bounds_misc();
 unsigned bounds_pointvalue();
+unsigned bounds_pointvalue_shock();
 unsigned bounds_surrogate();
 
 }  // namespace af

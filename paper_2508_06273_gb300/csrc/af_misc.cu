@@ -1,104 +1,17 @@
 // af_misc.cu -- ghost cells (Sec. 4.3), reductions and layout conversion
 // kernels.
-#include <type_traits>
-
 #include "af_common.cuh"
+#include "af_ghost.cuh"
 #include "af_kernels.h"
 
 namespace af {
 
 namespace {
 
-// Source index of a ghost entry along one axis.  Periodic: wrap.  Outflow:
-// mirror copy of the interior.  Solid wall: the same mirror, with the normal
-// velocity negated (flip).  node: the array sits on grid lines along the axis.
-__device__ __forceinline__ int ghost_src(int i, int n, int own, int node, int per, int blo,
-                                         int bhi, bool &flip) {
-  if (i >= 0 && i < own) return i;
-  if (per) {
-    int r = i % n;
-    return r < 0 ? r + n : r;
-  }
-  if (i < 0) {
-    flip = (blo == BC_REFLECTING);
-    return node ? -i : -1 - i;
-  }
-  flip = (bhi == BC_REFLECTING);
-  return node ? 2 * n - i : 2 * n - 1 - i;
-}
-
 struct GhostArgs {
   Grid g;
   float *a[5];  // avg_hi, avg_lo, vtx, xe, ye
 };
-
-// entries of array arr (0..4) in ghost order; total is their number
-struct GhostRange {
-  int nodex, nodey, ownx, owny, hix, hiy, wext, nb, nt, nl, wr, total;
-  __host__ __device__ GhostRange(const Grid &g, int arr) {
-    nodex = (arr == 2 || arr == 3);
-    nodey = (arr == 2 || arr == 4);
-    ownx = nodex ? g.nxv : g.nx;
-    owny = nodey ? g.nyv : g.ny;
-    hix = nodex ? g.nx + G + 1 : g.nx + G;
-    hiy = nodey ? g.ny + G + 1 : g.ny + G;
-    wext = hix + G;
-    nb = G * wext;
-    nt = (hiy - owny) * wext;
-    nl = owny * G;
-    wr = hix - ownx;
-    total = nb + nt + nl + owny * wr;
-  }
-};
-
-// ghost entry k of array arr (0 averages hi, 1 averages lo, 2..4 node
-// arrays): copy from its source, flipping the normal velocity at walls; on
-// an inflow side the side's state (conservative for the averages, zero low
-// word).  A corner entry takes the y side's rule applied to the x side's
-// value, as two passes (x, then y) would give.
-template <typename T>
-__device__ __forceinline__ void ghost_entry(const Grid &g, const GhostRange &R, T *p, int arr, int k) {
-  int i, j, r = k;
-  if (r < R.nb) {
-    j = -G + r / R.wext;
-    i = -G + r % R.wext;
-  } else if ((r -= R.nb) < R.nt) {
-    j = R.owny + r / R.wext;
-    i = -G + r % R.wext;
-  } else if ((r -= R.nt) < R.nl) {
-    j = r / G;
-    i = -G + r % G;
-  } else {
-    r -= R.nl;
-    j = r / R.wr;
-    i = R.ownx + r % R.wr;
-  }
-  bool fx = false, fy = false;
-  const int si = ghost_src(i, g.nx, R.ownx, R.nodex, g.per_x, g.bc[0], g.bc[1], fx);
-  const int sj = ghost_src(j, g.ny, R.owny, R.nodey, g.per_y, g.bc[2], g.bc[3], fy);
-  const int xside = i < 0 ? 0 : (i >= R.ownx ? 1 : -1), yside = j < 0 ? 2 : (j >= R.owny ? 3 : -1);
-  const bool xin = !g.per_x && xside >= 0 && g.bc[xside] == BC_INFLOW;
-  const bool yin = !g.per_y && yside >= 0 && g.bc[yside] == BC_INFLOW;
-  if constexpr (std::is_same<T, float>::value) {  // (the FP64 path has no inflow sides)
-  if (xin || yin) {
-    float U[4];
-#pragma unroll
-    for (int v = 0; v < NV; v++) U[v] = g.inflow[yin ? yside : xside][v];
-    if (!yin && fy) U[2] = -U[2];
-    float Q[4];
-    if (arr == 0) p2c(U, 1.0f / (g.gamma - 1.0f), Q);
-#pragma unroll
-    for (int v = 0; v < NV; v++) p[at(g, v, i, j)] = arr == 0 ? Q[v] : (arr == 1 ? 0.0f : U[v]);
-    return;
-  }
-  }
-#pragma unroll
-  for (int v = 0; v < NV; v++) {
-    T x = p[at(g, v, si, sj)];
-    if ((v == 1 && fx) || (v == 2 && fy)) x = -x;
-    p[at(g, v, i, j)] = x;
-  }
-}
 
 __global__ void ghost_kernel(GhostArgs A) {
   const int arr = blockIdx.y;
@@ -400,6 +313,162 @@ __global__ void pack_kernel(Grid g, const float *__restrict__ src, float *dst, i
   }
 }
 
+// ---- whole states: 32 x 32 points of one of the four arrays a block (blocks
+// [first[w], first[w + 1]) take array w), 4 rows and all variables a thread, so
+// that 16 loads are in flight; one launch moves a state where packing array by
+// array, clearing the low words, the ghost fill and the wave speed were nine.
+constexpr int ST_W = 32, ST_H = 32, ST_ROWS = 4;
+struct StateTiles {
+  unsigned first[5];
+  int tx[4];
+};
+__device__ __forceinline__ void state_tile(const StateTiles &T, int &w, int &i0, int &j0) {
+  unsigned b = blockIdx.x;
+  w = b < T.first[1] ? 0 : (b < T.first[2] ? 1 : (b < T.first[3] ? 2 : 3));
+  b -= T.first[w];
+  i0 = (int)(b % T.tx[w]) * ST_W;
+  j0 = (int)(b / T.tx[w]) * ST_H;
+}
+
+struct LoadArgs {
+  Grid g;
+  StateTiles T;
+  const float *ext[4];
+  float *pad[4], *lo;
+  int *status, *speed_bad;
+  unsigned *speed, *host_speed, *ticket;
+};
+__global__ void __launch_bounds__(ST_W *ST_H / ST_ROWS) load_state_kernel(const __grid_constant__ LoadArgs A) {
+  const Grid &g = A.g;
+  int w, i0, j0;
+  state_tile(A.T, w, i0, j0);
+  const int arr = w == 0 ? 0 : w + 1;  // as in GhostRange (1: the low words)
+  const GhostRange R(g, arr);
+  const int ni = g.nx + R.nodex, nj = g.ny + R.nodey;
+  const int i = i0 - G + (int)threadIdx.x;
+  float smax = 0.0f;
+  bool bad = false;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *A.status = 0;
+  float x[ST_ROWS][4];
+#pragma unroll
+  for (int r = 0; r < ST_ROWS; r++) {
+    const int j = j0 - G + (int)threadIdx.y + r * (ST_H / ST_ROWS);
+    bool fx = false, fy = false;
+    // (threads beyond the padded extents read an interior point and store nothing)
+    const int si = i < R.hix ? ghost_src(i, g.nx, R.ownx, R.nodex, g.per_x, g.bc[0], g.bc[1], fx) : 0;
+    const int sj = j < R.hiy ? ghost_src(j, g.ny, R.owny, R.nodey, g.per_y, g.bc[2], g.bc[3], fy) : 0;
+    const float *src = A.ext[w] + (long long)sj * ni + si;
+#pragma unroll
+    for (int v = 0; v < NV; v++) x[r][v] = __ldg(src + (long long)v * ni * nj);
+    const int xside = i < 0 ? 0 : (i >= R.ownx ? 1 : -1), yside = j < 0 ? 2 : (j >= R.owny ? 3 : -1);
+    const bool xin = !g.per_x && xside >= 0 && g.bc[xside] == BC_INFLOW;
+    const bool yin = !g.per_y && yside >= 0 && g.bc[yside] == BC_INFLOW;
+    if (xin || yin) {
+      float U[4];
+#pragma unroll
+      for (int v = 0; v < NV; v++) U[v] = g.inflow[yin ? yside : xside][v];
+      if (!yin && fy) U[2] = -U[2];
+      if (arr == 0) p2c(U, 1.0f / (g.gamma - 1.0f), x[r]);
+      else
+#pragma unroll
+        for (int v = 0; v < NV; v++) x[r][v] = U[v];
+    } else {
+      if (fx) x[r][1] = -x[r][1];
+      if (fy) x[r][2] = -x[r][2];
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < ST_ROWS; r++) {
+    const int j = j0 - G + (int)threadIdx.y + r * (ST_H / ST_ROWS);
+    if (i >= R.hix || j >= R.hiy) continue;
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      const long long e = at(g, v, i, j);
+      A.pad[w][e] = x[r][v];
+      if (arr == 0) A.lo[e] = 0.0f;
+    }
+    if (i >= 0 && j >= 0 && i < R.ownx && j < R.owny) {
+      float U[4];
+      if (arr == 0) c2p(x[r], g.gamma - 1.0f, U);
+      smax = fmaxf(smax, wave_speed(arr == 0 ? U : x[r], g.gamma, bad));
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+  __shared__ float wmax[ST_H / ST_ROWS];
+  const int anybad = __syncthreads_or(bad);
+  if (threadIdx.x == 0) wmax[threadIdx.y] = smax;
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    for (int k = 1; k < ST_H / ST_ROWS; k++) smax = fmaxf(smax, wmax[k]);
+    atomicMax(A.speed, __float_as_uint(smax));
+    if (anybad) atomicOr(A.speed_bad, 1);
+    __threadfence();
+    if (atomicAdd(A.ticket, 1u) == gridDim.x - 1) {
+      __threadfence();
+      volatile unsigned *h = A.host_speed;
+      h[0] = atomicMax(A.speed, 0u);
+      h[1] = (unsigned)atomicOr(A.speed_bad, 0);
+      *A.ticket = 0;
+      __threadfence_system();
+    }
+  }
+}
+
+struct StoreArgs {
+  Grid g;
+  StateTiles T;
+  const float *pad[4];
+  float *ext[4];
+};
+__global__ void __launch_bounds__(ST_W *ST_H / ST_ROWS) store_state_kernel(const __grid_constant__ StoreArgs A) {
+  const Grid &g = A.g;
+  int w, i0, j0;
+  state_tile(A.T, w, i0, j0);
+  const int ni = g.nx + (w == 1 || w == 2), nj = g.ny + (w == 1 || w == 3);
+  const int i = i0 + (int)threadIdx.x;
+  if (i >= ni) return;
+  float x[ST_ROWS][4];
+#pragma unroll
+  for (int r = 0; r < ST_ROWS; r++) {
+    const int j = min(j0 + (int)threadIdx.y + r * (ST_H / ST_ROWS), nj - 1);
+#pragma unroll
+    for (int v = 0; v < NV; v++) x[r][v] = __ldg(A.pad[w] + at(g, v, i, j));
+  }
+#pragma unroll
+  for (int r = 0; r < ST_ROWS; r++) {
+    const int j = j0 + (int)threadIdx.y + r * (ST_H / ST_ROWS);
+    if (j >= nj) continue;
+#pragma unroll
+    for (int v = 0; v < NV; v++) A.ext[w][((long long)v * nj + j) * ni + i] = x[r][v];
+  }
+}
+
+// periodic duplicate lines of the three node arrays (blockIdx.z; y: variable)
+struct CheckArgs {
+  Grid g;
+  const float *ext[4];
+  unsigned *bad, *speed;
+  int *speed_bad;
+};
+__global__ void check_state_kernel(const __grid_constant__ CheckArgs A) {
+  const Grid &g = A.g;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y, w = 1 + blockIdx.z;
+  if (k == 0 && v == 0 && w == 1) {
+    *A.speed = 0u;
+    *A.speed_bad = 0;
+  }
+  const int nodex = w == 1 || w == 2, nodey = w == 1 || w == 3, ni = g.nx + nodex, nj = g.ny + nodey;
+  const float *p = A.ext[w] + (long long)v * ni * nj;
+  bool bad = false;
+  if (g.per_x && nodex && k < nj) bad |= !(p[(long long)k * ni + ni - 1] == p[(long long)k * ni]);
+  if (g.per_y && nodey && k < ni) bad |= !(p[(long long)(nj - 1) * ni + k] == p[k]);
+  if (bad) {
+    *(volatile unsigned *)A.bad = 1u;
+    __threadfence_system();
+  }
+}
+
 __global__ void check_dup_kernel(const float *__restrict__ a, int ni, int nj, int dup_x, int dup_y,
                                  int *bad) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -495,6 +564,70 @@ cudaError_t launch_totals(const Grid &g, const float *avg_hi, const float *avg_l
                           double *out, cudaStream_t s) {
   totals_stage1<<<TOTALS_BLOCKS, 256, 0, s>>>(g, avg_hi, avg_lo, partials);
   totals_stage2<<<1, TOTALS_BLOCKS, 0, s>>>(partials, out);
+  return cudaGetLastError();
+}
+
+// tiles of the four arrays of extents ni x nj (0: left out)
+static StateTiles state_tiles(const int ni[4], const int nj[4]) {
+  StateTiles T;
+  T.first[0] = 0;
+  for (int w = 0; w < 4; w++) {
+    T.tx[w] = ni[w] > 0 ? (ni[w] + ST_W - 1) / ST_W : 1;
+    T.first[w + 1] = T.first[w] + (ni[w] > 0 ? (unsigned)T.tx[w] * ((nj[w] + ST_H - 1) / ST_H) : 0u);
+  }
+  return T;
+}
+
+cudaError_t launch_check_state(const Grid &g, const float *const ext[4], unsigned *bad, unsigned *speed, int *speed_bad,
+                               cudaStream_t s) {
+  CheckArgs A;
+  A.g = g;
+  for (int w = 0; w < 4; w++) A.ext[w] = ext[w];
+  A.bad = bad;
+  A.speed = speed;
+  A.speed_bad = speed_bad;
+  const int n = (g.nx > g.ny ? g.nx : g.ny) + 1;
+  check_state_kernel<<<dim3((n + 255) / 256, NV, 3), 256, 0, s>>>(A);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_load_state(const Grid &g, const StateArrays &a, float *avg_lo, int *status, unsigned *speed,
+                              int *speed_bad, unsigned *host_speed, unsigned *ticket, cudaStream_t s) {
+  LoadArgs A;
+  A.g = g;
+  int ni[4], nj[4];
+  for (int w = 0; w < 4; w++) {
+    const GhostRange R(g, w == 0 ? 0 : w + 1);
+    ni[w] = R.hix + G;
+    nj[w] = R.hiy + G;
+    A.ext[w] = a.ext[w];
+    A.pad[w] = a.pad[w];
+  }
+  A.T = state_tiles(ni, nj);
+  A.lo = avg_lo;
+  A.status = status;
+  A.speed = speed;
+  A.speed_bad = speed_bad;
+  A.host_speed = host_speed;
+  A.ticket = ticket;
+  load_state_kernel<<<A.T.first[4], dim3(ST_W, ST_H / ST_ROWS), 0, s>>>(A);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_store_state(const Grid &g, const float *const pad[4], float *const ext[4], cudaStream_t s) {
+  StoreArgs A;
+  A.g = g;
+  int ni[4], nj[4];
+  for (int w = 0; w < 4; w++) {
+    const bool on = ext[w] && pad[w];
+    ni[w] = on ? g.nx + (w == 1 || w == 2) : 0;
+    nj[w] = on ? g.ny + (w == 1 || w == 3) : 0;
+    A.pad[w] = pad[w];
+    A.ext[w] = ext[w];
+  }
+  A.T = state_tiles(ni, nj);
+  if (A.T.first[4] == 0) return cudaSuccess;
+  store_state_kernel<<<A.T.first[4], dim3(ST_W, ST_H / ST_ROWS), 0, s>>>(A);
   return cudaGetLastError();
 }
 
