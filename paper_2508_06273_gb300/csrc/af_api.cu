@@ -102,6 +102,17 @@ int ensure_staging(af_ctx *h) {
 // [4], [5] the wave speed's bits and bad flag; [6] a differing periodic duplicate
 enum { HW_SPEED = 4, HW_BAD = 6 };
 
+cudaError_t make_maps(af_ctx *h) {
+  cudaError_t e = cudaSuccess;
+  for (int b = 0; b < 2 && e == cudaSuccess; b++) {
+    const NodeSet &n = h->tbuf[b];
+    e = make_tile_maps(h->g, n.k[VTX], n.k[XE], n.k[YE], h->hi, h->tile_pv, &h->tmaps[b]);
+    if (e == cudaSuccess)
+      e = make_tile_maps(h->g, n.k[VTX], n.k[XE], n.k[YE], h->hi, h->tile_tall, &h->tmaps_tall[b]);
+  }
+  return e;
+}
+
 void drop_runs(af_ctx *h) {
   for (int p = 0; p < 2; p++)
     if (h->run_exec[p]) {
@@ -223,23 +234,21 @@ af_ctx *af_create(int nx, int ny, double dx, double dy, double gamma, uint32_t b
     }
   }
   h->tile_h = 8;
-  // A small grid leaves SMs idle: its tiles are 4 rows high with one block a
-  // node kind, so that a step's critical path is the vertex's update instead of
-  // three nodes'.  Up to two blocks an SM (8 rows, split, us a step: 32^2
-  // 18.9, 14.4; 96^2 18.9, 15.4; 256^2, beyond the line, 25.9, 27.8).
+  // A small grid leaves SMs idle: its tiles have one block a node kind, so that a
+  // step's critical path is the vertex's update instead of three nodes'.  Up to
+  // three blocks an SM (us a step, 4 rows / split: 32^2 16.9 / 14.4, 128^2 17.3 /
+  // 16.7; beyond the line 144^2 17.9 / 18.6, 256^2 25.3 / 27.8).
   const long long tiles4 = (long long)((g.nxv + 31) / 32) * ((g.nyv + 3) / 4);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-  h->tile_pv = tiles4 * 3 <= 2LL * sms ? TILE_SPLIT : 8;
-  for (int b = 0; b < 2; b++) {
-    cudaError_t te = make_tile_maps(g, h->tbuf[b].k[VTX], h->tbuf[b].k[XE], h->tbuf[b].k[YE], h->hi, h->tile_pv,
-                                   &h->tmaps[b]);
-    if (te != cudaSuccess) {
-      cuda_fail(te, "af_create: TMA descriptors");
-      cudaFree(h->base);
-      delete h;
-      return nullptr;
-    }
+  h->tile_pv = tiles4 * 3 <= 3LL * sms ? TILE_SPLIT : TILE_PLAIN;
+  h->tile_tall = TILE_TALL;
+  const cudaError_t te = make_maps(h);
+  if (te != cudaSuccess) {
+    cuda_fail(te, "af_create: TMA descriptors");
+    cudaFree(h->base);
+    delete h;
+    return nullptr;
   }
   const size_t small = 64 + 64 + 64 + 64 + sizeof(double) * (TOTALS_BLOCKS * NV + NV);
   e = cudaHostAlloc(&h->host_words, 64, cudaHostAllocMapped);
@@ -425,13 +434,11 @@ int af_set_option(af_ctx *h, int key, double value) {
       return AF_OK;
     case AF_OPT_TILE_H: {
       if (iv != 4 && iv != 8 && iv != 16) return fail(AF_ERR_ARG, "tile height must be 4, 8 or 16%s");
-      if (iv == h->tile_pv) return AF_OK;
+      if (iv == h->tile_h && iv == h->tile_pv && iv == h->tile_tall) return AF_OK;
       DeviceGuard dg(h->device);
       CK(cudaStreamSynchronize(h->stream), "sync");
-      for (int b = 0; b < 2; b++)
-        CK(make_tile_maps(h->g, h->tbuf[b].k[VTX], h->tbuf[b].k[XE], h->tbuf[b].k[YE], h->hi, iv, &h->tmaps[b]),
-           "TMA descriptors");
-      h->tile_h = h->tile_pv = iv;
+      h->tile_h = h->tile_pv = h->tile_tall = iv;
+      CK(make_maps(h), "TMA descriptors");
       for (int p = 0; p < 2; p++)  // captured steps hold the old launch shape
         if (h->run_exec[p]) {
           cudaGraphExecDestroy(h->run_exec[p]);
@@ -823,12 +830,15 @@ static int enqueue_step(af_ctx *h, double dt) {
        "shock indicator");
   }
   if (prof) cudaEventRecord(h->ev_stage[1], s);
+  const bool tall = shock_options(h->opt) || (h->opt.node_flux && !h->opt.surrogate);
+  const int tile_pv = tall ? h->tile_tall : h->tile_pv;
+  const TileMaps &maps = (tall ? h->tmaps_tall : h->tmaps)[h->tmap_cur];
   {
     NvtxScope pvr("point values");
     if (h->opt.surrogate) {
       // network at every node, then the exact operator at the nodes it rejected
       // (all three kinds of a flagged tile in one block)
-      const int tile = h->tile_pv == TILE_SPLIT ? 4 : h->tile_pv, tile_rows = tile;
+      const int tile = tile_pv == TILE_SPLIT ? 4 : tile_pv, tile_rows = tile;
       CK(cudaMemsetAsync(h->surr_tiles, 0, sizeof(int) * h->surr_tiles_x * ((h->g.nyv + tile_rows - 1) / tile_rows), s),
          "memset tiles");
       CK(launch_ubar(h->g, h->hi, h->lev[0], h->surr_ubar, s), "surrogate cell prep");
@@ -861,7 +871,7 @@ static int enqueue_step(af_ctx *h, double dt) {
         A.wait_limit = h->opt.test_timeout ? kTestWaitLimit : kWaitLimit;
         CK(launch_surrogate(k, A, h->sms, s), "surrogate");
       }
-      CK(launch_pointvalue_masked(h->g, h->lev[0], h->hi, h->tmaps[h->tmap_cur], h->lev[1], h->lev[2], (float)dt,
+      CK(launch_pointvalue_masked(h->g, h->lev[0], h->hi, maps, h->lev[1], h->lev[2], (float)dt,
                                   h->opt, h->d_status, counters, mask, h->surr_tiles, theta, tile, h->d_speed,
                                   h->d_speed_bad, s),
          "point values (fallback)");
@@ -870,8 +880,8 @@ static int enqueue_step(af_ctx *h, double dt) {
     } else if (!h->opt.node_flux) {
       // plain path: t^{n+1/2} and t^{n+1} written, the flux kernel forms the
       // node fluxes from three levels
-      CK(launch_pointvalue(h->g, h->lev[0], h->hi, h->tmaps[h->tmap_cur], h->lev[1], h->lev[2], (float)dt,
-                           h->opt, h->d_status, counters, theta, h->tile_pv, nullptr, h->d_speed, h->d_speed_bad, s),
+      CK(launch_pointvalue(h->g, h->lev[0], h->hi, maps, h->lev[1], h->lev[2], (float)dt,
+                           h->opt, h->d_status, counters, theta, tile_pv, nullptr, h->d_speed, h->d_speed_bad, s),
          "point values");
       h->launches[AF_STAGE_POINTVALUE] += 1;
       h->half_valid = true;
@@ -885,8 +895,8 @@ static int enqueue_step(af_ctx *h, double dt) {
       nf.write_half = h->keep_half;
       CK(cudaMemsetAsync(h->d_speed, 0, sizeof(unsigned), s), "memset speed");
       CK(cudaMemsetAsync(h->d_speed_bad, 0, sizeof(int), s), "memset speed");
-      CK(launch_pointvalue(h->g, h->lev[0], h->hi, h->tmaps[h->tmap_cur], h->lev[1], h->lev[2], (float)dt,
-                           h->opt, h->d_status, counters, theta, h->tile_pv, &nf, nullptr, nullptr, s),
+      CK(launch_pointvalue(h->g, h->lev[0], h->hi, maps, h->lev[1], h->lev[2], (float)dt,
+                           h->opt, h->d_status, counters, theta, tile_pv, &nf, nullptr, nullptr, s),
          "point values");
       h->launches[AF_STAGE_POINTVALUE] += 1;
       h->half_valid = h->keep_half != 0;

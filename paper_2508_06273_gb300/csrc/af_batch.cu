@@ -41,7 +41,7 @@ struct af_batch {
   int device = 0;
   cudaStream_t own_stream = nullptr, stream = nullptr;
   std::vector<af_ctx *> inst;
-  int tile_h = 8;
+  int tile_h = 0;  // tile height of every class, or 0: each class its own (TILE_OF_CLASS)
   std::vector<BatchCtl> ctl_h;  // host mirror, current after sync_ctl
   std::vector<char> has_state, speed_ok, stopped;
   BatchCtl *d_ctl = nullptr;
@@ -54,7 +54,7 @@ struct af_batch {
   // point-value tiles by class of their instance (the kernel instantiation its
   // options need; class of instance k in cls[k])
   std::vector<int> cls;
-  int n_pv_tiles[PV_CLASSES] = {};
+  int n_pv_tiles[PV_CLASSES] = {}, heights[PV_CLASSES] = {};
   int n_fx_tiles = 0, pv_tiles_h = 0;
   int n_fx_plain = -1;  // flux tiles of instances without the flux limiter (listed first)
   int4 *d_ghost_chunks = nullptr;  // (instance, array, first entry) per ghost-fill block
@@ -216,18 +216,20 @@ int upload_args(af_batch *b) {
   return AF_OK;
 }
 
-// TMA descriptors and the point-value tile list for tile height b->tile_h
+// TMA descriptors and the point-value tile list for the classes' tile heights
 int build_tiles(af_batch *b) {
   if (b->maps_ok && b->pv_tiles_h == b->tile_h) return AF_OK;
   drop_graphs(b);
+  const int *hs = b->heights;
+  for (int c = 0; c < PV_CLASSES; c++) b->heights[c] = b->tile_h ? b->tile_h : TILE_OF_CLASS[c];
   std::vector<TileMaps> maps(2 * b->n);
   std::vector<int4> pv;
   for (int k = 0; k < b->n; k++) {
     af_ctx *h = b->inst[k];
     const Grid &g = h->g;
     for (int q = 0; q < 2; q++) {
-      cudaError_t e = make_tile_maps(g, h->tbuf[q].k[VTX], h->tbuf[q].k[XE], h->tbuf[q].k[YE], h->hi, b->tile_h,
-                                     &maps[2 * k + q]);
+      cudaError_t e = make_tile_maps(g, h->tbuf[q].k[VTX], h->tbuf[q].k[XE], h->tbuf[q].k[YE], h->hi,
+                                     hs[b->cls[k]], &maps[2 * k + q]);
       if (e != cudaSuccess) return bcuda(e, "batch: TMA descriptors");
     }
   }
@@ -236,7 +238,7 @@ int build_tiles(af_batch *b) {
     for (int k = 0; k < b->n; k++) {
       const Grid &g = b->inst[k]->g;
       if (b->cls[k] != c) continue;
-      for (int j0 = 0; j0 < g.nyv; j0 += b->tile_h)
+      for (int j0 = 0; j0 < g.nyv; j0 += hs[c])
         for (int i0 = 0; i0 < g.nxv; i0 += 32) pv.push_back(make_int4(k, i0, j0, 0));
     }
     b->n_pv_tiles[c] = (int)(pv.size() - before);
@@ -281,10 +283,12 @@ int enqueue_batch_step(af_batch *b, double *hist, int hist_steps, cudaStream_t s
   BCK(launch_batch_dt(b->d_ctl, b->n, hist, hist_steps, DT_STEP, b->d_pv, s), "batch: dt");
   const int pre = enqueue_pre_pointvalue(b, s);
   if (pre) return pre;
-  BCK(launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->tile_h, s), "batch: point values");
-  if (b->sampling)
-    BCK(launch_sample_batch(b->sampler, b->d_pv_tiles, b->n_pv_tiles[0] + b->n_pv_tiles[1] + b->n_pv_tiles[2], b->tile_h, b->d_ctl, b->d_pv, s),
-        "batch: sampler");
+  BCK(launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->heights, s), "batch: point values");
+  const int4 *tiles = b->d_pv_tiles;
+  for (int c = 0; b->sampling && c < PV_CLASSES; tiles += b->n_pv_tiles[c++])
+    if (b->n_pv_tiles[c] > 0)
+      BCK(launch_sample_batch(b->sampler, tiles, b->n_pv_tiles[c], b->heights[c], b->d_ctl, b->d_pv, s),
+          "batch: sampler");
   FluxBatch F;
   F.tiles = b->d_fx_tiles;
   F.ctl = b->d_ctl;
@@ -619,10 +623,10 @@ int af_batch_autotune(af_batch *b, int *tile_h, double *ms) {
     if (rc) break;
     // dt of the coming step, nothing advanced
     cudaError_t e = launch_batch_dt(b->d_ctl, b->n, nullptr, 0, DT_PROBE, b->d_pv, b->stream);
-    if (e == cudaSuccess) e = launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->tile_h, b->stream);
+    if (e == cudaSuccess) e = launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->heights, b->stream);
     if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
     for (int r = 0; r < 3 && e == cudaSuccess; r++)
-      e = launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->tile_h, b->stream);
+      e = launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->heights, b->stream);
     if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float t = 0.0f;

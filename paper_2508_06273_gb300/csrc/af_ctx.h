@@ -46,11 +46,13 @@ struct af_ctx {
   bool half_valid;  // lev[1] holds the t^{n+1/2} level of the last step
   // TMA descriptors for t^n held in either of the two buffers that swap
   // roles each step; tmap_cur selects the one now holding t^n
-  TileMaps tmaps[2];
+  TileMaps tmaps[2], tmaps_tall[2];
   NodeSet tbuf[2];
   int tmap_cur;
   int tile_h;   // AF_OPT_TILE_H: point-value tile height (4, 8, 16) in rows of 32 cells
-  int tile_pv;  // the tile the kernel takes: tile_h, or TILE_SPLIT on a small grid while the option is not set
+  // the tiles that tmaps and tmaps_tall are for (TILE_PLAIN or TILE_SPLIT; TILE_TALL): tile_h
+  // once the option is set
+  int tile_pv, tile_tall;
   // small device buffers
   void *small;
   int *d_status, *d_bad, *d_speed_bad;

@@ -202,22 +202,33 @@ cudaError_t launch_ghost_fill(const Grid &g, float *avg_hi, float *avg_lo, const
 // Point-value tile of the single-grid kernel: 4, 8 or 16 rows of 32 cells, or
 // TILE_SPLIT: 4 rows with one block for each node kind
 constexpr int TILE_SPLIT = -4;
+// Tile heights while none is chosen.  The plain kernels are a little faster on 4
+// rows (more, smaller blocks an SM wait less for one another at their barriers),
+// those for discontinuous data and node fluxes, with more work or scratch a tile,
+// on 8; us a step, 4 / 8 rows: vortex 256^2 25.1 / 25.8, 600^2 77.2 / 79.6, 2048^2
+// 770 / 791; Riemann data with every switch 256^2 62.8 / 51.1, 600^2 199 / 177,
+// 2048^2 1888 / 1692; point values with node fluxes 4096^2 2817 / 2777.
+constexpr int TILE_PLAIN = 4, TILE_TALL = 8;
 // tile_h: the point-value tile the maps are for (4, 8, 16 or TILE_SPLIT)
 cudaError_t make_tile_maps(const Grid &g, float *vtx, float *xe, float *ye, float *avg, int tile_h,
                            TileMaps *out);
 // one-time kernel attributes (shared-memory size) on the current device
 cudaError_t prepare_pointvalue();
-// batched point values over a tile list of tile height tile_h (4, 8 or 16): the
-// tiles of the instances of class 0 first, ntiles[0] of them, then those of class 1
+// whether a run takes the kernels with the switches for discontinuous data
+inline bool shock_options(const Options &o) { return o.tsw || o.shock_blend || o.node_bounds || o.force_lo; }
+// batched point values over a tile list: the tiles of the instances of class 0
+// first, ntiles[0] of them of height tile_h[0] (4, 8 or 16), then those of class 1
 // and 2 (batch_class of an instance's arguments: which instantiation of the
 // kernel its options need; a launch a class)
 constexpr int PV_CLASSES = 3;
 int batch_class(const PointValueArgs &A);
+constexpr int TILE_OF_CLASS[PV_CLASSES] = {TILE_PLAIN, TILE_PLAIN, TILE_TALL};
 // of the unit with the switches for discontinuous data (af_pointvalue_shock.cu)
 cudaError_t prepare_pointvalue_shock();
 cudaError_t launch_pointvalue_shock(const PointValueArgs &A, const TileMaps &maps, int tile_h, cudaStream_t s);
 void launch_pointvalue_shock_batch(const PointValueBatch &B, int ntiles, int tile_h, cudaStream_t s);
-cudaError_t launch_pointvalue_batch(const PointValueBatch &B, const int ntiles[PV_CLASSES], int tile_h, cudaStream_t s);
+cudaError_t launch_pointvalue_batch(const PointValueBatch &B, const int ntiles[PV_CLASSES],
+                                    const int tile_h[PV_CLASSES], cudaStream_t s);
 // t^n snapshot (hi -> q0) of every active instance with the flux limiter on
 cudaError_t launch_snapshot_batch(const FluxBatch &B, int n, cudaStream_t s);
 // batched flux / update over a tile list of 32 x 8 cells: the first nplain

@@ -120,21 +120,24 @@ cudaError_t launch_pointvalue_masked(const Grid &g, const NodeSet &n0, const flo
 int batch_class(const PointValueArgs &A) { return pv_class(A); }
 
 template <int TY>
-static void launch_batch_h(PointValueBatch B, const int ntiles[PV_CLASSES], cudaStream_t s) {
+static void launch_batch_h(const PointValueBatch &B, int c, int ntiles, cudaStream_t s) {
   const dim3 blk(TX, TY);
-  if (ntiles[PV_LEAN] > 0) pointvalue_batch_kernel<TY, PV_LEAN><<<ntiles[PV_LEAN], blk, Tile<TY>::SMEM_BYTES, s>>>(B);
-  B.tiles += ntiles[PV_LEAN];
-  if (ntiles[PV_FULL] > 0) pointvalue_batch_kernel<TY, PV_FULL><<<ntiles[PV_FULL], blk, Tile<TY>::SMEM_BYTES, s>>>(B);
-  B.tiles += ntiles[PV_FULL];
-  if (ntiles[PV_SHOCK] > 0) launch_pointvalue_shock_batch(B, ntiles[PV_SHOCK], TY, s);
+  if (c == PV_LEAN) pointvalue_batch_kernel<TY, PV_LEAN><<<ntiles, blk, Tile<TY>::SMEM_BYTES, s>>>(B);
+  else if (c == PV_FULL) pointvalue_batch_kernel<TY, PV_FULL><<<ntiles, blk, Tile<TY>::SMEM_BYTES, s>>>(B);
+  else launch_pointvalue_shock_batch(B, ntiles, TY, s);
 }
-cudaError_t launch_pointvalue_batch(const PointValueBatch &B, const int ntiles[PV_CLASSES], int tile_h, cudaStream_t s) {
+cudaError_t launch_pointvalue_batch(const PointValueBatch &B, const int ntiles[PV_CLASSES],
+                                    const int tile_h[PV_CLASSES], cudaStream_t s) {
   static_assert(PV_LEAN == 0 && PV_FULL == 1 && PV_SHOCK == 2 && PV_CLASSES == 3, "order of the tile list");
-  switch (tile_h) {
-    case 4: launch_batch_h<4>(B, ntiles, s); break;
-    case 8: launch_batch_h<8>(B, ntiles, s); break;
-    case 16: launch_batch_h<16>(B, ntiles, s); break;
-    default: return cudaErrorInvalidValue;
+  PointValueBatch L = B;
+  for (int c = 0; c < PV_CLASSES; L.tiles += ntiles[c++]) {
+    if (ntiles[c] == 0) continue;
+    switch (tile_h[c]) {
+      case 4: launch_batch_h<4>(L, c, ntiles[c], s); break;
+      case 8: launch_batch_h<8>(L, c, ntiles[c], s); break;
+      case 16: launch_batch_h<16>(L, c, ntiles[c], s); break;
+      default: return cudaErrorInvalidValue;
+    }
   }
   return cudaGetLastError();
 }
