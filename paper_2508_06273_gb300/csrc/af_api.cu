@@ -98,10 +98,6 @@ int ensure_staging(af_ctx *h) {
   return AF_OK;
 }
 
-// the words of host_words that kernels write: [0], [1] export_words_kernel;
-// [4], [5] the wave speed's bits and bad flag; [6] a differing periodic duplicate
-enum { HW_SPEED = 4, HW_BAD = 6 };
-
 cudaError_t make_maps(af_ctx *h) {
   cudaError_t e = cudaSuccess;
   for (int b = 0; b < 2 && e == cudaSuccess; b++) {
@@ -126,6 +122,7 @@ void drop_runs(af_ctx *h) {
 int load_state(af_ctx *h, const float *const src[4]) {
   h->speed_valid = false;
   cudaStream_t s = h->stream;
+  h->words_on_host = false;
   h->host_words[HW_BAD] = 0;
   CK(launch_check_state(h->g, src, h->host_words_dev + HW_BAD, h->d_speed, h->d_speed_bad, s), "check_dup");
   if (h->g.per_x || h->g.per_y) {
@@ -250,8 +247,8 @@ af_ctx *af_create(int nx, int ny, double dx, double dy, double gamma, uint32_t b
     delete h;
     return nullptr;
   }
-  const size_t small = 64 + 64 + 64 + 64 + sizeof(double) * (TOTALS_BLOCKS * NV + NV);
-  e = cudaHostAlloc(&h->host_words, 64, cudaHostAllocMapped);
+  const size_t small = 64 + 64 + 64 + 64 + sizeof(double) * TOTALS_BLOCKS * NV;
+  e = cudaHostAlloc(&h->host_words, HW_WORDS * sizeof(unsigned), cudaHostAllocMapped);
   if (e == cudaSuccess) e = cudaHostGetDevicePointer(&h->host_words_dev, h->host_words, 0);
   if (e == cudaSuccess) e = cudaMalloc(&h->small, small);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking);
@@ -266,6 +263,7 @@ af_ctx *af_create(int nx, int ny, double dx, double dy, double gamma, uint32_t b
     delete h;
     return nullptr;
   }
+  std::memset(h->host_words, 0, HW_WORDS * sizeof(unsigned));
   char *sp = (char *)h->small;
   h->d_status = (int *)sp;
   h->d_bad = (int *)(sp + 64);
@@ -273,10 +271,8 @@ af_ctx *af_create(int nx, int ny, double dx, double dy, double gamma, uint32_t b
   h->d_speed = (unsigned *)(sp + 128);
   h->d_ticket = (unsigned *)(sp + 136);
   h->d_speed_bad = (int *)(sp + 160);
-  h->d_min_keys = (unsigned *)(sp + 164);
   h->d_counters = (unsigned long long *)(sp + 192);  // two slots of four
-  h->d_totals = (double *)(sp + 256);
-  h->d_partials = h->d_totals + NV;
+  h->d_partials = (double *)(sp + 256);
   h->stream = h->own_stream;
   // the whole state starts zeroed, ghosts included; checking builds fill it
   // with NaN instead, so that a read of a point no step or set call wrote
@@ -540,6 +536,7 @@ int af_set_state_host(af_ctx *h, const float *avg, const float *vtx, const float
   CK(cudaMemcpyAsync(&bad, h->d_bad, sizeof(int), cudaMemcpyDeviceToHost, s), "memcpy");
   CK(cudaMemsetAsync(h->lo, 0, sizeof(float) * NV * h->g.plane, s), "memset lo");
   CK(cudaMemsetAsync(h->d_status, 0, sizeof(int), s), "memset status");
+  h->words_on_host = false;
   CK(cudaStreamSynchronize(s), "sync");
   if (bad) {
     h->has_state = false;
@@ -696,6 +693,7 @@ int af_set_state_host_async(af_ctx *h, const float *avg, const float *vtx, const
   CK(cudaEventRecord(h->in_free, s), "event");
   CK(cudaMemsetAsync(h->lo, 0, sizeof(float) * NV * h->g.plane, s), "memset lo");
   CK(cudaMemsetAsync(h->d_status, 0, sizeof(int), s), "memset status");
+  h->words_on_host = false;
   h->speed_valid = false;
   h->ghost_valid = false;
   h->has_state = true;
@@ -915,7 +913,7 @@ static int enqueue_step(af_ctx *h, double dt) {
   // fills the new state's ghosts and hands the wave speed to the host
   const bool small = flux_fills_ghosts(h->g);
   const StepTail tail = {h->lev[2], h->d_counters + 4 * (h->tmap_cur ^ 1), small ? h->host_words_dev + HW_SPEED : nullptr,
-                         small ? h->d_ticket : nullptr};
+                         small ? h->d_ticket : nullptr, counters};
   if (h->opt.surrogate || !h->opt.node_flux) {
     CK(launch_flux_update(h->g, h->lev[0], h->lev[1], h->lev[2], h->hi, h->lo, dt / h->dx, dt / h->dy,
                           h->d_status, h->d_speed, h->d_speed_bad, h->opt.flux_limiter, h->q0, tail, s),
@@ -927,7 +925,7 @@ static int enqueue_step(af_ctx *h, double dt) {
        "flux update");
   }
   h->speed_valid = true;
-  h->speed_on_host = h->ghost_valid = small;
+  h->speed_on_host = h->words_on_host = h->ghost_valid = small;
   h->launches[AF_STAGE_FLUX] += 1;
   if (prof) {
     cudaEventRecord(h->ev_stage[4], s);
@@ -974,6 +972,7 @@ static int step64(af_ctx *h, double dt) {
   S.lin_mode = o.lin_mode;
   S.correction = o.correction;
   S.status = h->d_status;
+  h->words_on_host = false;
   CK(launch_step64(S, dt / h->dx, dt / h->dy, s), "FP64 step");
   for (int k = 0; k < 3; k++) std::swap(h->f64_lev[0][k], h->f64_lev[2][k]);
   return AF_OK;
@@ -1076,7 +1075,7 @@ int af_run(af_ctx *h, int nsteps, double dt) {
     h->launches[AF_STAGE_FLUX] += 2;
   }
   h->speed_valid = true;
-  h->speed_on_host = h->ghost_valid = flux_fills_ghosts(h->g);
+  h->speed_on_host = h->words_on_host = h->ghost_valid = flux_fills_ghosts(h->g);
   if (nsteps & 1) return enqueue_step(h, dt);
   return AF_OK;
 }
@@ -1096,6 +1095,11 @@ int af_debug_bounds(unsigned *out) {
 int af_status(af_ctx *h) {
   if (!h) return fail(AF_ERR_ARG, "null handle%s");
   DeviceGuard dg(h->device);
+  if (h->words_on_host) {  // written by the last step's flux kernel: nothing to fetch or clear if no bit is set
+    CK(cudaStreamSynchronize(h->stream), "sync");
+    if (reinterpret_cast<volatile unsigned *>(h->host_words)[HW_STATUS] == 0) return h->timed_out ? AF_ST_TIMEOUT : 0;
+    h->host_words[HW_STATUS] = 0;
+  }
   CK(launch_export_words(reinterpret_cast<unsigned *>(h->d_status), nullptr, 1, h->host_words_dev, h->stream),
      "status");
   CK(cudaStreamSynchronize(h->stream), "sync");
@@ -1107,9 +1111,12 @@ int af_status(af_ctx *h) {
 int af_counters(af_ctx *h, int64_t out[4]) {
   if (!h || !out) return fail(AF_ERR_ARG, "null argument%s");
   DeviceGuard dg(h->device);
-  unsigned long long c[4];
-  CK(cudaMemcpyAsync(c, h->d_counters + 4 * (h->tmap_cur ^ 1), sizeof(c), cudaMemcpyDeviceToHost, h->stream), "counters");
+  if (!h->words_on_host)
+    CK(launch_export_counters(h->d_counters + 4 * (h->tmap_cur ^ 1),
+                              reinterpret_cast<unsigned long long *>(h->host_words_dev + HW_COUNTERS), h->stream),
+       "counters");
   CK(cudaStreamSynchronize(h->stream), "sync");
+  const volatile unsigned long long *c = reinterpret_cast<unsigned long long *>(h->host_words + HW_COUNTERS);
   for (int k = 0; k < 4; k++) out[k] = (int64_t)c[k];
   return AF_OK;
 }
@@ -1124,11 +1131,12 @@ int af_conserved_totals(af_ctx *h, double out[4]) {
     CK(cudaStreamSynchronize(h->stream), "sync");
     return AF_OK;
   }
-  CK(launch_totals(h->g, h->hi, h->lo, h->d_partials, h->d_totals, h->stream), "totals");
-  h->launches[AF_STAGE_REDUCE] += 2;
-  double t[4];
-  CK(cudaMemcpyAsync(t, h->d_totals, sizeof(t), cudaMemcpyDeviceToHost, h->stream), "totals");
+  CK(launch_totals(h->g, h->hi, h->lo, h->d_partials, reinterpret_cast<double *>(h->host_words_dev + HW_TOTALS),
+                   h->d_ticket, h->stream),
+     "totals");
+  h->launches[AF_STAGE_REDUCE] += 1;
   CK(cudaStreamSynchronize(h->stream), "sync");
+  const volatile double *t = reinterpret_cast<double *>(h->host_words + HW_TOTALS);
   for (int v = 0; v < 4; v++) out[v] = t[v] * h->dx * h->dy;
   return AF_OK;
 }
@@ -1151,10 +1159,10 @@ int af_state_min(af_ctx *h, float out[2]) {
   if (!h->has_state) return fail(AF_ERR_STATE, "no state set%s");
   if (h->fp64) return fail(AF_ERR_STATE, "af_state_min: the FP64 state has no FP32 minima (use af_get_state_f64)%s");
   DeviceGuard dg(h->device);
-  CK(launch_state_min(h->g, h->hi, h->lev[0], h->d_min_keys, h->stream), "state minima");
-  unsigned keys[3];
-  CK(cudaMemcpyAsync(keys, h->d_min_keys, sizeof(keys), cudaMemcpyDeviceToHost, h->stream), "state minima");
+  CK(launch_state_min(h->g, h->hi, h->lev[0], h->d_partials, h->host_words_dev + HW_RESULT, h->d_ticket, h->stream),
+     "state minima");
   CK(cudaStreamSynchronize(h->stream), "sync");
+  const volatile unsigned *keys = h->host_words + HW_RESULT;
   for (int q = 0; q < 2; q++) {
     const unsigned u = (keys[q] & 0x80000000u) ? (keys[q] & 0x7FFFFFFFu) : ~keys[q];
     std::memcpy(&out[q], &u, sizeof(float));
@@ -1203,12 +1211,14 @@ int af_max_speed(af_ctx *h, float *out) {
     CK(cudaEventCreate(&e1), "event");
     cudaEventRecord(e0, h->stream);
   }
-  CK(launch_max_speed(h->g, h->hi, h->lev[0], h->d_speed, h->d_speed_bad, h->stream), "max speed");
+  CK(launch_max_speed(h->g, h->hi, h->lev[0], h->d_partials, h->d_speed, h->d_speed_bad, h->host_words_dev + HW_SPEED,
+                      h->d_ticket, h->stream),
+     "max speed");
   h->launches[AF_STAGE_REDUCE] += 1;
   if (h->profile) cudaEventRecord(e1, h->stream);
-  unsigned bits = 0;
-  int bad = 0;
-  CK(read_speed(h, bits, bad), "speed");
+  CK(cudaStreamSynchronize(h->stream), "sync");
+  const unsigned bits = w[HW_SPEED];
+  const int bad = (int)w[HW_SPEED + 1];
   if (h->profile) {
     float ms = 0.0f;
     if (cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) h->stage_ms[AF_STAGE_REDUCE] += ms;
@@ -1218,8 +1228,7 @@ int af_max_speed(af_ctx *h, float *out) {
   float m;
   std::memcpy(&m, &bits, sizeof(m));
   *out = bad ? NAN : m;
-  h->speed_valid = true;
-  h->speed_on_host = false;
+  h->speed_valid = h->speed_on_host = true;
   return AF_OK;
 }
 

@@ -339,7 +339,8 @@ int ensure_speeds(af_batch *b) {
     if (b->speed_ok[k]) continue;
     af_ctx *h = b->inst[k];
     BatchCtl *c = b->d_ctl + k;
-    BCK(launch_max_speed(h->g, h->hi, h->tbuf[b->ctl_h[k].cur], &c->speed, &c->speed_bad, b->stream),
+    BCK(launch_max_speed(h->g, h->hi, h->tbuf[b->ctl_h[k].cur], h->d_partials, &c->speed, &c->speed_bad,
+                         h->host_words_dev + HW_RESULT, h->d_ticket, b->stream),
         "batch: max speed");
     b->speed_ok[k] = 1;
   }

@@ -22,6 +22,13 @@ struct NvtxScope {
   NvtxScope &operator=(const NvtxScope &) = delete;
 };
 
+// the host words that kernels write: [0], [1] export_words_kernel's; by a step's flux
+// kernel and a state's load the wave speed's bits and bad flag; a differing
+// periodic duplicate; by a step the status and the four event counters (64 bits
+// each); the FP64 totals; minima
+enum { HW_SPEED = 4, HW_BAD = 6, HW_STATUS = 7, HW_COUNTERS = 8, HW_TOTALS = 16, HW_RESULT = 24, HW_WORDS = 32 };
+static_assert(HW_STATUS == HW_SPEED + 3 && HW_COUNTERS == HW_SPEED + 4, "FluxArgs::host_words");
+
 struct af_ctx {
   Grid g;
   double dx, dy, gamma;  // as given to af_create
@@ -62,7 +69,7 @@ struct af_ctx {
   unsigned long long *d_counters;
   unsigned *d_ticket;  // blocks done, of the kernels whose last block writes host words
   bool ghost_valid;    // the ghost entries of the averages and of lev[0] belong to the current state
-  double *d_partials, *d_totals;
+  double *d_partials;  // scratch of the reductions
   // host transfers: one staging area and one copy stream per external array
   // (lazily created), so that the four copies of a transfer run concurrently
   float *staging;
@@ -77,10 +84,9 @@ struct af_ctx {
   cudaEvent_t in_free, out_ready, out_done[2][4];
   bool async_init, async_pending;
   int *d_bad_async;
-  // two words of mapped pinned host memory (host and device addresses) for
-  // the small reads (status, max speed)
-  unsigned *d_min_keys;  // state minima (af_state_min): rho, p as ordered keys, non-finite flag
-  unsigned *host_words, *host_words_dev;  // a periodic duplicate line differed in an asynchronous upload
+  // mapped pinned host memory (host and device addresses) that kernels write
+  // small results to
+  unsigned *host_words, *host_words_dev;
   bool has_state;
   // a block's wait for staged data or for the tensor cores ran out (seen by
   // af_status): the state is invalid and the handle refuses further steps
@@ -91,7 +97,8 @@ struct af_ctx {
   double run_dt[2];
   Options run_opt[2];
   bool speed_valid;    // d_speed holds the max wave speed of the current state
-  bool speed_on_host;  // and so do host_words[4], [5] once the stream is done
+  bool speed_on_host;  // and so do host words HW_SPEED once the stream is done
+  bool words_on_host;  // the same of the status and the event counters
   cudaEvent_t ev_in, ev_out;
   // profiling: events around each stage of the last step, accumulated times
   int profile;

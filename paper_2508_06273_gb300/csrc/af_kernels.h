@@ -138,18 +138,22 @@ struct FluxArgs {
   float *ghost[3];                     // node arrays of the new state, whose ghost entries the blocks
                                        // beyond the tiles fill; the averages' images are stored with them
   unsigned long long *clear_counters;  // the next step's event counters
-  unsigned *host_speed;                // mapped host words: speed bits and the bad flag, by the last block
+  // mapped host words, by the last block: [0], [1] speed bits and the bad flag,
+  // [3] the status, [4] on the step's event counters (64 bits each)
+  unsigned *host_words;
   unsigned *ticket;                    // blocks done so far (returns to 0)
+  const unsigned long long *counters;  // this step's event counters
 };
 // whether the flux kernel of this grid takes the form that fills the new state's
-// ghosts and hands the wave speed to the host (host_speed and ticket are then
+// ghosts and hands the small results to the host (host_words and ticket are then
 // given, else NULL; clear_counters always)
 bool flux_fills_ghosts(const Grid &g);
 // what FluxArgs::ghost .. ticket are set to for a single grid
 struct StepTail {
   NodeSet ghost;
   unsigned long long *clear_counters;
-  unsigned *host_speed, *ticket;
+  unsigned *host_words, *ticket;
+  const unsigned long long *counters;
 };
 FluxArgs flux_args(const Grid &g, const NodeSet &n0, const NodeSet &n1, const NodeSet &n2, float *avg_hi,
                    float *avg_lo, int *status, unsigned *speed, int *speed_bad);
@@ -282,21 +286,28 @@ cudaError_t launch_flux_update(const Grid &g, const NodeSet &n0, const NodeSet &
 cudaError_t launch_flux_nf(const Grid &g, const float *const nf[4], float *avg_hi, float *avg_lo, double lamx,
                            double lamy, int *status, unsigned *speed, int *speed_bad, int flux_limiter,
                            const float *q0, const StepTail &tail, cudaStream_t s);
-// max over averages and owned point values of max(|u|,|v|) + c (as float bits)
 // words a and b (b may be null) into mapped host memory dst, clearing a if
 // clear_a: small results reach the host without a copy engine, so that they
 // do not queue behind a large transfer
 cudaError_t launch_export_words(unsigned *a, unsigned *b, int clear_a, unsigned *dst, cudaStream_t s);
-// minimum rho and p over the primitive averages and the node arrays into
-// keys[0], keys[1] (order-preserving keys of the floats), keys[2] = 1 if a
-// value is not finite
-cudaError_t launch_state_min(const Grid &g, const float *avg_hi, const NodeSet &n, unsigned *keys, cudaStream_t s);
-cudaError_t launch_max_speed(const Grid &g, const float *avg_hi, const NodeSet &n,
-                             unsigned *out_bits, int *bad, cudaStream_t s);
-// fixed-order FP64 sums of hi + lo per variable: partials[nblk][4] -> out[4]
+// The reductions below take one launch each and leave their result in mapped
+// host memory; scratch: TOTALS_BLOCKS * NV doubles, ticket: a zero word that they
+// leave zero.
 constexpr int TOTALS_BLOCKS = 256;
-cudaError_t launch_totals(const Grid &g, const float *avg_hi, const float *avg_lo, double *partials,
-                          double *out, cudaStream_t s);
+// minimum rho and p over the primitive averages and the node arrays into
+// host[0], host[1] (order-preserving keys of the floats), host[2] = 1 if a
+// value is not finite
+cudaError_t launch_state_min(const Grid &g, const float *avg_hi, const NodeSet &n, double *scratch, unsigned *host,
+                             unsigned *ticket, cudaStream_t s);
+// max over averages and owned point values of max(|u|,|v|) + c (as float bits)
+// and the bad flag into the device words and host[0], host[1]
+cudaError_t launch_max_speed(const Grid &g, const float *avg_hi, const NodeSet &n, double *scratch, unsigned *out_bits,
+                             int *bad, unsigned *host, unsigned *ticket, cudaStream_t s);
+// fixed-order FP64 sums of hi + lo per variable into host[4]
+cudaError_t launch_totals(const Grid &g, const float *avg_hi, const float *avg_lo, double *scratch, double *host,
+                          unsigned *ticket, cudaStream_t s);
+// a step's four event counters into host[4]
+cudaError_t launch_export_counters(const unsigned long long *c, unsigned long long *host, cudaStream_t s);
 // a state's four external arrays (averages, vertices, x-edges, y-edges; device
 // memory) into the padded planes in one launch: ghost entries included, low
 // words and *status cleared, and the state's max wave speed into *speed /

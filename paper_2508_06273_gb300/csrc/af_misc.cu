@@ -159,50 +159,6 @@ __global__ void export_words_kernel(unsigned *a, unsigned *b, int clear_a, unsig
   __threadfence_system();
 }
 
-__global__ void max_speed_kernel(Grid g, const float *__restrict__ avg, const float *__restrict__ V,
-                                 const float *__restrict__ X, const float *__restrict__ Y,
-                                 unsigned *out, int *badflag) {
-  const long long nc = (long long)g.nx * g.ny, nv = (long long)g.nxv * g.nyv;
-  const long long nxe = (long long)g.nxv * g.ny, nye = (long long)g.nx * g.nyv;
-  const long long total = nc + nv + nxe + nye;
-  float m = 0.0f;
-  bool bad = false;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total;
-       k += (long long)gridDim.x * blockDim.x) {
-    float U[4];
-    long long r = k;
-    if (r < nc) {
-      const int i = (int)(r % g.nx), j = (int)(r / g.nx);
-      float Q[4];
-#pragma unroll
-      for (int v = 0; v < NV; v++) Q[v] = __ldg(avg + at(g, v, i, j));
-      c2p(Q, g.gamma - 1.0f, U);
-    } else {
-      const float *p;
-      int ni;
-      if ((r -= nc) < nv) {
-        p = V;
-        ni = g.nxv;
-      } else if ((r -= nv) < nxe) {
-        p = X;
-        ni = g.nxv;
-      } else {
-        r -= nxe;
-        p = Y;
-        ni = g.nx;
-      }
-      const int i = (int)(r % ni), j = (int)(r / ni);
-#pragma unroll
-      for (int v = 0; v < NV; v++) U[v] = __ldg(p + at(g, v, i, j));
-    }
-    m = fmaxf(m, wave_speed(U, g.gamma, bad));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));
-  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(badflag, 1);
-}
-
 // order-preserving unsigned key of a float (atomicMin on keys is a min on
 // the floats; -0 and +0 get neighbouring keys)
 __device__ __forceinline__ unsigned float_key(float f) {
@@ -210,93 +166,56 @@ __device__ __forceinline__ unsigned float_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// minimum density and pressure over the primitive cell averages and the three
-// node arrays of a state (keys[0], keys[1]); keys[2] set if a value is not finite
-__global__ void state_min_kernel(Grid g, const float *__restrict__ avg, const float *__restrict__ V,
-                                 const float *__restrict__ X, const float *__restrict__ Y, unsigned *keys) {
-  const long long nc = (long long)g.nx * g.ny, nv = (long long)g.nxv * g.nyv;
-  const long long nxe = (long long)g.nxv * g.ny, nye = (long long)g.nx * g.nyv;
-  const long long total = nc + nv + nxe + nye;
-  float rmin = __int_as_float(0x7f800000), pmin = __int_as_float(0x7f800000);
-  bool bad = false;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total;
-       k += (long long)gridDim.x * blockDim.x) {
-    float U[4];
-    long long r = k;
-    if (r < nc) {
-      const int i = (int)(r % g.nx), j = (int)(r / g.nx);
-      float Q[4];
-#pragma unroll
-      for (int v = 0; v < NV; v++) Q[v] = __ldg(avg + at(g, v, i, j));
-      c2p(Q, g.gamma - 1.0f, U);
-    } else {
-      const float *p;
-      int ni;
-      if ((r -= nc) < nv) {
-        p = V;
-        ni = g.nxv;
-      } else if ((r -= nv) < nxe) {
-        p = X;
-        ni = g.nxv;
-      } else {
-        r -= nxe;
-        p = Y;
-        ni = g.nx;
-      }
-      const int i = (int)(r % ni), j = (int)(r / ni);
-#pragma unroll
-      for (int v = 0; v < NV; v++) U[v] = __ldg(p + at(g, v, i, j));
-    }
-    bad |= !(isfinite(U[0]) && isfinite(U[1]) && isfinite(U[2]) && isfinite(U[3]));
-    rmin = fminf(rmin, U[0]);
-    pmin = fminf(pmin, U[3]);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
-    pmin = fminf(pmin, __shfl_xor_sync(0xffffffffu, pmin, o));
-  }
-  const bool anybad = __any_sync(0xffffffffu, bad);
-  if ((threadIdx.x & 31) == 0) {
-    atomicMin(keys, float_key(rmin));
-    atomicMin(keys + 1, float_key(pmin));
-    if (anybad) atomicOr(keys + 2, 1u);
-  }
-}
-
-// stage 1: block b sums rows b, b + nblk, ... in a fixed order
-__global__ void totals_stage1(Grid g, const float *__restrict__ hi, const float *__restrict__ lo,
-                              double *partials) {
-  __shared__ double sm[4][256];
+// Block b sums rows b, b + nblk, ... in a fixed order; the last block to finish
+// sums the blocks' sums, in a fixed order too, into mapped host memory.  A read
+// of this, of the minima or of the wave speed is bound by latency on all but the
+// largest grids: it takes one launch and a wait, where it took memsets, a second
+// launch and a device-to-host copy (8 steps on 211 x 149 cells with all of a log's
+// reads each: 1065 -> 760 us).
+__global__ void __launch_bounds__(TOTALS_BLOCKS) totals_kernel(Grid g, const float *__restrict__ hi,
+                                                               const float *__restrict__ lo, double *partials,
+                                                               unsigned *ticket, double *host) {
+  __shared__ double sm[4][TOTALS_BLOCKS];
+  __shared__ bool last;
   double acc[4] = {0, 0, 0, 0};
   for (int j = blockIdx.x; j < g.ny; j += gridDim.x)
     for (int i = threadIdx.x; i < g.nx; i += blockDim.x)
 #pragma unroll
       for (int v = 0; v < NV; v++) acc[v] += (double)hi[at(g, v, i, j)] + (double)lo[at(g, v, i, j)];
+  auto block_sum = [&] {
 #pragma unroll
-  for (int v = 0; v < NV; v++) sm[v][threadIdx.x] = acc[v];
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-#pragma unroll
-      for (int v = 0; v < NV; v++) sm[v][threadIdx.x] += sm[v][threadIdx.x + s];
+    for (int v = 0; v < NV; v++) sm[v][threadIdx.x] = acc[v];
     __syncthreads();
+    for (int s = TOTALS_BLOCKS / 2; s > 0; s >>= 1) {
+      if (threadIdx.x < s)
+#pragma unroll
+        for (int v = 0; v < NV; v++) sm[v][threadIdx.x] += sm[v][threadIdx.x + s];
+      __syncthreads();
+    }
+  };
+  block_sum();
+  if (threadIdx.x < NV) {
+    partials[blockIdx.x * NV + threadIdx.x] = sm[threadIdx.x][0];
+    __threadfence();
   }
-  if (threadIdx.x < NV) partials[blockIdx.x * NV + threadIdx.x] = sm[threadIdx.x][0];
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+#pragma unroll
+  for (int v = 0; v < NV; v++) acc[v] = __ldcg(partials + threadIdx.x * NV + v);
+  block_sum();
+  if (threadIdx.x < NV) {
+    ((volatile double *)host)[threadIdx.x] = sm[threadIdx.x][0];
+    __threadfence_system();
+  }
+  if (threadIdx.x == 0) *ticket = 0;
 }
 
-__global__ void totals_stage2(const double *partials, double *out) {
-  __shared__ double sm[4][TOTALS_BLOCKS];
-#pragma unroll
-  for (int v = 0; v < NV; v++) sm[v][threadIdx.x] = partials[threadIdx.x * NV + v];
-  __syncthreads();
-  for (int s = TOTALS_BLOCKS / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-#pragma unroll
-      for (int v = 0; v < NV; v++) sm[v][threadIdx.x] += sm[v][threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x < NV) out[threadIdx.x] = sm[threadIdx.x][0];
+__global__ void export_counters_kernel(const unsigned long long *c, unsigned long long *host) {
+  if (threadIdx.x < 4) ((volatile unsigned long long *)host)[threadIdx.x] = c[threadIdx.x];
+  __threadfence_system();
 }
 
 __global__ void pack_kernel(Grid g, const float *__restrict__ src, float *dst, int ni, int nj,
@@ -444,6 +363,105 @@ __global__ void __launch_bounds__(ST_W *ST_H / ST_ROWS) store_state_kernel(const
   }
 }
 
+// Reductions over a whole state (averages in primitive form and owned point
+// values), tile by tile as above: MIN: the minimum density and pressure (as
+// ordered keys); else the maximum wave speed.  part[block] = (value, value or 0,
+// bad); the last block reduces the blocks' and writes the result to mapped host
+// memory and, for the speed, to the device words.
+struct ReduceArgs {
+  Grid g;
+  StateTiles T;
+  const float *pad[4];
+  unsigned *part, *ticket, *host;
+  unsigned *speed;
+  int *speed_bad;
+};
+constexpr int RED_THREADS = ST_W * ST_H / ST_ROWS;
+template <bool MIN>
+__global__ void __launch_bounds__(RED_THREADS) reduce_state_kernel(const __grid_constant__ ReduceArgs A) {
+  const Grid &g = A.g;
+  unsigned k0 = MIN ? ~0u : 0u, k1 = k0;  // keys of rho and p, or the speed's bits
+  float m = 0.0f;
+  bool bad = false;
+  for (unsigned t = blockIdx.x; t < A.T.first[4]; t += gridDim.x) {
+    unsigned b = t;
+    const int w = b < A.T.first[1] ? 0 : (b < A.T.first[2] ? 1 : (b < A.T.first[3] ? 2 : 3));
+    b -= A.T.first[w];
+    const int ni = w == 1 || w == 2 ? g.nxv : g.nx, nj = w == 1 || w == 3 ? g.nyv : g.ny;
+    const int i = (int)(b % A.T.tx[w]) * ST_W + (int)threadIdx.x, j0 = (int)(b / A.T.tx[w]) * ST_H + (int)threadIdx.y;
+    if (i >= ni) continue;
+    float x[ST_ROWS][4];
+#pragma unroll
+    for (int r = 0; r < ST_ROWS; r++) {
+      const int j = min(j0 + r * (ST_H / ST_ROWS), nj - 1);  // (a row beyond the last repeats it)
+#pragma unroll
+      for (int v = 0; v < NV; v++) x[r][v] = __ldg(A.pad[w] + at(g, v, i, j));
+    }
+#pragma unroll
+    for (int r = 0; r < ST_ROWS; r++) {
+      float U[4] = {x[r][0], x[r][1], x[r][2], x[r][3]};
+      if (w == 0) c2p(x[r], g.gamma - 1.0f, U);
+      if (MIN) {
+        bad |= !(isfinite(U[0]) && isfinite(U[1]) && isfinite(U[2]) && isfinite(U[3]));
+        k0 = min(k0, float_key(U[0]));
+        k1 = min(k1, float_key(U[3]));
+      } else {
+        m = fmaxf(m, wave_speed(U, g.gamma, bad));
+      }
+    }
+  }
+  if (!MIN) k0 = __float_as_uint(m);
+  __shared__ unsigned s0[RED_THREADS / 32], s1[RED_THREADS / 32];
+  __shared__ bool last;
+  const int tid = threadIdx.y * ST_W + threadIdx.x;
+  auto block_reduce = [&](unsigned &a, unsigned &b, bool f) {
+    a = MIN ? __reduce_min_sync(0xffffffffu, a) : __reduce_max_sync(0xffffffffu, a);
+    b = MIN ? __reduce_min_sync(0xffffffffu, b) : 0u;
+    if ((tid & 31) == 0) {
+      s0[tid >> 5] = a;
+      s1[tid >> 5] = b;
+    }
+    const bool any = __syncthreads_or(f) != 0;
+    for (int w = 0; w < RED_THREADS / 32; w++) {
+      a = MIN ? min(a, s0[w]) : max(a, s0[w]);
+      b = MIN ? min(b, s1[w]) : 0u;
+    }
+    return any;
+  };
+  const bool any = block_reduce(k0, k1, bad);
+  if (tid == 0) {
+    A.part[3 * blockIdx.x] = k0;
+    A.part[3 * blockIdx.x + 1] = k1;
+    A.part[3 * blockIdx.x + 2] = any;
+    __threadfence();
+    last = atomicAdd(A.ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  bool f = false;
+  k0 = k1 = MIN ? ~0u : 0u;
+  for (unsigned q = tid; q < gridDim.x; q += RED_THREADS) {
+    const unsigned a = __ldcg(A.part + 3 * q), b = __ldcg(A.part + 3 * q + 1);
+    k0 = MIN ? min(k0, a) : max(k0, a);
+    k1 = MIN ? min(k1, b) : 0u;
+    f |= __ldcg(A.part + 3 * q + 2) != 0u;
+  }
+  const bool flag = block_reduce(k0, k1, f);
+  if (tid == 0) {
+    volatile unsigned *h = A.host;
+    h[0] = k0;
+    h[1] = MIN ? k1 : (unsigned)flag;
+    if (MIN) h[2] = flag;
+    if (!MIN) {
+      *A.speed = k0;
+      *A.speed_bad = flag;
+    }
+    *A.ticket = 0;
+    __threadfence_system();
+  }
+}
+
 // periodic duplicate lines of the three node arrays (blockIdx.z; y: variable)
 struct CheckArgs {
   Grid g;
@@ -539,34 +557,6 @@ cudaError_t launch_export_words(unsigned *a, unsigned *b, int clear_a, unsigned 
   return cudaGetLastError();
 }
 
-cudaError_t launch_max_speed(const Grid &g, const float *avg_hi, const NodeSet &n,
-                             unsigned *out_bits, int *bad, cudaStream_t s) {
-  cudaMemsetAsync(out_bits, 0, sizeof(unsigned), s);
-  cudaMemsetAsync(bad, 0, sizeof(int), s);
-  long long total = 4LL * (g.nx + 1) * (g.ny + 1);
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 4096) blocks = 4096;
-  max_speed_kernel<<<blocks, 256, 0, s>>>(g, avg_hi, n.k[VTX], n.k[XE], n.k[YE], out_bits, bad);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_state_min(const Grid &g, const float *avg_hi, const NodeSet &n, unsigned *keys, cudaStream_t s) {
-  cudaMemsetAsync(keys, 0xFF, 2 * sizeof(unsigned), s);
-  cudaMemsetAsync(keys + 2, 0, sizeof(unsigned), s);
-  long long total = 4LL * (g.nx + 1) * (g.ny + 1);
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 4096) blocks = 4096;
-  state_min_kernel<<<blocks, 256, 0, s>>>(g, avg_hi, n.k[VTX], n.k[XE], n.k[YE], keys);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_totals(const Grid &g, const float *avg_hi, const float *avg_lo, double *partials,
-                          double *out, cudaStream_t s) {
-  totals_stage1<<<TOTALS_BLOCKS, 256, 0, s>>>(g, avg_hi, avg_lo, partials);
-  totals_stage2<<<1, TOTALS_BLOCKS, 0, s>>>(partials, out);
-  return cudaGetLastError();
-}
-
 // tiles of the four arrays of extents ni x nj (0: left out)
 static StateTiles state_tiles(const int ni[4], const int nj[4]) {
   StateTiles T;
@@ -576,6 +566,49 @@ static StateTiles state_tiles(const int ni[4], const int nj[4]) {
     T.first[w + 1] = T.first[w] + (ni[w] > 0 ? (unsigned)T.tx[w] * ((nj[w] + ST_H - 1) / ST_H) : 0u);
   }
   return T;
+}
+
+static ReduceArgs reduce_args(const Grid &g, const float *avg_hi, const NodeSet &n, double *scratch, unsigned *host,
+                              unsigned *ticket) {
+  ReduceArgs A;
+  A.g = g;
+  const int ni[4] = {g.nx, g.nxv, g.nxv, g.nx}, nj[4] = {g.ny, g.nyv, g.ny, g.nyv};
+  A.T = state_tiles(ni, nj);
+  A.pad[0] = avg_hi;
+  for (int k = 0; k < 3; k++) A.pad[1 + k] = n.k[k];
+  A.part = reinterpret_cast<unsigned *>(scratch);
+  A.ticket = ticket;
+  A.host = host;
+  A.speed = nullptr;
+  A.speed_bad = nullptr;
+  return A;
+}
+// (as many blocks as the scratch has room for three words of each)
+constexpr unsigned RED_BLOCKS = TOTALS_BLOCKS * NV * 2 / 3;
+cudaError_t launch_max_speed(const Grid &g, const float *avg_hi, const NodeSet &n, double *scratch, unsigned *out_bits,
+                             int *bad, unsigned *host, unsigned *ticket, cudaStream_t s) {
+  ReduceArgs A = reduce_args(g, avg_hi, n, scratch, host, ticket);
+  A.speed = out_bits;
+  A.speed_bad = bad;
+  const unsigned blocks = A.T.first[4] < RED_BLOCKS ? A.T.first[4] : RED_BLOCKS;
+  reduce_state_kernel<false><<<blocks, dim3(ST_W, ST_H / ST_ROWS), 0, s>>>(A);
+  return cudaGetLastError();
+}
+cudaError_t launch_state_min(const Grid &g, const float *avg_hi, const NodeSet &n, double *scratch, unsigned *host,
+                             unsigned *ticket, cudaStream_t s) {
+  const ReduceArgs A = reduce_args(g, avg_hi, n, scratch, host, ticket);
+  const unsigned blocks = A.T.first[4] < RED_BLOCKS ? A.T.first[4] : RED_BLOCKS;
+  reduce_state_kernel<true><<<blocks, dim3(ST_W, ST_H / ST_ROWS), 0, s>>>(A);
+  return cudaGetLastError();
+}
+cudaError_t launch_totals(const Grid &g, const float *avg_hi, const float *avg_lo, double *partials, double *host,
+                          unsigned *ticket, cudaStream_t s) {
+  totals_kernel<<<TOTALS_BLOCKS, TOTALS_BLOCKS, 0, s>>>(g, avg_hi, avg_lo, partials, ticket, host);
+  return cudaGetLastError();
+}
+cudaError_t launch_export_counters(const unsigned long long *c, unsigned long long *host, cudaStream_t s) {
+  export_counters_kernel<<<1, 32, 0, s>>>(c, host);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_check_state(const Grid &g, const float *const ext[4], unsigned *bad, unsigned *speed, int *speed_bad,
