@@ -841,39 +841,36 @@ static int enqueue_step(af_ctx *h, double dt) {
          "memset tiles");
       CK(launch_ubar(h->g, h->hi, h->lev[0], h->surr_ubar, s), "surrogate cell prep");
       const unsigned char *mask[3];
-      for (int k = 0; k < 3; k++) {
-        SurrogateArgs A;
-        A.g = h->g;
-        for (int q = 0; q < 3; q++) {
-          A.n0[q] = h->lev[0].k[q];
-          A.n1[q] = h->lev[1].k[q];
-          A.n2[q] = h->lev[2].k[q];
-        }
-        A.hi = h->hi;
-        A.ubar = h->surr_ubar;
-        A.dt = (float)dt;
-        A.tol = h->opt.surr_tol;
-        A.tol_abs = h->opt.surr_abs;
-        A.smooth = h->opt.surr_smooth;
-        af_mlp *net = h->surr[k == VTX ? 0 : 1];
-        A.wb = net->wb;
-        A.params = net->params;
-        A.mask = h->surr_mask + (size_t)k * h->g.plane;
-        mask[k] = A.mask;
-        A.tile_flag = h->surr_tiles;
-        A.tiles_x = h->surr_tiles_x;
-        A.tile_rows = tile_rows;
-        A.stats = h->surr_stats;
-        A.status = h->d_status;
-        A.test_no_issue = h->opt.test_timeout != 0;
-        A.wait_limit = h->opt.test_timeout ? kTestWaitLimit : kWaitLimit;
-        CK(launch_surrogate(k, A, h->sms, s), "surrogate");
+      SurrogateArgs A;
+      A.g = h->g;
+      for (int q = 0; q < 3; q++) {
+        A.n0[q] = h->lev[0].k[q];
+        A.n1[q] = h->lev[1].k[q];
+        A.n2[q] = h->lev[2].k[q];
+        mask[q] = A.mask[q] = h->surr_mask + (size_t)q * h->g.plane;
       }
+      for (int q = 0; q < 2; q++) {
+        A.wb[q] = h->surr[q]->wb;
+        A.params[q] = h->surr[q]->params;
+      }
+      A.ubar = h->surr_ubar;
+      A.dt = (float)dt;
+      A.tol = h->opt.surr_tol;
+      A.tol_abs = h->opt.surr_abs;
+      A.smooth = h->opt.surr_smooth;
+      A.tile_flag = h->surr_tiles;
+      A.tiles_x = h->surr_tiles_x;
+      A.tile_rows = tile_rows;
+      A.stats = h->surr_stats;
+      A.status = h->d_status;
+      A.test_no_issue = h->opt.test_timeout != 0;
+      A.wait_limit = h->opt.test_timeout ? kTestWaitLimit : kWaitLimit;
+      CK(launch_surrogate(A, h->sms, s), "surrogate");
       CK(launch_pointvalue_masked(h->g, h->lev[0], h->hi, maps, h->lev[1], h->lev[2], (float)dt,
                                   h->opt, h->d_status, counters, mask, h->surr_tiles, theta, tile, h->d_speed,
                                   h->d_speed_bad, s),
          "point values (fallback)");
-      h->launches[AF_STAGE_POINTVALUE] += 5;
+      h->launches[AF_STAGE_POINTVALUE] += 3;
       h->half_valid = true;
     } else if (!h->opt.node_flux) {
       // plain path: t^{n+1/2} and t^{n+1} written, the flux kernel forms the
@@ -1071,7 +1068,7 @@ int af_run(af_ctx *h, int nsteps, double dt) {
   for (int k = 0; k + 1 < nsteps; k += 2) {
     CK(cudaGraphLaunch(h->run_exec[p], h->stream), "af_run: graph launch");
     if (!flux_fills_ghosts(h->g)) h->launches[AF_STAGE_PREP] += 2;
-    h->launches[AF_STAGE_POINTVALUE] += h->opt.surrogate ? 10 : 2;
+    h->launches[AF_STAGE_POINTVALUE] += h->opt.surrogate ? 6 : 2;
     h->launches[AF_STAGE_FLUX] += 2;
   }
   h->speed_valid = true;

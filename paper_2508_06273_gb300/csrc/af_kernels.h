@@ -382,19 +382,18 @@ struct SampleBatch {
 };
 cudaError_t launch_sample_batch(const SampleBatch &B, const int4 *tiles, int ntiles, int tile_h, const BatchCtl *ctl,
                                 const PointValueArgs *args, cudaStream_t s);
-// fused inference of one node kind: network on the tensor cores, decode,
+// fused inference of the three node kinds: networks on the tensor cores, decode,
 // a-posteriori check; failing nodes get mask = 1 and their tile flagged
 struct SurrogateArgs {
   Grid g;
   const float *n0[3];
-  const float *hi;
   const float *ubar;  // primitive cell averages Ubar of cells -1 .. n (launch_ubar)
   float *n1[3], *n2[3];
   float dt, tol, tol_abs;
   float smooth;  // the network's values are used only where every scaled stencil range is <= smooth
-  const __nv_bfloat16 *wb;  // network weights (row-major, packed)
-  const float *params;      // FP32 parameters (biases, scales)
-  unsigned char *mask;      // this kind's fallback bytes
+  const __nv_bfloat16 *wb[2];  // weights (row-major, packed) of the vertices' and the edges' network
+  const float *params[2];      // FP32 parameters (biases, scales)
+  unsigned char *mask[3];      // fallback bytes by kind
   int *tile_flag;           // per point-value tile (32 x tile_rows)
   int tiles_x, tile_rows;
   unsigned long long *stats;  // [0] nodes from the network, [1] nodes sent to the exact operator
@@ -407,7 +406,7 @@ struct SurrogateArgs {
 cudaError_t prepare_surrogate();
 // Ubar of the cells -1 .. nx, -1 .. ny of the t^n state into ub (4 planes)
 cudaError_t launch_ubar(const Grid &g, const float *avg_hi, const NodeSet &n0, float *ub, cudaStream_t s);
-cudaError_t launch_surrogate(int kind, const SurrogateArgs &A, int sms, cudaStream_t s);
+cudaError_t launch_surrogate(const SurrogateArgs &A, int sms, cudaStream_t s);
 // point values of the single-grid kernel restricted to flagged nodes
 cudaError_t launch_pointvalue_masked(const Grid &g, const NodeSet &n0, const float *avg_hi, const TileMaps &maps,
                                      const NodeSet &n1, const NodeSet &n2, float dt, const Options &o, int *status,

@@ -124,5 +124,17 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, float v[32]) {
   for (int k = 0; k < 32; k++) v[k] = __uint_as_float(r[k]);
 }
 
+// the same of 8 columns
+__device__ __forceinline__ void tmem_ld8(unsigned taddr, float v[8]) {
+  unsigned r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int k = 0; k < 8; k++) v[k] = __uint_as_float(r[k]);
+}
+
 }  // namespace tc
 }  // namespace af
