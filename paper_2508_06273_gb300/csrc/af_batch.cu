@@ -42,7 +42,10 @@ struct af_batch {
   cudaStream_t own_stream = nullptr, stream = nullptr;
   std::vector<af_ctx *> inst;
   int tile_h = 0;  // tile height of every class, or 0: each class its own (TILE_OF_CLASS)
-  std::vector<BatchCtl> ctl_h;  // host mirror, current after sync_ctl
+  // host mirror of the control blocks: current after sync_ctl and until the next
+  // run; changes to it wait (ctl_dirty) for flush_ctl
+  std::vector<BatchCtl> ctl_h;
+  bool ctl_current = false, ctl_dirty = false;
   std::vector<char> has_state, speed_ok, stopped;
   BatchCtl *d_ctl = nullptr;
   PointValueArgs *d_pv = nullptr;  // [n][2]
@@ -102,9 +105,10 @@ void drop_graphs(af_batch *b) {
   b->graphs.clear();
 }
 
-// device control blocks -> host mirror; instance handles follow the buffer
-// that now holds each instance's t^n
+// device control blocks -> host mirror, unless it is current (no run since); the
+// instance handles follow the buffer that now holds each instance's t^n
 int sync_ctl(af_batch *b) {
+  if (b->ctl_current) return AF_OK;
   BCK(cudaStreamSynchronize(b->stream), "batch: sync");
   BCK(cudaMemcpy(b->ctl_h.data(), b->d_ctl, sizeof(BatchCtl) * b->n, cudaMemcpyDeviceToHost), "batch: ctl");
   for (int k = 0; k < b->n; k++) {
@@ -117,13 +121,19 @@ int sync_ctl(af_batch *b) {
     if (!c.active && (c.status & ST_STOPPED)) b->stopped[k] = 1;
     if (c.status & ST_TIMEOUT) b->timed_out = true;
   }
+  b->ctl_current = true;
+  b->ctl_dirty = false;
   return AF_OK;
 }
 
-int put_ctl(af_batch *b) {
+// the mirror, if it has changed, to the device before the next launch: once for
+// any number of changes
+int flush_ctl(af_batch *b) {
+  if (!b->ctl_dirty) return AF_OK;
   BCK(cudaMemcpyAsync(b->d_ctl, b->ctl_h.data(), sizeof(BatchCtl) * b->n, cudaMemcpyHostToDevice, b->stream),
       "batch: ctl");
   BCK(cudaStreamSynchronize(b->stream), "batch: sync");
+  b->ctl_dirty = false;
   return AF_OK;
 }
 
@@ -333,8 +343,23 @@ int graph_for(af_batch *b, int steps, double *hist, int hist_steps, cudaGraphExe
 }
 
 // wave speeds of instances whose state was just set (the flux kernel keeps
-// them current afterwards)
+// them current afterwards), and every pending change of the control blocks:
+// the speed came with the state's load, in host memory, or is computed here
 int ensure_speeds(af_batch *b) {
+  bool synced = false;
+  for (int k = 0; k < b->n; k++) {
+    const af_ctx *h = b->inst[k];
+    if (b->speed_ok[k] || !h->speed_valid || !h->speed_on_host) continue;
+    if (!synced) BCK(cudaStreamSynchronize(b->stream), "batch: sync");
+    synced = true;
+    const volatile unsigned *w = h->host_words;
+    b->ctl_h[k].speed = w[HW_SPEED];
+    b->ctl_h[k].speed_bad = (int)w[HW_SPEED + 1];
+    b->speed_ok[k] = 1;
+    b->ctl_dirty = true;
+  }
+  const int rc = flush_ctl(b);
+  if (rc) return rc;
   for (int k = 0; k < b->n; k++) {
     if (b->speed_ok[k]) continue;
     af_ctx *h = b->inst[k];
@@ -343,6 +368,7 @@ int ensure_speeds(af_batch *b) {
                          h->host_words_dev + HW_RESULT, h->d_ticket, b->stream),
         "batch: max speed");
     b->speed_ok[k] = 1;
+    b->ctl_current = false;
   }
   return AF_OK;
 }
@@ -399,6 +425,7 @@ af_batch *af_batch_create(int n, const int *nx, const int *ny, const double *dx,
     af_set_stream(b->inst[k], b->stream);
   }
   b->ctl_h.assign(n, BatchCtl());
+  b->ctl_current = true;
   b->has_state.assign(n, 0);
   b->speed_ok.assign(n, 0);
   b->stopped.assign(n, 0);
@@ -435,7 +462,8 @@ af_batch *af_batch_create(int n, const int *nx, const int *ny, const double *dx,
     free_batch(b);
     return nullptr;
   }
-  if (put_ctl(b) != AF_OK || upload_args(b) != AF_OK || build_tiles(b) != AF_OK) {
+  b->ctl_dirty = true;
+  if (upload_args(b) != AF_OK || build_tiles(b) != AF_OK) {
     free_batch(b);
     return nullptr;
   }
@@ -505,7 +533,8 @@ int af_batch_set_state(af_batch *b, int k, const float *avg, const float *vtx, c
   b->has_state[k] = 1;
   b->speed_ok[k] = 0;
   b->stopped[k] = 0;
-  return put_ctl(b);
+  b->ctl_dirty = true;
+  return AF_OK;
 }
 
 int af_batch_get_state(af_batch *b, int k, float *avg, float *vtx, float *xe, float *ye, void *stream) {
@@ -532,7 +561,8 @@ int af_batch_set_end(af_batch *b, const double *t_end, double cfl) {
     const bool before_end = std::isinf(c.t_end) ? c.t_end > 0 : (c.t_end - c.t) > 1e-12 * std::fabs(c.t_end);
     c.active = b->has_state[k] && !b->stopped[k] && before_end;
   }
-  return put_ctl(b);
+  b->ctl_dirty = true;
+  return AF_OK;
 }
 
 int af_batch_run(af_batch *b, int nsteps, double *hist, int hist_steps) {
@@ -549,6 +579,7 @@ int af_batch_run(af_batch *b, int nsteps, double *hist, int hist_steps) {
   if (rc) return rc;
   rc = ensure_speeds(b);
   if (rc) return rc;
+  b->ctl_current = false;
   int left = nsteps;
   while (left > 0) {
     const int steps = left > GRAPH_CHUNK ? GRAPH_CHUNK : left;
@@ -575,7 +606,7 @@ int af_batch_query(af_batch *b, double *t, int *steps, int *active, int *status)
   }
   if (status) {
     for (int k = 0; k < b->n; k++) b->ctl_h[k].status = 0;
-    return put_ctl(b);
+    b->ctl_dirty = true;
   }
   return AF_OK;
 }
@@ -646,13 +677,14 @@ int af_batch_autotune(af_batch *b, int *tile_h, double *ms) {
   cudaEventDestroy(e1);
   // the timed launches touched only scratch levels, status and counters
   b->ctl_h = saved;
+  b->ctl_current = b->ctl_dirty = true;
+  for (int k = 0; k < b->n; k++) b->speed_ok[k] = 0;  // recomputed at the next run
   if (rc) return rc;
   b->tile_h = best_h;
   rc = build_tiles(b);
   if (rc) return rc;
-  for (int k = 0; k < b->n; k++) b->speed_ok[k] = 0;  // recomputed at the next run
   if (tile_h) *tile_h = best_h;
-  return put_ctl(b);
+  return AF_OK;
 }
 
 int af_batch_set_sampler(af_batch *b, float *Xv, float *Tv, int *idv, int cap_v, float *Xe, float *Te, int *ide,
