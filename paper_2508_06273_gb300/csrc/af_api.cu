@@ -494,6 +494,45 @@ int af_set_state(af_ctx *h, const float *avg, const float *vtx, const float *xe,
   return rc;
 }
 
+// The four external arrays from host memory, each copied on a stream of its own
+// (not before the event `from`), then checked and loaded as it arrives; the last
+// load finishes the state's ghosts and hands over its wave speed (a ghost fill, a
+// reduction and a clear less a step; with each download's copy starting when its
+// array is packed, two steps of 1024^2 through host memory 2077 -> 1951 us, of
+// which 1878 are the bare copies and the steps).
+static int upload(af_ctx *h, const float *const src[4], cudaEvent_t from, int *d_bad) {
+  cudaStream_t s = h->stream;
+  h->speed_valid = h->ghost_valid = h->words_on_host = false;
+  for (int w = 0; w < 4; w++) {
+    int ni, nj;
+    extents(h, w, ni, nj);
+    CK(cudaStreamWaitEvent(h->xs[w], from, 0), "event");
+    CK(cudaMemcpyAsync(h->staging + h->staging_off[w], src[w], sizeof(float) * NV * ni * nj, cudaMemcpyHostToDevice,
+                       h->xs[w]),
+       "H2D");
+    CK(cudaEventRecord(h->xev[w], h->xs[w]), "event");
+  }
+  CK(cudaMemsetAsync(h->d_speed, 0, sizeof(unsigned), s), "memset speed");
+  CK(cudaMemsetAsync(h->d_speed_bad, 0, sizeof(int), s), "memset speed");
+  float *dst[4] = {h->hi, h->lev[0].k[VTX], h->lev[0].k[XE], h->lev[0].k[YE]};
+  for (int w = 0; w < 4; w++) {
+    int ni, nj;
+    extents(h, w, ni, nj);
+    const float *stg = h->staging + h->staging_off[w];
+    CK(cudaStreamWaitEvent(s, h->xev[w], 0), "event");
+    const int dup_x = h->g.per_x && (w == 1 || w == 2), dup_y = h->g.per_y && (w == 1 || w == 3);
+    if (dup_x || dup_y) CK(launch_check_dup(stg, ni, nj, dup_x, dup_y, d_bad, s), "check_dup");
+    StateArrays a = {};
+    a.ext[w] = stg;
+    a.pad[w] = dst[w];
+    CK(launch_load_state(h->g, a, h->lo, h->d_status, h->d_speed, h->d_speed_bad,
+                         w == 3 ? h->host_words_dev + HW_SPEED : nullptr, h->d_ticket, s),
+       "load");
+  }
+  h->speed_valid = h->speed_on_host = h->ghost_valid = true;
+  return AF_OK;
+}
+
 int af_set_state_host(af_ctx *h, const float *avg, const float *vtx, const float *xe,
                       const float *ye) {
   if (!h) return fail(AF_ERR_ARG, "null handle%s");
@@ -509,37 +548,16 @@ int af_set_state_host(af_ctx *h, const float *avg, const float *vtx, const float
   if (rc) return rc;
   cudaStream_t s = h->stream;
   const float *src[4] = {avg, vtx, xe, ye};
-  float *dst[4] = {h->hi, h->lev[0].k[VTX], h->lev[0].k[XE], h->lev[0].k[YE]};
   CK(cudaMemsetAsync(h->d_bad, 0, sizeof(int), s), "memset");
-  // the four copies run on their own streams once the handle's stream has
-  // reached this point; each array is checked and packed when it has arrived
+  // the copies run on their own streams once the handle's stream has reached this point
   CK(cudaEventRecord(h->xev[4], s), "event");
-  for (int w = 0; w < 4; w++) {
-    int ni, nj;
-    extents(h, w, ni, nj);
-    CK(cudaStreamWaitEvent(h->xs[w], h->xev[4], 0), "event");
-    CK(cudaMemcpyAsync(h->staging + h->staging_off[w], src[w], sizeof(float) * NV * ni * nj,
-                       cudaMemcpyHostToDevice, h->xs[w]),
-       "af_set_state_host: H2D");
-    CK(cudaEventRecord(h->xev[w], h->xs[w]), "event");
-  }
-  for (int w = 0; w < 4; w++) {
-    int ni, nj;
-    extents(h, w, ni, nj);
-    float *stg = h->staging + h->staging_off[w];
-    CK(cudaStreamWaitEvent(s, h->xev[w], 0), "event");
-    const int dup_x = h->g.per_x && (w == 1 || w == 2), dup_y = h->g.per_y && (w == 1 || w == 3);
-    if (dup_x || dup_y) CK(launch_check_dup(stg, ni, nj, dup_x, dup_y, h->d_bad, s), "check_dup");
-    CK(launch_pack(h->g, stg, dst[w], ni, nj, true, s), "pack");
-  }
+  rc = upload(h, src, h->xev[4], h->d_bad);
+  if (rc) return rc;
   int bad = 0;
   CK(cudaMemcpyAsync(&bad, h->d_bad, sizeof(int), cudaMemcpyDeviceToHost, s), "memcpy");
-  CK(cudaMemsetAsync(h->lo, 0, sizeof(float) * NV * h->g.plane, s), "memset lo");
-  CK(cudaMemsetAsync(h->d_status, 0, sizeof(int), s), "memset status");
-  h->words_on_host = false;
   CK(cudaStreamSynchronize(s), "sync");
   if (bad) {
-    h->has_state = false;
+    h->has_state = h->speed_valid = false;
     return fail(AF_ERR_ARG, "periodic state: the duplicated last node line differs from the first%s");
   }
   h->has_state = true;
@@ -668,34 +686,11 @@ int af_set_state_host_async(af_ctx *h, const float *avg, const float *vtx, const
   DeviceGuard dg(h->device);
   int rc = ensure_async(h);
   if (rc) return rc;
-  cudaStream_t s = h->stream;
   const float *src[4] = {avg, vtx, xe, ye};
-  float *dst[4] = {h->hi, h->lev[0].k[VTX], h->lev[0].k[XE], h->lev[0].k[YE]};
-  // each copy waits until the previous upload's unpack has read the staging
-  for (int w = 0; w < 4; w++) {
-    int ni, nj;
-    extents(h, w, ni, nj);
-    CK(cudaStreamWaitEvent(h->xs[w], h->in_free, 0), "event");
-    CK(cudaMemcpyAsync(h->staging + h->staging_off[w], src[w], sizeof(float) * NV * ni * nj,
-                       cudaMemcpyHostToDevice, h->xs[w]),
-       "af_set_state_host_async: H2D");
-    CK(cudaEventRecord(h->xev[w], h->xs[w]), "event");
-  }
-  for (int w = 0; w < 4; w++) {
-    int ni, nj;
-    extents(h, w, ni, nj);
-    float *stg = h->staging + h->staging_off[w];
-    CK(cudaStreamWaitEvent(s, h->xev[w], 0), "event");
-    const int dup_x = h->g.per_x && (w == 1 || w == 2), dup_y = h->g.per_y && (w == 1 || w == 3);
-    if (dup_x || dup_y) CK(launch_check_dup(stg, ni, nj, dup_x, dup_y, h->d_bad_async, s), "check_dup");
-    CK(launch_pack(h->g, stg, dst[w], ni, nj, true, s), "pack");
-  }
-  CK(cudaEventRecord(h->in_free, s), "event");
-  CK(cudaMemsetAsync(h->lo, 0, sizeof(float) * NV * h->g.plane, s), "memset lo");
-  CK(cudaMemsetAsync(h->d_status, 0, sizeof(int), s), "memset status");
-  h->words_on_host = false;
-  h->speed_valid = false;
-  h->ghost_valid = false;
+  // each copy waits until the previous upload's loads have read the staging
+  rc = upload(h, src, h->in_free, h->d_bad_async);
+  if (rc) return rc;
+  CK(cudaEventRecord(h->in_free, h->stream), "event");
   h->has_state = true;
   h->half_valid = false;
   h->async_pending = true;
@@ -717,15 +712,14 @@ int af_get_state_host_async(af_ctx *h, float *avg, float *vtx, float *xe, float 
   const int b = h->out_slot;
   float *stg = h->staging_out + (size_t)b * h->staging_off[4];
   for (int w = 0; w < 4; w++) CK(cudaStreamWaitEvent(s, h->out_done[b][w], 0), "event");
+  // (each array's copy starts when that array is packed)
   for (int w = 0; w < 4; w++) {
     int ni, nj;
     extents(h, w, ni, nj);
-    CK(launch_pack(h->g, src[w], stg + h->staging_off[w], ni, nj, false, s), "pack");
-  }
-  CK(cudaEventRecord(h->out_ready, s), "event");
-  for (int w = 0; w < 4; w++) {
-    int ni, nj;
-    extents(h, w, ni, nj);
+    float *ext[4] = {};
+    ext[w] = stg + h->staging_off[w];
+    CK(launch_store_state(h->g, src, ext, s), "pack");
+    CK(cudaEventRecord(h->out_ready, s), "event");
     CK(cudaStreamWaitEvent(h->xo[w], h->out_ready, 0), "event");
     CK(cudaMemcpyAsync(dst[w], stg + h->staging_off[w], sizeof(float) * NV * ni * nj, cudaMemcpyDeviceToHost,
                        h->xo[w]),

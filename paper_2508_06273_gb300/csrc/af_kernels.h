@@ -308,12 +308,13 @@ cudaError_t launch_totals(const Grid &g, const float *avg_hi, const float *avg_l
                           unsigned *ticket, cudaStream_t s);
 // a step's four event counters into host[4]
 cudaError_t launch_export_counters(const unsigned long long *c, unsigned long long *host, cudaStream_t s);
-// a state's four external arrays (averages, vertices, x-edges, y-edges; device
-// memory) into the padded planes in one launch: ghost entries included, low
-// words and *status cleared, and the state's max wave speed into *speed /
-// *speed_bad (cleared by the caller) and, by the last block, host_speed[0..1]
+// a state's external arrays (averages, vertices, x-edges, y-edges; device
+// memory) that are given into the padded planes in one launch: ghost entries
+// included, low words (with the averages) and *status cleared, and their max wave
+// speed into *speed / *speed_bad (cleared by the caller) and, if given, by the last
+// block into host_speed[0..1]
 struct StateArrays {
-  const float *ext[4];  // external (NULL: skipped by store_state)
+  const float *ext[4];  // external (NULL: left out)
   float *pad[4];        // averages hi, vertices, x-edges, y-edges
 };
 cudaError_t launch_load_state(const Grid &g, const StateArrays &a, float *avg_lo, int *status, unsigned *speed,

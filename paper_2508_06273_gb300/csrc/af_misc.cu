@@ -331,6 +331,7 @@ __global__ void __launch_bounds__(ST_W *ST_H / ST_ROWS) load_state_kernel(const 
     for (int k = 1; k < ST_H / ST_ROWS; k++) smax = fmaxf(smax, wmax[k]);
     atomicMax(A.speed, __float_as_uint(smax));
     if (anybad) atomicOr(A.speed_bad, 1);
+    if (!A.host_speed) return;  // (a launch after this one finishes the state)
     __threadfence();
     if (atomicAdd(A.ticket, 1u) == gridDim.x - 1) {
       __threadfence();
@@ -640,7 +641,7 @@ cudaError_t launch_load_state(const Grid &g, const StateArrays &a, float *avg_lo
   int ni[4], nj[4];
   for (int w = 0; w < 4; w++) {
     const GhostRange R(g, w == 0 ? 0 : w + 1);
-    ni[w] = R.hix + G;
+    ni[w] = a.ext[w] ? R.hix + G : 0;
     nj[w] = R.hiy + G;
     A.ext[w] = a.ext[w];
     A.pad[w] = a.pad[w];
