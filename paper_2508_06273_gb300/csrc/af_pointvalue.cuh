@@ -257,7 +257,7 @@ __device__ __forceinline__ void build_cell(const Grid &g, const float *raw, int 
 // registers): 3735 thread instructions a cell at 66 % of the issue slots.  The
 // earlier form took differences of all 9 coefficients of each cell on the
 // circle with two half tables and an arc table live together (4990
-// instructions).  Measured, point values, 4096^2 vortex moving / at rest
+// instructions).  Measured on 8-row tiles, 4096^2 vortex moving / at rest
 // (crossings at no / every vertex): 3.05 / 3.32 -> 2.37 / 2.53 ms; Alg. 1
 // linearisation at 2048^2 1.16 -> 0.85 ms.  80 or 96 registers (24 or 20 warps) spill to a local memory
 // that the L1 beside the shared memory cannot hold: 2.97 and 2.88 ms.

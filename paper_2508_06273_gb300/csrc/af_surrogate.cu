@@ -90,49 +90,45 @@ __device__ __forceinline__ void stencil(const Grid &g, const float *avg, const f
   }
 }
 
-// entry (i + a, j + b) of a plane relative to entry (i, j) of variable v (in
-// checking builds through at)
-__device__ __forceinline__ long long rel(const Grid &g, int v, int i, int j, int a, int b) {
-#ifdef AF_CHECK_BOUNDS
-  return at(g, v, i + a, j + b) - at(g, v, i, j);
-#else
-  return (long long)b * g.P + a;
-#endif
-}
-
-// variable v of the same stencil, with the cells' Ubar read from a precomputed array
+// the same stencil with the cells' Ubar read from a precomputed array
 template <int K>
-__device__ __forceinline__ void stencil_var(const Grid &g, const float *ub, const float *vtx, const float *xe,
-                                            const float *ye, int v, int i, int j, float W[]) {
-  const auto ld = [&](const float *p, int a, int b) { return __ldg(p + rel(g, v, i, j, a, b)); };
-  const long long o = at(g, v, i, j);
-  ub += o;
-  vtx += o;
+__device__ __forceinline__ void stencil_ub(const Grid &g, const float *ub, const float *vtx, const float *xe,
+                                           const float *ye, int i, int j, float W[][4]) {
   if (K == VTX) {
-    W[0] = ld(ub, -1, -1);
-    W[1] = ld(ub, 0, -1);
-    W[2] = ld(ub, -1, 0);
-    W[3] = ld(ub, 0, 0);
+    ld4g(g, ub, i - 1, j - 1, W[0]);
+    ld4g(g, ub, i, j - 1, W[1]);
+    ld4g(g, ub, i - 1, j, W[2]);
+    ld4g(g, ub, i, j, W[3]);
 #pragma unroll
     for (int b = -1; b <= 1; b++)
 #pragma unroll
-      for (int a = -1; a <= 1; a++) W[4 + 3 * (b + 1) + (a + 1)] = ld(vtx, a, b);
-  } else {
-    // one along (dx, dy) and across (ex, ey) the frame's first axis
-    constexpr int dx = K == XE ? 1 : 0, dy = 1 - dx, ex = dy, ey = dx;
-    const float *own = (K == XE ? xe : ye) + o, *other = (K == XE ? ye : xe) + o;
-    W[0] = ld(ub, -dx, -dy);
-    W[1] = ld(ub, 0, 0);
+      for (int a = -1; a <= 1; a++) ld4g(g, vtx, i + a, j + b, W[4 + 3 * (b + 1) + (a + 1)]);
+  } else if (K == XE) {
+    ld4g(g, ub, i - 1, j, W[0]);
+    ld4g(g, ub, i, j, W[1]);
 #pragma unroll
     for (int a = -1; a <= 1; a++) {
-      W[2 + a + 1] = ld(vtx, a * dx, a * dy);
-      W[5 + a + 1] = ld(vtx, a * dx + ex, a * dy + ey);
-      W[8 + a + 1] = ld(own, a * dx, a * dy);
+      ld4g(g, vtx, i + a, j, W[2 + a + 1]);
+      ld4g(g, vtx, i + a, j + 1, W[5 + a + 1]);
+      ld4g(g, xe, i + a, j, W[8 + a + 1]);
     }
-    W[11] = ld(other, -dx, -dy);
-    W[12] = ld(other, 0, 0);
-    W[13] = ld(other, ex - dx, ey - dy);
-    W[14] = ld(other, ex, ey);
+    ld4g(g, ye, i - 1, j, W[11]);
+    ld4g(g, ye, i, j, W[12]);
+    ld4g(g, ye, i - 1, j + 1, W[13]);
+    ld4g(g, ye, i, j + 1, W[14]);
+  } else {
+    ld4g(g, ub, i, j - 1, W[0]);
+    ld4g(g, ub, i, j, W[1]);
+#pragma unroll
+    for (int a = -1; a <= 1; a++) {
+      ld4g(g, vtx, i, j + a, W[2 + a + 1]);
+      ld4g(g, vtx, i + 1, j + a, W[5 + a + 1]);
+      ld4g(g, ye, i, j + a, W[8 + a + 1]);
+    }
+    ld4g(g, xe, i, j - 1, W[11]);
+    ld4g(g, xe, i, j, W[12]);
+    ld4g(g, xe, i + 1, j - 1, W[13]);
+    ld4g(g, xe, i + 1, j, W[14]);
   }
 }
 
@@ -250,20 +246,22 @@ __global__ void sample_batch_kernel(SampleBatch B, const int4 *tiles, const Batc
 }
 
 // ---------------------------------------------------------------- inference
-// One CTA per SM runs NG independent pipelines ("groups") of 8 warps.  A
-// group owns a tile of TM = 128 nodes at a time: its threads, two to a node,
-// build the nodes' features into the group's activation buffer (two frame slots
-// a thread), one thread issues the layer's MMAs into the group's 128
-// tensor-memory columns, and the group's threads apply bias and GELU to half of
-// their row and write the next layer's input back into the same buffer.  The four
-// groups (all that the activations and the accumulators leave room for) interleave
-// on the tensor core and hide one another's latency; the weights are shared in
-// shared memory.  The kernel is bound by the latency of a tile's chain of loads,
-// MMAs and epilogues at NG tiles an SM: two threads a node halve what each does in
-// turn.  One launch holds all three kinds: a block keeps the weights of one network
-// and walks that network's tiles, so that start-up and the last, partly filled
-// round come once instead of three times.  Four steps at 640^2: 1578 -> 1270 us,
-// with one thread a node and a launch a kind before.
+// One CTA per SM runs NG independent pipelines ("groups") of 4 warps.  A
+// group owns a tile of TM = 128 nodes at a time: its threads build the
+// nodes' features into the group's activation buffer, one thread issues
+// the layer's MMAs into the group's 128 tensor-memory columns, and the
+// group's threads apply bias and GELU to their row and write the next
+// layer's input back into the same buffer.  The four groups (all that the
+// activations and the accumulators leave room for) interleave on the tensor core
+// and hide one another's epilogue latency; the weights are shared in shared
+// memory.  One launch holds all three node kinds: a block keeps the weights of one
+// network and walks that network's tiles, so that start-up and the last, partly
+// filled round come once instead of three times.  While a layer's MMAs run, one
+// warp of the group polls and the others wait at its barrier.  Bound by the issue
+// and latency of features, GELU and decode.  us a step, a launch a kind before:
+// 128^2 108 -> 64, 320^2 227 -> 121, 640^2 393 -> 277, 1000^2 717 -> 605, 4096^2
+// 9394 -> 9298.  (Two threads a node, 64 registers, are slower: 297 at 640^2 and
+// 10247 at 4096^2, since both form the node's state and scales.)
 constexpr int TM = 128;  // nodes per tile (MMA M)
 constexpr int NG = 4;    // groups per CTA
 constexpr unsigned SZ_W1 = NH * NIN * 2, SZ_W2 = NH * NH * 2, SZ_W4 = NOUT_PAD * NH * 2;
@@ -307,85 +305,65 @@ __device__ __forceinline__ void gelu_row32(unsigned char *tile, int row, int cb,
         make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
 }
 
-// Element k of a row in BF16 into the pack w (8 elements) of a thread that
-// writes elements B .. E - 1 (both even): a whole pack goes to the tile as one
-// 16-byte store, a pack shared with the row's other thread as words.  (k is a
-// compile-time index in the unrolled callers.)
-template <int B, int E>
+// element k of a row in BF16 into the pack w (8 elements); at the 8th the
+// pack goes to the tile as one 16-byte store (k is a compile-time index in
+// the unrolled callers)
 __device__ __forceinline__ void pack_put(unsigned char *tile, int row, int k, float x, unsigned w[4]) {
   const unsigned b = __bfloat16_as_ushort(__float2bfloat16_rn(x));
-  const int e = k & 7, k0 = k - e;
+  const int e = k & 7;
   if (e & 1) w[e >> 1] |= b << 16;
   else w[e >> 1] = b;
-  if (e != 7 && k != E - 1) return;
-  unsigned char *p = tile + tc::chunk_offset(TM, row, k0);
-  if (k0 >= B && k0 + 8 <= E) {
-    *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; q++)
-      if (k0 + 2 * q >= B && k0 + 2 * q < E) *reinterpret_cast<unsigned *>(p + 4 * q) = w[q];
-  }
+  if (e == 7)
+    *reinterpret_cast<uint4 *>(tile + tc::chunk_offset(TM, row, k - 7)) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// what a thread needs of its node beyond the features: its two slots' scales,
-// the ranges of their scaled stencils and their scaled own values, for the check
-struct SlotCheck {
-  float s[2], lo[2], hi[2], self[2];
-};
-
-// The features of node (K, i, j) times the input scales, as row `row` of the
-// group's buffer (K = 64): frame slots 2 H and 2 H + 1, and for H = 1 what
-// follows them.
-template <int K, int H>
+// the features of node (K, i, j) times the input scales, as row `row` of the
+// group's buffer (K = 64); u~ and the scales, and per frame slot the range of
+// the scaled stencil and the scaled own value, for the check
+template <int K>
 __device__ __forceinline__ void features_to_row(const Grid &g, const float *ub, const float *vtx, const float *xe,
                                                 const float *ye, int i, int j, float dt, const float *ins,
-                                                unsigned char *buf, int row, SlotCheck &C) {
+                                                unsigned char *buf, int row, float s[4], float lo[4], float hi[4],
+                                                float self[4]) {
   using St = Stencil<K>;
-  constexpr int B = H == 0 ? 0 : 2 * St::N, E = H == 0 ? 2 * St::N : 64;
-  constexpr int dx = K == YE ? 0 : 1, dy = K == XE ? 0 : 1;
+  float W[St::N][4];
+  stencil_ub<K>(g, ub, vtx, xe, ye, i, j, W);
   float ut[4];
 #pragma unroll
   for (int v = 0; v < NV; v++) {
     float a = 0.0f;
-    const float *u = ub + at(g, v, i, j);
-    a += __ldg(u + rel(g, v, i, j, -dx, -dy));
-    if (K == VTX) {
-      a += __ldg(u + rel(g, v, i, j, 0, -1));
-      a += __ldg(u + rel(g, v, i, j, -1, 0));
-    }
-    a += __ldg(u);
+#pragma unroll
+    for (int c = 0; c < St::NC; c++) a += W[c][v];
     ut[v] = a * (1.0f / St::NC);
   }
   const float c = sqrtf(g.gamma * ut[3] / ut[0]);
+  s[0] = ut[0];
+  s[1] = s[2] = c;
+  s[3] = ut[0] * c * c;
   unsigned w[4];
 #pragma unroll
-  for (int h = 0; h < 2; h++) {
-    const int q = 2 * H + h, v = var_of_slot<K>(q);
-    const float s = v == 0 ? ut[0] : (v == 3 ? ut[0] * c * c : c), is = 1.0f / s;
-    float W[St::N];
-    stencil_var<K>(g, ub, vtx, xe, ye, v, i, j, W);
+  for (int q = 0; q < NV; q++) {
+    const int v = var_of_slot<K>(q);
+    const float is = 1.0f / s[v];
     float mn = 3.0e38f, mx = -3.0e38f;
 #pragma unroll
     for (int m = 0; m < St::N; m++) {
-      const float x = (W[m] - ut[v]) * is;
-      pack_put<B, E>(buf, row, q * St::N + m, x * ins[q * St::N + m], w);
+      const float x = (W[m][v] - ut[v]) * is;
+      pack_put(buf, row, q * St::N + m, x * ins[q * St::N + m], w);
       mn = fminf(mn, x);
       mx = fmaxf(mx, x);
-      if (m == St::SELF) C.self[h] = x;
+      if (m == St::SELF) self[q] = x;
     }
-    C.s[h] = s;
-    C.lo[h] = mn;
-    C.hi[h] = mx;
+    lo[q] = mn;
+    hi[q] = mx;
   }
-  if (H == 0) return;
   const float r = dt * g.idx;
   constexpr int k0 = 4 * St::N;
-  pack_put<B, E>(buf, row, k0, c * r * ins[k0], w);
-  pack_put<B, E>(buf, row, k0 + 1, ut[var_of_slot<K>(1)] * r * ins[k0 + 1], w);
-  pack_put<B, E>(buf, row, k0 + 2, ut[var_of_slot<K>(2)] * r * ins[k0 + 2], w);
+  pack_put(buf, row, k0, c * r * ins[k0], w);
+  pack_put(buf, row, k0 + 1, ut[var_of_slot<K>(1)] * r * ins[k0 + 1], w);
+  pack_put(buf, row, k0 + 2, ut[var_of_slot<K>(2)] * r * ins[k0 + 2], w);
 #pragma unroll
-  for (int k = k0 + 3; k < 64; k++) pack_put<B, E>(buf, row, k, 0.0f, w);
+  for (int k = k0 + 3; k < 64; k++) pack_put(buf, row, k, 0.0f, w);
 }
 
 // D = A (TM x Kd, at a_s) * W^T (N x Kd, at w_s): one elected thread
@@ -401,137 +379,125 @@ __device__ __forceinline__ void issue_layer(unsigned tmem, unsigned a_s, unsigne
   tc::mma_commit(bar);
 }
 
-// barrier of the 2 TM threads of group grp (ids 1..NG; 0 is __syncthreads)
+__device__ __forceinline__ void st4g(const Grid &g, float *p, int i, int j, const float U[4]) {
+#pragma unroll
+  for (int v = 0; v < NV; v++) p[at(g, v, i, j)] = U[v];
+}
+
+// barrier of the 128 threads of group grp (ids 1..NG; 0 is __syncthreads)
 __device__ __forceinline__ void group_sync(int grp) {
-  asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(2 * TM) : "memory");
+  asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(TM) : "memory");
 }
 
 // what a thread is and shares with its group
 struct Group {
-  int grp, row, half;
-  unsigned char *buf, *smem;  // activations; weights
+  int grp, row;
+  unsigned char *buf, *smem;
   const float *bias;
-  unsigned tcol, tld;  // the group's accumulator; this warp's lanes of it
+  unsigned tcol, tld;
   unsigned long long *bar;
   unsigned phase;
   int *fail;
-  unsigned char *good;  // [2][TM]
   unsigned n_fall, n_net;
 };
-
 // one tile of nodes of kind K; false: the wait for the tensor cores ran out
 template <int K>
 __device__ __forceinline__ bool surrogate_tile(const SurrogateArgs &A, Group &G, unsigned tile, unsigned total, unsigned ni) {
   const Grid &g = A.g;
+  const int row = G.row, grp = G.grp;
+  unsigned char *buf = G.buf;
   const float *b4 = G.bias + 3 * NH, *ins = b4 + NOUT_PAD, *outs = ins + NIN;
-  const unsigned lin = tile * TM + G.row;
+  const unsigned lin = tile * TM + row;
   const bool valid = lin < total;
   const int i = valid ? (int)(lin % ni) : 0, j = valid ? (int)(lin / ni) : 0;
-  const float *vtx = A.n0[VTX], *xe = A.n0[XE], *ye = A.n0[YE];
-  SlotCheck C = {};
-  if (!valid) {
-    for (int k = 32 * G.half; k < 32 * G.half + 32; k += 8)
-      *reinterpret_cast<uint4 *>(G.buf + tc::chunk_offset(TM, G.row, k)) = make_uint4(0, 0, 0, 0);
-  } else if (G.half == 0) {
-    features_to_row<K, 0>(g, A.ubar, vtx, xe, ye, i, j, A.dt, ins, G.buf, G.row, C);
+  float s[4] = {1, 1, 1, 1}, lo[4], hi[4], self[4];
+  if (valid) {
+    features_to_row<K>(g, A.ubar, A.n0[VTX], A.n0[XE], A.n0[YE], i, j, A.dt, ins, buf, row, s, lo, hi, self);
   } else {
-    features_to_row<K, 1>(g, A.ubar, vtx, xe, ye, i, j, A.dt, ins, G.buf, G.row, C);
+    for (int k = 0; k < 64; k += 8) *reinterpret_cast<uint4 *>(buf + tc::chunk_offset(TM, row, k)) = make_uint4(0, 0, 0, 0);
   }
   // layers 1..3: H = gelu(in W^T + b) back into the buffer; layer 4: y = H W4^T + b4
   int Kd = NIN;
   for (int l = 0; l < 4; l++) {
     tc::fence_async_smem();
     tc::fence_before_sync();
-    group_sync(G.grp);
-    if (G.row == 0 && G.half == 0) {
+    group_sync(grp);
+    if (row == 0) {
       tc::fence_after_sync();
       const unsigned char *w = G.smem + (l == 0 ? O_W1 : (l == 1 ? O_W2 : (l == 2 ? O_W3 : O_W4)));
-      if (!A.test_no_issue) issue_layer(G.tcol, tc::smem_u32(G.buf), tc::smem_u32(w), Kd, l < 3 ? NH : NOUT_PAD, G.bar);
+      if (!A.test_no_issue) issue_layer(G.tcol, tc::smem_u32(buf), tc::smem_u32(w), Kd, l < 3 ? NH : NOUT_PAD, G.bar);
     }
-    if (!tc::bar_wait(G.bar, G.phase, A.wait_limit)) *G.fail = 1;
+    if (row < 32 && !tc::bar_wait(G.bar, G.phase, A.wait_limit)) *G.fail = 1;
     G.phase ^= 1;
-    group_sync(G.grp);
+    group_sync(grp);
     if (*G.fail) return false;
     tc::fence_after_sync();
     if (l < 3) {
       const float *bl = G.bias + l * NH;
 #pragma unroll 1
-      for (int cb = 64 * G.half; cb < 64 * G.half + 64; cb += 32) {
+      for (int cb = 0; cb < NH; cb += 32) {
         float v[32];
         tc::tmem_ld32(G.tld + cb, v);
-        gelu_row32(G.buf, G.row, cb, v, bl + cb);
+        gelu_row32(buf, row, cb, v, bl + cb);
       }
       Kd = NH;
     }
   }
   float y[8];
   tc::tmem_ld8(G.tld, y);
-  // decode, check (admissible, inside the stencil's range widened by tol
-  // times its width plus tol_abs, finite, a stencil no wider than smooth),
-  // store or flag for the exact operator; each thread its two slots
-  float Un[2][2];
-  bool good = true;
-#pragma unroll
-  for (int h = 0; h < 2; h++) {
-    const int q = 2 * G.half + h, v = var_of_slot<K>(q);
-    const float U0 = __ldg(A.n0[K] + at(g, v, i, j));
-    const float w = A.tol * (C.hi[h] - C.lo[h]) + A.tol_abs;
-    good = good && (C.hi[h] - C.lo[h] <= A.smooth);
+  if (valid) {
+    // decode, check (admissible, inside the stencil's range widened by tol
+    // times its width plus tol_abs, finite, a stencil no wider than smooth),
+    // store or flag for the exact operator
+    bool good = true;
+    float Un[2][4];
+    float U0[4];
+    ld4g(g, A.n0[K], i, j, U0);
 #pragma unroll
     for (int lev = 0; lev < 2; lev++) {
-      const float d = ((G.half ? y[4 * lev + 2 + h] : y[4 * lev + h]) + b4[4 * lev + q]) * outs[4 * lev + q];
-      const float x = C.self[h] + d;
-      const float U = U0 + C.s[h] * d;
-      good = good && (x >= C.lo[h] - w) && (x <= C.hi[h] + w) && ((v == 0 || v == 3) ? U > 0.0f : isfinite(U));
-      Un[lev][h] = U;
+#pragma unroll
+      for (int q = 0; q < NV; q++) {
+        const int v = var_of_slot<K>(q);
+        const float d = (y[4 * lev + q] + b4[4 * lev + q]) * outs[4 * lev + q];
+        const float x = self[q] + d, w = A.tol * (hi[q] - lo[q]) + A.tol_abs;
+        good = good && (x >= lo[q] - w) && (x <= hi[q] + w) && (hi[q] - lo[q] <= A.smooth);
+        Un[lev][v] = U0[v] + s[v] * d;
+      }
+      good = good && Un[lev][0] > 0.0f && Un[lev][3] > 0.0f && isfinite(Un[lev][1]) && isfinite(Un[lev][2]);
     }
-  }
-  G.good[G.half * TM + G.row] = good;
-  group_sync(G.grp);
-  good = G.good[G.row] && G.good[TM + G.row];
-  if (!valid) return true;
-  if (G.half == 0) {
     const long long mi = (long long)(j + OY) * g.P + (i + OX);
     A.mask[K][mi] = good ? 0 : 1;
     if (good) {
       G.n_net++;
+#pragma unroll
+      for (int lev = 0; lev < 2; lev++) {
+        float *dst = lev == 0 ? A.n1[K] : A.n2[K];
+        st4g(g, dst, i, j, Un[lev]);
+        const bool dx_ = (K != YE) && g.per_x && i == 0, dy_ = (K != XE) && g.per_y && j == 0;
+        if (dx_) st4g(g, dst, g.nx, j, Un[lev]);
+        if (dy_) st4g(g, dst, i, g.ny, Un[lev]);
+        if (dx_ && dy_) st4g(g, dst, g.nx, g.ny, Un[lev]);
+      }
     } else {
       G.n_fall++;
       A.tile_flag[(j / A.tile_rows) * A.tiles_x + i / 32] = 1;
     }
   }
-  if (good) {
-    const bool dx_ = (K != YE) && g.per_x && i == 0, dy_ = (K != XE) && g.per_y && j == 0;
-#pragma unroll
-    for (int lev = 0; lev < 2; lev++)
-#pragma unroll
-      for (int h = 0; h < 2; h++) {
-        const int v = var_of_slot<K>(2 * G.half + h);
-        float *dst = lev == 0 ? A.n1[K] : A.n2[K];
-        const float U = Un[lev][h];
-        dst[at(g, v, i, j)] = U;
-        if (dx_) dst[at(g, v, g.nx, j)] = U;
-        if (dy_) dst[at(g, v, i, g.ny)] = U;
-        if (dx_ && dy_) dst[at(g, v, g.nx, g.ny)] = U;
-      }
-  }
   return true;
 }
 
 // blocks 0 .. nb_v - 1 evaluate the vertices' network, the others the edges'
-__global__ void __launch_bounds__(2 * NG *TM, 1) surrogate_kernel(const __grid_constant__ SurrogateArgs A, int nb_v) {
+__global__ void __launch_bounds__(NG *TM, 1) surrogate_kernel(const __grid_constant__ SurrogateArgs A, int nb_v) {
   extern __shared__ __align__(128) unsigned char ssm[];
   __shared__ alignas(8) unsigned long long bars[NG];
   __shared__ unsigned tslot;
   __shared__ int gfail[NG];
-  __shared__ unsigned char sgood[NG][2 * TM];
   const Grid &g = A.g;
   const int tid = threadIdx.x, warp = tid >> 5;
   const bool vert = (int)blockIdx.x < nb_v;
   Group G;
-  G.grp = warp >> 3;
+  G.grp = warp >> 2;
   G.row = tid & (TM - 1);
-  G.half = (warp >> 2) & 1;
   G.smem = ssm;
   G.buf = ssm + O_BUF + G.grp * SZ_BUF;
   float *bias = reinterpret_cast<float *>(ssm + O_B);
@@ -564,7 +530,6 @@ __global__ void __launch_bounds__(2 * NG *TM, 1) surrogate_kernel(const __grid_c
   G.bar = &bars[G.grp];
   G.phase = 0;
   G.fail = &gfail[G.grp];
-  G.good = sgood[G.grp];
   G.n_fall = G.n_net = 0;
 
   bool ok = true;
@@ -586,7 +551,7 @@ __global__ void __launch_bounds__(2 * NG *TM, 1) surrogate_kernel(const __grid_c
     // memory is released, and stop this group; if even that runs out, the
     // group goes on with an MMA unfinished.  Under the test hook no MMA was
     // issued and nothing is in flight.
-    if (G.row == 0 && G.half == 0) atomicOr(A.status, ST_TIMEOUT);
+    if (G.row == 0) atomicOr(A.status, ST_TIMEOUT);
     if (!A.test_no_issue) tc::bar_wait(G.bar, G.phase ^ 1, kDrainFactor * A.wait_limit);
   }
   if (G.n_net) atomicAdd(A.stats, (unsigned long long)G.n_net);
@@ -618,7 +583,7 @@ cudaError_t launch_surrogate(const SurrogateArgs &A, int sms, cudaStream_t s) {
     }
     if (best < 0) nb_v = 1;
   }
-  surrogate_kernel<<<nb, 2 * NG * TM, SURR_SMEM, s>>>(A, nb_v);
+  surrogate_kernel<<<nb, NG * TM, SURR_SMEM, s>>>(A, nb_v);
   return cudaGetLastError();
 }
 
