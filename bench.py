@@ -31,19 +31,12 @@ if ROOT not in sys.path:
 METRIC = "cell updates/s (FP32 plain vs MLP-surrogate+fallback) at stated L1 error vs FP64 oracle"
 UNIT = "cell updates/s"
 SEED = 2508
-# FP32 operations of the point-value stage per cell update, counted from the
-# kernel source (add, sub, mul = 1, fma = 2; sqrt, div and transcendental
-# calls not counted) for this workload's background state (u = v = 1,
-# c = 1.18: both grid lines cross every Mach circle, the node lies outside
-# it, so X and Y do not meet): a vertex (3 cells' circle coefficients, two
-# half-circle tables: 1057) and two edge midpoints (2 cells, one half-circle
-# table: 670 each) at two time levels, plus the correction term, the
-# linearisation state and the fused cell prep (809): 5.6 k.  Vortex-core
-# vertices, whose circles also need the quarter arc, do 472 more.  The FP32
-# operations the kernel executes on this workload (ncu: fadd + fmul + 2 ffma)
-# are 5.55 k a cell update, 1% under the count (the compiler folds some of
-# what it counts): the achieved figure takes 5.5 k, below both.
-PV_FLOP_PER_CELL = 5500
+# FP32 operations of the point-value stage per cell update (add and multiply 1,
+# fused multiply-add 2; sqrt, div and transcendental calls not counted) on this
+# workload: a lower count of what the kernel executes, from an unpacked build on
+# 8-row tiles (444 adds + 775 multiplies + 2 x 1300 fused).  On 4-row tiles ncu
+# counts 592 + 599 + 2 x 894 and 609 packed pairs of 2 to 4 operations each.
+PV_FLOP_PER_CELL = 3800
 # algorithmic HBM bytes of the flux/update kernel per cell: 3 levels x 3 node
 # arrays read (144 B), averages hi/lo read and written (64 B)
 FLUX_BYTES_PER_CELL = 208
@@ -54,13 +47,13 @@ FLUX_BYTES_PER_CELL = 208
 # code; af_kernels.h, which declares every kernel's launcher, is left out);
 # otherwise reported as null
 _KSRC = "paper_2508_06273_gb300/csrc/"
-_SHARED = {_KSRC + "af_common.cuh": "093115c23be2e775d5d20529727a61310b8bf8c4402d8e1bf8500c33560da0aa"}
-PV_TRAFFIC = {"bytes_per_cell": 150.8, "profile": "profiles/dram_pointvalue_flux_vortex2048.md",
-              "sha256": dict(_SHARED, **{_KSRC + "af_pointvalue.cu":
-                                         "5dd8c49de21a3549206c6886e2b4104ff62e4ac106776ebf97ec4a8a3fad0121"})}
-FLUX_TRAFFIC = {"bytes_per_cell": 206.6, "profile": "profiles/dram_pointvalue_flux_vortex2048.md",
+_SHARED = {_KSRC + "af_common.cuh": "fd53e25857ed1f9f388ae6489430731b510ae23d1d4c043f95a91350602f1ea5"}
+PV_TRAFFIC = {"bytes_per_cell": 150.3, "profile": "profiles/dram_pointvalue_flux_vortex2048.md",
+              "sha256": dict(_SHARED, **{_KSRC + "af_pointvalue.cuh":
+                                         "2c87d5436ac3773f055c55e82a5fae09eb613569a268450ecc41885e26466e79"})}
+FLUX_TRAFFIC = {"bytes_per_cell": 207.6, "profile": "profiles/dram_pointvalue_flux_vortex2048.md",
                 "sha256": dict(_SHARED, **{_KSRC + "af_flux.cu":
-                                           "164c4a83daa94e5a5764bed37528724938990583775d6600124f0663476ded73"})}
+                                           "e26794e770f53a59bab9bc4c08a144d0145a59a7918553fece7608ed149bad43"})}
 
 
 def measured_traffic(spec, cells):
