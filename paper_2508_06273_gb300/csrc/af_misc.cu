@@ -273,7 +273,8 @@ __global__ void __launch_bounds__(ST_W *ST_H / ST_ROWS) load_state_kernel(const 
   const int arr = w == 0 ? 0 : w + 1;  // as in GhostRange (1: the low words)
   const GhostRange R(g, arr);
   const int ni = g.nx + R.nodex, nj = g.ny + R.nodey;
-  const int i = i0 - G + (int)threadIdx.x;
+  const int i = i0 - OX + (int)threadIdx.x;  // (so that a warp's stores fill aligned lines)
+  const bool ion = i >= -G && i < R.hix;
   float smax = 0.0f;
   bool bad = false;
   if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *A.status = 0;
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(ST_W *ST_H / ST_ROWS) load_state_kernel(const 
     const int j = j0 - G + (int)threadIdx.y + r * (ST_H / ST_ROWS);
     bool fx = false, fy = false;
     // (threads beyond the padded extents read an interior point and store nothing)
-    const int si = i < R.hix ? ghost_src(i, g.nx, R.ownx, R.nodex, g.per_x, g.bc[0], g.bc[1], fx) : 0;
+    const int si = ion ? ghost_src(i, g.nx, R.ownx, R.nodex, g.per_x, g.bc[0], g.bc[1], fx) : 0;
     const int sj = j < R.hiy ? ghost_src(j, g.ny, R.owny, R.nodey, g.per_y, g.bc[2], g.bc[3], fy) : 0;
     const float *src = A.ext[w] + (long long)sj * ni + si;
 #pragma unroll
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(ST_W *ST_H / ST_ROWS) load_state_kernel(const 
 #pragma unroll
   for (int r = 0; r < ST_ROWS; r++) {
     const int j = j0 - G + (int)threadIdx.y + r * (ST_H / ST_ROWS);
-    if (i >= R.hix || j >= R.hiy) continue;
+    if (!ion || j >= R.hiy) continue;
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       const long long e = at(g, v, i, j);
@@ -331,7 +332,7 @@ __global__ void __launch_bounds__(ST_W *ST_H / ST_ROWS) load_state_kernel(const 
     for (int k = 1; k < ST_H / ST_ROWS; k++) smax = fmaxf(smax, wmax[k]);
     atomicMax(A.speed, __float_as_uint(smax));
     if (anybad) atomicOr(A.speed_bad, 1);
-    if (!A.host_speed) return;  // (a launch after this one finishes the state)
+    if (!A.host_speed) return;
     __threadfence();
     if (atomicAdd(A.ticket, 1u) == gridDim.x - 1) {
       __threadfence();
@@ -641,7 +642,7 @@ cudaError_t launch_load_state(const Grid &g, const StateArrays &a, float *avg_lo
   int ni[4], nj[4];
   for (int w = 0; w < 4; w++) {
     const GhostRange R(g, w == 0 ? 0 : w + 1);
-    ni[w] = a.ext[w] ? R.hix + G : 0;
+    ni[w] = a.ext[w] ? R.hix + OX : 0;
     nj[w] = R.hiy + G;
     A.ext[w] = a.ext[w];
     A.pad[w] = a.pad[w];
