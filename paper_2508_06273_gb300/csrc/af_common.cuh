@@ -80,7 +80,12 @@ __host__ __device__ __forceinline__ long long at(const Grid &g, int v, int i, in
 // while the one before it in the stream is still finishing.  pdl_start lets the
 // next kernel begin (its blocks take slots that the last ones of this kernel
 // leave free); pdl_wait holds a kernel until the one before it has ended and its
-// writes are visible, and stands before every access to global memory.
+// writes are visible, and stands before every access to global memory.  A kernel
+// that waits so is alive while the launches before it still write, several of them
+// where each begins early, so that what they write is not constant during its
+// lifetime: it is read with plain loads, which pdl_wait orders, and never through
+// __ldg, whose promise of constant memory lets the compiler move a load up over
+// the wait and the hardware serve it from lines cached before.
 __device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... P, typename... A>

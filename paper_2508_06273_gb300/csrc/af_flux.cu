@@ -74,7 +74,7 @@ __device__ __forceinline__ void time_flux(const Args &A, int kind, int i, int j,
   for (int l = 0; l < 3; l++) {
     float U[4];
 #pragma unroll
-    for (int v = 0; v < NV; v++) U[v] = __ldg(A.n[l][kind] + at(A.g, v, i, j));
+    for (int v = 0; v < NV; v++) U[v] = A.n[l][kind][at(A.g, v, i, j)];
     add_time_flux(U, gm1i, dir, l == 1 ? 4.0f : 1.0f, F);
     if (l == 2 && fold) smax = fmaxf(smax, wave_speed(U, A.g.gamma, bad));
   }
@@ -87,7 +87,7 @@ __device__ __forceinline__ void time_flux_fg(const Args &A, int i, int j, float 
 #pragma unroll
   for (int l = 0; l < 3; l++)
 #pragma unroll
-    for (int v = 0; v < NV; v++) U[l][v] = __ldg(A.n[l][VTX] + at(A.g, v, i, j));
+    for (int v = 0; v < NV; v++) U[l][v] = A.n[l][VTX][at(A.g, v, i, j)];
 #pragma unroll
   for (int v = 0; v < NV; v++) F[v] = G[v] = 0.0f;
 #pragma unroll
@@ -256,7 +256,7 @@ __device__ __noinline__ void limit_tile(const Args &A, FluxSmem &S, LimSmem &L, 
 // y-edges)
 __device__ __forceinline__ void ld_nf(const Args &A, int q, int i, int j, float F[4]) {
 #pragma unroll
-  for (int v = 0; v < NV; v++) F[v] = __ldg(A.nf[q] + at(A.g, v, i, j));
+  for (int v = 0; v < NV; v++) F[v] = A.nf[q][at(A.g, v, i, j)];
 }
 
 // the new (hi, lo) averages of a cell next to a side into its ghost images, by

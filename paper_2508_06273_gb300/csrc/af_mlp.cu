@@ -417,13 +417,19 @@ struct WgradArgs {
 // rows [0, R) (zero from `rows` on) of a row-major R x B array, columns k0 ..
 // k0 + 255 (zero from B on), into the K-major core layout of R rows
 __device__ __forceinline__ void load_step(unsigned char *dst, const __nv_bfloat16 *X, int rows, int R, int B, int k0) {
-#pragma unroll 16
-  for (int idx = threadIdx.x; idx < R * (WG_STEP / 8); idx += WG_THREADS) {
-    const int r = (idx & 7) + 8 * (idx / WG_STEP), kv = (idx >> 3) % (WG_STEP / 8), k = k0 + 8 * kv;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (r < rows && k < B) v = __ldg(reinterpret_cast<const uint4 *>(X + (long long)r * B + k));
-    *reinterpret_cast<uint4 *>(dst + tc::chunk_offset(R, r, 8 * kv)) = v;
+  static_assert(WG_THREADS == WG_STEP && NH % 8 == 0, "8 rows of WG_STEP / 8 pieces a round");
+  const int r0 = threadIdx.x & 7, kv = threadIdx.x >> 3, k = k0 + 8 * kv;
+  // (the loads first: plain ones, of the launch before, do not pass the stores)
+  uint4 v[NH / 8];
+#pragma unroll
+  for (int q = 0; q < NH / 8; q++) {
+    const int r = r0 + 8 * q;
+    v[q] = make_uint4(0u, 0u, 0u, 0u);
+    if (r < rows && k < B) v[q] = *reinterpret_cast<const uint4 *>(X + (long long)r * B + k);
   }
+#pragma unroll
+  for (int q = 0; q < NH / 8; q++)
+    if (8 * q < R) *reinterpret_cast<uint4 *>(dst + tc::chunk_offset(R, r0 + 8 * q, 8 * kv)) = v[q];
 }
 __global__ void __launch_bounds__(WG_THREADS, 1) weight_grad_kernel(WgradArgs a) {
   extern __shared__ __align__(128) unsigned char wsm[];
@@ -502,7 +508,7 @@ __device__ __forceinline__ float gradient(const Partials &P, int k) {
   for (int q0 = 0; q0 < n; q0 += 32) {
     float x[32];
 #pragma unroll
-    for (int q = 0; q < 32; q++) x[q] = q0 + q < n ? __ldg(p + (long long)(q0 + q) * stride) : 0.0f;
+    for (int q = 0; q < 32; q++) x[q] = q0 + q < n ? p[(long long)(q0 + q) * stride] : 0.0f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll

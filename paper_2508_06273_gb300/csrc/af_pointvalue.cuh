@@ -116,7 +116,7 @@ __device__ __forceinline__ void raw4(const float *raw, int arr, int i, int j, in
 }
 
 __device__ __forceinline__ float ld(const Args &A, const float *p, int v, int i, int j) {
-  return __ldg(p + at(A.g, v, i, j));
+  return p[at(A.g, v, i, j)];
 }
 __device__ __forceinline__ void ld4(const Args &A, const float *p, int i, int j, float U[4]) {
 #pragma unroll
@@ -1056,11 +1056,11 @@ __device__ __forceinline__ void node_update(const Args &A, const float *sm, cons
   // Sec. 3.4 blend weight (the same for both levels; from the t^n averages)
   float th = 1.0f;
   if (SHOCK && A.theta[0]) {
-    if (K == XE) th = __ldg(A.theta[0] + at(g, 0, i, j));
-    else if (K == YE) th = __ldg(A.theta[1] + at(g, 0, i, j));
+    if (K == XE) th = A.theta[0][at(g, 0, i, j)];
+    else if (K == YE) th = A.theta[1][at(g, 0, i, j)];
     else
-      th = fminf(fminf(__ldg(A.theta[0] + at(g, 0, i, j)), __ldg(A.theta[0] + at(g, 0, i, j - 1))),
-                 fminf(__ldg(A.theta[1] + at(g, 0, i, j)), __ldg(A.theta[1] + at(g, 0, i - 1, j))));
+      th = fminf(fminf(A.theta[0][at(g, 0, i, j)], A.theta[0][at(g, 0, i, j - 1)]),
+                 fminf(A.theta[1][at(g, 0, i, j)], A.theta[1][at(g, 0, i - 1, j)]));
   }
   bool sw = false;
   if (SHOCK && A.tsw) {
