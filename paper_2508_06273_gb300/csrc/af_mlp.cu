@@ -572,6 +572,7 @@ __global__ void colrms_kernel(const float *A, long long n, int cols, double *out
 
 int mfail(int code, const char *msg) { return set_error(code, msg); }
 int mcuda(cudaError_t e, const char *where) {
+  cudaGetLastError();  // reported here: not once more by the check after a later launch
   char m[400];
   std::snprintf(m, sizeof(m), "%s: %s", where, cudaGetErrorString(e));
   return set_error(AF_ERR_CUDA, m);
@@ -608,7 +609,7 @@ int ensure_cap(af_mlp *m, int B, int steps) {
   if (steps < m->hist_cap) steps = m->hist_cap;
   if (m->scratch) cudaFree(m->scratch);
   m->scratch = nullptr;
-  m->cap = m->hist_cap = 0;
+  m->cap = m->hist_cap = -1;  // nothing held: should the allocation fail, the next call of any size allocates
   const size_t b16 = sizeof(__nv_bfloat16), f32 = sizeof(float);
   const size_t sizes[] = {(size_t)B * NIN * b16,      3 * (size_t)B * NH * b16,      3 * (size_t)B * NH * b16,  // XT, HT, dZT
                           (size_t)B * NOUT_PAD * b16, MAX_SPLITS * (size_t)NTRAIN * f32,                       // dYT, partW
