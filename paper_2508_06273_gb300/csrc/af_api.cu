@@ -242,7 +242,10 @@ af_ctx *af_create(int nx, int ny, double dx, double dy, double gamma, uint32_t b
   const long long tiles4 = (long long)((g.nxv + 31) / 32) * ((g.nyv + 3) / 4);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-  h->tile_pv = tiles4 * 3 <= 3LL * sms ? TILE_SPLIT : TILE_PLAIN;
+  // (the rows of tiles lie on the launch grid's y axis, which ends at 65535: a
+  // grid of more than 262140 rows of nodes takes taller tiles)
+  const bool fits = (g.nyv + TILE_PLAIN - 1) / TILE_PLAIN <= 65535;
+  h->tile_pv = !fits ? TILE_TALL : (tiles4 * 3 <= 3LL * sms ? TILE_SPLIT : TILE_PLAIN);
   h->tile_tall = TILE_TALL;
   const cudaError_t te = make_maps(h);
   if (te != cudaSuccess) {

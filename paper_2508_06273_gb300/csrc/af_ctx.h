@@ -57,8 +57,8 @@ struct af_ctx {
   NodeSet tbuf[2];
   int tmap_cur;
   int tile_h;   // AF_OPT_TILE_H: point-value tile height (4, 8, 16) in rows of 32 cells
-  // the tiles that tmaps and tmaps_tall are for (TILE_PLAIN or TILE_SPLIT; TILE_TALL): tile_h
-  // once the option is set
+  // the tiles that tmaps (TILE_PLAIN, TILE_SPLIT or, on the tallest grids, TILE_TALL) and
+  // tmaps_tall (TILE_TALL) are for: tile_h once the option is set
   int tile_pv, tile_tall;
   // small device buffers
   void *small;
