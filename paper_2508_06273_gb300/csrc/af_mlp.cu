@@ -112,7 +112,8 @@ constexpr unsigned S_ACT = S_W4 + NOUT_PAD * NH * 2;  // the layer's input: X, H
 constexpr unsigned S_F32 = S_ACT + TROWS * NH * 2;    // biases, scales, bias-gradient slots, loss slots
 constexpr int NBIAS_G = 3 * NH + NOUT_PAD;            // bias gradients: b1, b2, b3, b4
 constexpr int F_BIAS = 0, F_INS = F_BIAS + NBIAS_G, F_OUTS = F_INS + NIN, F_DB = F_OUTS + NOUT,
-              F_LOSS = F_DB + 4 * NBIAS_G, F_TOTAL = F_LOSS + 4;
+              F_LOSS = F_DB + 4 * NBIAS_G, F_TOTAL = F_LOSS + 4 * 2;  // the loss slots are doubles
+static_assert(S_F32 % 8 == 0 && F_LOSS % 2 == 0, "alignment of the loss slots");
 constexpr unsigned S_BACK = (S_F32 + F_TOTAL * 4 + 127) & ~127u;  // backward only: W2^T, W3^T, W4^T, dY
 constexpr unsigned S_W2T = S_BACK, S_W3T = S_W2T + NH * NH * 2, S_W4T = S_W3T + NH * NH * 2,
                    S_DY = S_W4T + NOUT_PAD * NH * 2;
@@ -215,6 +216,7 @@ __global__ void __launch_bounds__(NET_THREADS, 1) network_kernel(NetArgs A) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int row = 32 * (warp & 3) + lane, cb = 32 * (warp >> 2);
   float *f = reinterpret_cast<float *>(nsm + S_F32);
+  double *loss = reinterpret_cast<double *>(f + F_LOSS);  // by row group, over all tiles of the CTA
   float *db = f + F_DB + (warp & 3) * NBIAS_G;  // this row group's slots; a column belongs to one warp of it
   unsigned char *act = nsm + S_ACT;
   pdl_start();
@@ -347,7 +349,7 @@ __global__ void __launch_bounds__(NET_THREADS, 1) network_kernel(NetArgs A) {
           for (int k = 0; k < NOUT; k++) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
         }
         if (lane == 0) {
-          f[F_LOSS + warp] += l;
+          loss[warp] += l;
 #pragma unroll
           for (int k = 0; k < NOUT; k++) db[3 * NH + k] += d[k];
         }
@@ -389,7 +391,7 @@ __global__ void __launch_bounds__(NET_THREADS, 1) network_kernel(NetArgs A) {
       out[k] = (d[0] + d[NBIAS_G]) + (d[2 * NBIAS_G] + d[3 * NBIAS_G]);
     }
     if (tid == 0) {
-      const double l = ((double)f[F_LOSS] + f[F_LOSS + 1]) + ((double)f[F_LOSS + 2] + f[F_LOSS + 3]);
+      const double l = (loss[0] + loss[1]) + (loss[2] + loss[3]);
       *reinterpret_cast<double *>(out + NBIAS_G) = l / (double)(NOUT * (long long)A.nvalid);
     }
   }
