@@ -406,8 +406,11 @@ __global__ void __launch_bounds__(NET_THREADS, 1) network_kernel(NetArgs A) {
 // all loads in flight and contracted by 16 MMAs: 12.8 us (cold) for B = 4096,
 // where the four products took four launches of 38 us, their results added by
 // scattered atomics.  128-row steps are no faster at 4096 and 17 % slower a
-// training step at 16384 (twice the partial products).
-constexpr int WG_THREADS = 256, WG_STEP = 256;
+// training step at 16384 (twice the partial products).  At most WG_CHAIN steps (512
+// rows) are summed in tensor memory; a split of more adds its chains in registers,
+// so that the small terms of a large batch are not lost one by one beside a large
+// partial sum.
+constexpr int WG_THREADS = 256, WG_STEP = 256, WG_CHAIN = 2;
 constexpr unsigned WG_OP = NH * WG_STEP * 2, WG_SMEM = 2 * WG_OP + 1024;
 struct WgradArgs {
   const __nv_bfloat16 *A[4], *Bm[4];  // per layer: dZ^T (or dY^T), the input's transpose
@@ -453,6 +456,9 @@ __global__ void __launch_bounds__(WG_THREADS, 1) weight_grad_kernel(WgradArgs a)
   unsigned phase = 0;
   bool ok = true;
   const int c0 = blockIdx.x * a.per, c1 = min((a.B + WG_STEP - 1) / WG_STEP, c0 + a.per);
+  // this thread's row, columns cb0 .. + 31 and cb0 + 64 .. + 95
+  const int row = 32 * (warp & 3) + lane, cb0 = 32 * (warp >> 2);
+  float acc[2][32] = {};
   for (int c = c0; c < c1 && ok; c++) {
     load_step(sA, a.A[l], M, NH, a.B, c * WG_STEP);
     load_step(sB, a.Bm[l], N, N, a.B, c * WG_STEP);
@@ -464,27 +470,38 @@ __global__ void __launch_bounds__(WG_THREADS, 1) weight_grad_kernel(WgradArgs a)
 #pragma unroll
       for (int k = 0; k < WG_STEP / 16; k++)
         tc::mma_bf16(tmem, tc::make_desc(ba + 2 * k * lboA, lboA, 128), tc::make_desc(bb + 2 * k * lboB, lboB, 128),
-                     idesc, (c > c0 || k > 0) ? 1 : 0);
+                     idesc, ((c - c0) % WG_CHAIN > 0 || k > 0) ? 1 : 0);
       tc::mma_commit(&bar);
     }
     ok = __syncthreads_and(tc::bar_wait(&bar, phase, MLP_WAIT)) != 0;
     phase ^= 1;
+    if (ok && ((c - c0) % WG_CHAIN == WG_CHAIN - 1 || c == c1 - 1)) {  // the chain ends
+      tc::fence_after_sync();
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        if (cb0 + 64 * h >= N) break;
+        float v[32];
+        tc::tmem_ld32(tmem + ((unsigned)(32 * (warp & 3)) << 16) + (unsigned)(cb0 + 64 * h), v);
+#pragma unroll
+        for (int j = 0; j < 32; j++) acc[h][j] += v[j];
+      }
+      tc::fence_before_sync();  // before the next chain's MMAs, issued after a __syncthreads
+    }
   }
   if (!ok) {
     if (tid == 0) atomicOr(a.err, 1);
     tc::bar_wait(&bar, phase ^ 1, MLP_WAIT);
   } else {
-    tc::fence_after_sync();
-    const int row = 32 * (warp & 3) + lane;
-    float *out = a.partW + (long long)blockIdx.x * NTRAIN + a.off[l] + row * N;
-    for (int cb = 32 * (warp >> 2); cb < N; cb += 64) {
-      float v[32];
-      tc::tmem_ld32(tmem + ((unsigned)(32 * (warp & 3)) << 16) + (unsigned)cb, v);
-      if (row < M)
+    float *out = a.partW + (long long)blockIdx.x * NTRAIN + a.off[l] + row * N + cb0;
+    if (row < M)
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        if (cb0 + 64 * h >= N) break;
+        const float *v = acc[h];
 #pragma unroll
         for (int q = 0; q < 8; q++)
-          reinterpret_cast<float4 *>(out + cb)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-    }
+          reinterpret_cast<float4 *>(out + 64 * h)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
   }
   tc::fence_before_sync();
   __syncthreads();
