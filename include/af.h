@@ -374,10 +374,13 @@ int af_batch_query(af_batch *b, double *t, int *steps, int *active, int *status)
  * accumulated since af_batch_set_state). */
 int af_batch_counters(af_batch *b, int64_t *out);
 /* Point-value tile height (4, 8 or 16 rows of 32 cells) of the batched
- * kernel.  af_batch_autotune times each height on the batch's current state
- * (point-value launches only; the state and time are unchanged), keeps the
- * fastest and returns it in *tile_h (and the mean milliseconds of each
- * candidate in ms[3] if given).  Needs every instance's state. */
+ * kernel, the same for every instance; until it is set, instances with the
+ * switches for discontinuous data take 8 and the others 4.  af_batch_autotune
+ * times each height on the batch's current state (point-value launches only;
+ * the state and time are unchanged) and keeps the fastest for each of these
+ * groups; *tile_h is the fastest of one height for all of them and ms[3], if
+ * given, the mean milliseconds of each height so.  Needs every instance's
+ * state.  Results do not depend on the heights. */
 int af_batch_set_tile(af_batch *b, int tile_h);
 int af_batch_autotune(af_batch *b, int *tile_h, double *ms);
 /* Training-set sampler for the surrogate: during every later batch step,

@@ -423,7 +423,8 @@ class Batch:
         _check(self.L.af_batch_set_tile(self.h, int(tile_h)))
 
     def autotune(self):
-        """Pick the fastest point-value tile height; returns (height, {height: ms})."""
+        """Pick the fastest point-value tile height of each group of instances; returns
+        (the fastest one height for all, {height: ms})."""
         th, ms = C.c_int(), np.zeros(3, dtype=np.float64)
         _check(self.L.af_batch_autotune(self.h, C.byref(th), C.c_void_p(ms.ctypes.data)))
         return th.value, dict(zip((4, 8, 16), ms.tolist()))

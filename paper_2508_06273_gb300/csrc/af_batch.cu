@@ -43,7 +43,9 @@ struct af_batch {
   cudaStream_t side = nullptr;  // the second branch of a captured step
   cudaEvent_t fork = nullptr, join = nullptr;
   std::vector<af_ctx *> inst;
-  int tile_h = 0;  // tile height of every class, or 0: each class its own (TILE_OF_CLASS)
+  // point-value tile height of each class: TILE_OF_CLASS until one is set (the same
+  // for all) or tuned (each its own)
+  int class_h[PV_CLASSES] = {TILE_OF_CLASS[0], TILE_OF_CLASS[1], TILE_OF_CLASS[2]};
   // host mirror of the control blocks: current after sync_ctl and until the next
   // run; changes to it wait (ctl_dirty) for flush_ctl
   std::vector<BatchCtl> ctl_h;
@@ -59,8 +61,8 @@ struct af_batch {
   // point-value tiles by class of their instance (the kernel instantiation its
   // options need; class of instance k in cls[k])
   std::vector<int> cls;
-  int n_pv_tiles[PV_CLASSES] = {}, heights[PV_CLASSES] = {};
-  int n_fx_tiles = 0, pv_tiles_h = 0;
+  int n_pv_tiles[PV_CLASSES] = {}, heights[PV_CLASSES] = {};  // heights: that the list was built for
+  int n_fx_tiles = 0;
   int n_fx_plain = -1;  // flux tiles of instances without the flux limiter (listed first)
   int4 *d_ghost_chunks = nullptr;  // (instance, array, first entry) per ghost-fill block
   int n_ghost_chunks = 0;
@@ -230,10 +232,11 @@ int upload_args(af_batch *b) {
 
 // TMA descriptors and the point-value tile list for the classes' tile heights
 int build_tiles(af_batch *b) {
-  if (b->maps_ok && b->pv_tiles_h == b->tile_h) return AF_OK;
+  if (b->maps_ok && std::memcmp(b->heights, b->class_h, sizeof(b->heights)) == 0) return AF_OK;
   drop_graphs(b);
+  b->maps_ok = false;  // until the end: a failure leaves them to the next call
+  std::memcpy(b->heights, b->class_h, sizeof(b->heights));
   const int *hs = b->heights;
-  for (int c = 0; c < PV_CLASSES; c++) b->heights[c] = b->tile_h ? b->tile_h : TILE_OF_CLASS[c];
   std::vector<TileMaps> maps(2 * b->n);
   std::vector<int4> pv;
   for (int k = 0; k < b->n; k++) {
@@ -260,7 +263,6 @@ int build_tiles(af_batch *b) {
   BCK(cudaMalloc(&b->d_pv_tiles, sizeof(int4) * pv.size()), "batch: cudaMalloc(tiles)");
   BCK(cudaMemcpy(b->d_pv_tiles, pv.data(), sizeof(int4) * pv.size(), cudaMemcpyHostToDevice), "batch: tiles");
   BCK(cudaMemcpy(b->d_maps, maps.data(), sizeof(TileMaps) * maps.size(), cudaMemcpyHostToDevice), "batch: maps");
-  b->pv_tiles_h = b->tile_h;
   b->maps_ok = true;
   return AF_OK;
 }
@@ -661,7 +663,7 @@ int af_batch_set_tile(af_batch *b, int tile_h) {
   if (tile_h != 4 && tile_h != 8 && tile_h != 16) return bfail(AF_ERR_ARG, "tile height must be 4, 8 or 16");
   Dev d(b->device);
   BCK(cudaStreamSynchronize(b->stream), "batch: sync");
-  b->tile_h = tile_h;
+  for (int &h : b->class_h) h = tile_h;
   return build_tiles(b);
 }
 
@@ -683,30 +685,46 @@ int af_batch_autotune(af_batch *b, int *tile_h, double *ms) {
   cudaEvent_t e0, e1;
   BCK(cudaEventCreate(&e0), "event");
   BCK(cudaEventCreate(&e1), "event");
-  double best = 1e300;
-  int best_h = b->tile_h;
+  // Each class's launch is timed by itself and takes its own fastest height (the
+  // kernels with the switches for discontinuous data and the plain ones differ in it:
+  // see TILE_PLAIN); *tile_h and ms are of one height for all classes.
+  int before[PV_CLASSES], best_h[PV_CLASSES], all_h = TILE_HEIGHTS[0];
+  std::memcpy(before, b->class_h, sizeof(before));
+  std::memcpy(best_h, before, sizeof(before));  // (a class without tiles keeps its height)
+  double best[PV_CLASSES], best_all = 1e300;
+  for (double &t : best) t = 1e300;
   for (int c = 0; c < 3 && rc == AF_OK; c++) {
-    b->tile_h = TILE_HEIGHTS[c];
+    for (int &h : b->class_h) h = TILE_HEIGHTS[c];
     rc = build_tiles(b);
     if (rc) break;
     // dt of the coming step, nothing advanced
     cudaError_t e = launch_batch_dt(b->d_ctl, b->n, nullptr, 0, DT_PROBE, b->d_pv, b->stream);
-    if (e == cudaSuccess) e = launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->heights, b->stream);
-    if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
-    for (int r = 0; r < 3 && e == cudaSuccess; r++)
-      e = launch_pointvalue_batch(pv_batch(b), b->n_pv_tiles, b->heights, b->stream);
-    if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
-    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-    float t = 0.0f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+    PointValueBatch P = pv_batch(b);
+    double all = 0.0;
+    for (int q = 0; q < PV_CLASSES && e == cudaSuccess; P.tiles += b->n_pv_tiles[q++]) {
+      int only[PV_CLASSES] = {};  // (P.tiles is at the class's first tile)
+      if ((only[q] = b->n_pv_tiles[q]) == 0) continue;
+      e = launch_pointvalue_batch(P, only, b->heights, b->stream);
+      if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
+      for (int r = 0; r < 3 && e == cudaSuccess; r++) e = launch_pointvalue_batch(P, only, b->heights, b->stream);
+      if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+      float t = 0.0f;
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+      all += t;
+      if (t < best[q]) {
+        best[q] = t;
+        best_h[q] = TILE_HEIGHTS[c];
+      }
+    }
     if (e != cudaSuccess) {
       rc = bcuda(e, "af_batch_autotune");
       break;
     }
-    if (ms) ms[c] = t / 3.0;
-    if (t < best) {
-      best = t;
-      best_h = TILE_HEIGHTS[c];
+    if (ms) ms[c] = all / 3.0;
+    if (all < best_all) {
+      best_all = all;
+      all_h = TILE_HEIGHTS[c];
     }
   }
   cudaEventDestroy(e0);
@@ -715,11 +733,11 @@ int af_batch_autotune(af_batch *b, int *tile_h, double *ms) {
   b->ctl_h = saved;
   b->ctl_current = b->ctl_dirty = true;
   for (int k = 0; k < b->n; k++) b->speed_ok[k] = 0;  // recomputed at the next run
+  std::memcpy(b->class_h, rc ? before : best_h, sizeof(before));
   if (rc) return rc;
-  b->tile_h = best_h;
   rc = build_tiles(b);
   if (rc) return rc;
-  if (tile_h) *tile_h = best_h;
+  if (tile_h) *tile_h = all_h;
   return AF_OK;
 }
 
