@@ -1285,7 +1285,6 @@ int af_set_surrogate(af_ctx *h, af_mlp *vertex_net, af_mlp *edge_net) {
     h->surr_ubar = (float *)p;
     h->surr_mask = (unsigned char *)p + ub_bytes;
     h->surr_tiles = (int *)((char *)h->surr_mask + mask_bytes);
-    h->surr_ntiles = tx * ty;
     h->surr_tiles_x = tx;
     h->surr_stats = (unsigned long long *)((char *)h->surr_tiles + tile_bytes);
     CK(prepare_surrogate(), "af_set_surrogate: kernel attributes");

@@ -114,7 +114,7 @@ struct af_ctx {
   unsigned char *surr_mask;
   float *surr_ubar;
   int *surr_tiles;
-  int surr_ntiles, surr_tiles_x;
+  int surr_tiles_x;
   unsigned long long *surr_stats;
   int sms;
 };

@@ -331,7 +331,6 @@ cudaError_t launch_pack(const Grid &g, const float *src, float *dst, int ni, int
 // checks periodic duplicate lines of an external array; sets *bad
 cudaError_t launch_check_dup(const float *ext, int ni, int nj, int dup_x, int dup_y, int *bad,
                              cudaStream_t s);
-cudaError_t launch_zero(float *p, long long n, cudaStream_t s);
 
 // tcgen05 BF16 GEMM: D[M x N] (+)= A[M x K] B[N x K]^T (+ bias); N <= 128,
 // K, lda, ldb multiples of 8; split-K over `splits` CTAs per row block

@@ -689,10 +689,6 @@ cudaError_t launch_check_dup(const float *ext, int ni, int nj, int dup_x, int du
   return cudaGetLastError();
 }
 
-cudaError_t launch_zero(float *p, long long n, cudaStream_t s) {
-  return cudaMemsetAsync(p, 0, (size_t)n * sizeof(float), s);
-}
-
 AF_BOUNDS_READER(bounds_misc)
 
 }  // namespace af
