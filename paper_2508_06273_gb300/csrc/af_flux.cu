@@ -501,8 +501,13 @@ __global__ void __launch_bounds__(NTHR, 4) flux_kernel(const __grid_constant__ A
 // Small grids take the TAIL form: it saves the ghost fill's launch and the
 // export of the wave speed (about 3 us each on an idle GPU) and costs its tiles
 // 14 % (a fence and an atomic a block, the registers of the rare image store:
-// 0.71 -> 0.83 ms at 4096^2), which meet near 3000 tiles.
-constexpr unsigned TAIL_TILES = 2432;
+// 0.71 -> 0.83 ms at 4096^2).  For a program that reads the wave speed before each
+// step the two meet near 3000 tiles (us a step, without / with: 512 tiles 71.5 / 68,
+// 2432 143.2 / 142.2, 3072 177.0 / 176.0, 4900 260.7 / 262.9); in a captured run, which
+// reads nothing between steps, they are even at 512 tiles and TAIL costs 3 % at 2432
+// (129.9 / 133.6).  The line lies a little below the first crossing: 16 tiles an SM
+// on 152 SMs.
+constexpr unsigned TAIL_TILES = 16 * 152;
 template <bool NF>
 cudaError_t launch_flux(const Args &A, const StepTail &t, cudaStream_t s) {
   const Grid &g = A.g;

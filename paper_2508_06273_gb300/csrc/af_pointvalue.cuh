@@ -1309,8 +1309,10 @@ constexpr int min_blocks() {
 }
 
 // L2 prefetch of the tile that the block PREFETCH_AHEAD places later in
-// launch order takes (about two blocks an SM ahead), so that its TMA copy
-// finds the data in L2 (measured: 12.96 -> 12.87 ms at 8192^2, same results)
+// launch order takes, so that its TMA copy finds the data in L2.  304 is a wave of
+// the 8-row kernels (two blocks an SM), for which it was chosen (with their former
+// sums 12.96 -> 12.87 ms at 8192^2).  Half a wave of the plain 4-row kernel, which it
+// costs 0.4 %: 9.13 against 9.09 ms without it and 9.13 at a whole wave, 608.
 constexpr unsigned PREFETCH_AHEAD = 304;
 template <int TY>
 __device__ __forceinline__ void tile_prefetch_l2(const TileMaps &T) {
