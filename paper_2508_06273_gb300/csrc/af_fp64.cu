@@ -131,8 +131,8 @@ __device__ void build_record(const Grid &g, double gam, const double *avg, const
 // (a, sqrt(1 - a^2), acos a) without sin or cos calls, one division and one
 // reciprocal square root serve the linearisation state.  The form before it
 // built three full 5 x 5 tables with sines and cosines of the arcs' ends and
-// contracted four cells' nine coefficients.  Now 2430 FP64 instructions a cell
-// at 89 % of the pipe; node updates at 192^2 381 -> 180 us, a whole step 468 ->
+// contracted four cells' nine coefficients.  Now 2380 FP64 instructions a cell
+// at 88 % of the pipe; node updates at 192^2 381 -> 180 us, a whole step 468 ->
 // 241 us (512^2: 3.03 -> 1.67 ms).
 __device__ __forceinline__ void taylor_d(double a0, double a1, double a2, double x0, double &t0, double &t1) {
   const double t = fma(a2, x0, a1);
